@@ -1,6 +1,6 @@
-// Shared by the attention kernels of step 5 (Eq. 3): the launch parameters, the decoding of a unit index and the
-// kernels' declarations.  A unit is (layer, kv head, question, pair of 128-row tiles); a launch covers
-// units * ncf (unit, context frame) steps, cut into contiguous ranges of `per` steps per CTA.
+// Shared by the decode-shaped attention kernel of step 5 (Eq. 3) and its merge kernels: the launch parameters and the
+// decoding of a unit index.  A unit is (layer, kv head, question); a launch covers units * ncf (unit, context frame)
+// steps, cut into contiguous ranges of `per` steps per CTA.
 #pragma once
 
 #include "ptx_helpers.cuh"
@@ -22,49 +22,28 @@ struct TcParams {
   int* status;
   QBatch qb;
   int Hq, Hkv, G, Nf, Npad, ncf, MP, layer0;
-  int Ns;           // tensor-core kernel: rows a frame takes in the token stream, N_f rounded up to a multiple of 8
-  // test-only knobs (0 = off): iteration limit of the bounded waits, and the ring entry whose copy the
-  // producer of CTA 0 leaves out so that a wait runs out with nothing in flight
+  // test-only knobs (0 = off): iteration limit of the bounded waits, and the frame whose copy CTA 0 leaves out so that a
+  // wait runs out with nothing in flight
   unsigned wait_limit;
   int skip_copy_entry;
-  long long part_slots;   // capacity of part_o / part_ml in 128-row partial slots (checks build)
   int per;          // (unit, frame) steps per CTA
-  // A unit with one row tile has no second tile to overlap with; it is run as two half-streams on the two tile
-  // slots instead -- the same rows, the frame's token chunks dealt alternately -- whose (max, sum, O) partials the
-  // merge kernel joins.  n_split = questions whose last unit is such a unit (0 = off).
-  int n_split;
   long long total;  // units * ncf
   float scale_log2;
 };
 
 struct UnitInfo {
-  int l, g, qi, m0, rows_q, tiles;
-  int split;   // one row tile, run as two half-streams
-  int srank;   // its rank among the launch's split units (partial slots when units are not cut)
+  int l, g, qi, rows_q;
   long long q_row0;
 };
 
 __device__ __forceinline__ UnitInfo decode_unit(const TcParams& p, long long u) {
   UnitInfo ui;
-  int mpg = (int)(u % p.MP);
-  long long r = u / p.MP;
+  ui.qi = (int)(u % p.MP);
+  const long long r = u / p.MP;
   ui.g = (int)(r % p.Hkv);
   ui.l = p.layer0 + (int)(r / p.Hkv);
-  int qi = 0, mp = mpg, before = 0;  // before = earlier questions whose last unit has one row tile
-  for (; qi < p.qb.nQ - 1; ++qi) {
-    const int rows = (p.qb.cu[qi + 1] - p.qb.cu[qi]) * p.G;
-    int t = (rows + 255) / 256;
-    if (mp < t) break;
-    mp -= t;
-    before += ((rows - 1) & 255) < 128;
-  }
-  ui.qi = qi;
-  ui.rows_q = (p.qb.cu[qi + 1] - p.qb.cu[qi]) * p.G;
-  ui.m0 = mp * 256;
-  ui.tiles = (ui.rows_q - ui.m0 > 128) ? 2 : 1;
-  ui.split = p.n_split > 0 && ui.tiles == 1;
-  ui.srank = ((ui.l - p.layer0) * p.Hkv + ui.g) * p.n_split + before;
-  ui.q_row0 = (long long)ui.l * p.qb.sumNq + p.qb.cu[qi];
+  ui.rows_q = (p.qb.cu[ui.qi + 1] - p.qb.cu[ui.qi]) * p.G;
+  ui.q_row0 = (long long)ui.l * p.qb.sumNq + p.qb.cu[ui.qi];
   return ui;
 }
 

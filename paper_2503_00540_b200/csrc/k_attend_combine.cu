@@ -5,51 +5,21 @@ using namespace rekv_ptx;
 
 namespace rekv_att {
 
-// The unit a block of the merge kernels works on, from blockIdx.x.  When units are not cut (per == ncf) only the units
-// with one row tile have partials (their two half-streams): the grid then counts those units only -- blockIdx.x =
-// ((layer, kv head) * n_split + rank among the batch's such questions) -- instead of every unit of a large batch, most
-// of which would have nothing to do.  Returns -1 if there is none.
-__device__ __forceinline__ long long combine_unit(const TcParams& p) {
-  if (p.per != p.ncf) return blockIdx.x;
-  const int rank = (int)(blockIdx.x % p.n_split);
-  const long long lg = blockIdx.x / p.n_split;   // (layer - layer0) * H_kv + kv head
-  int mp = 0, seen = 0;
-  for (int qi = 0; qi < p.qb.nQ; ++qi) {  // the rank-th question whose last unit has one row tile: that unit
-    const int rows = (p.qb.cu[qi + 1] - p.qb.cu[qi]) * p.G;
-    const int units_q = (rows + 255) / 256;
-    if (((rows - 1) & 255) < 128) {
-      if (seen == rank) return lg * p.MP + mp + units_q - 1;
-      ++seen;
-    }
-    mp += units_q;
-  }
-  return -1;
-}
-
 // Merge the partials of the units that were cut by a CTA boundary.
-// grid = (units, 2 row tiles, 32 groups of 4 rows); a warp per row, float4 per lane: one short
+// grid = (units, 1, 4 groups of 4 rows); a warp per row, float4 per lane: one short
 // dependent chain per warp, enough warps in flight to hide its latency.
 __global__ void __launch_bounds__(128) combine_tc5_kernel(const TcParams p) {
-  const long long u = combine_unit(p);
-  if (u < 0) return;
-  const int t = blockIdx.y;
+  const long long u = blockIdx.x;
   const long long c_first = (u * p.ncf) / p.per, c_last = ((u + 1) * p.ncf - 1) / p.per;
   const UnitInfo ui = decode_unit(p, u);
-  if (c_first == c_last && !ui.split) return;  // the unit was produced whole by one CTA
-  if (t >= ui.tiles) return;
-  // parts of this (unit, row tile): one per CTA that worked on the unit -- two per CTA, the half-streams, for a
-  // unit with one row tile -- each in its partial slot
-  const int n_parts = (int)(c_last - c_first + 1) * (ui.split ? 2 : 1);
-  auto slot_of = [&](int k) -> long long {
-    const long long c = c_first + (ui.split ? k >> 1 : k);
-    const long long base = p.per == p.ncf ? (long long)ui.srank : c + u;
-    return base * 2 + (ui.split ? (k & 1) : t);
-  };
+  if (c_first == c_last) return;  // the unit was produced whole by one CTA
+  const int n_parts = (int)(c_last - c_first + 1);  // one per CTA that worked on the unit, each in its partial slot
+  auto slot_of = [&](int k) -> long long { return (c_first + k + u) * 2; };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   grid_dep_wait();
   {
     const int r = blockIdx.z * 4 + warp;
-    const int rr = ui.m0 + t * 128 + r;
+    const int rr = r;
     if (rr >= ui.rows_q) return;
     const int n = rr / p.G, j = rr - n * p.G;
     const long long out_row = (ui.q_row0 + n) * p.Hq + ui.g * p.G + j;
@@ -97,23 +67,14 @@ __global__ void __launch_bounds__(128) combine_tc5_kernel(const TcParams p) {
 }
 
 // The same for units of many parts (a launch of few units, such as one layer, spreads each unit over dozens of CTAs).
-// grid = (units, 2 row tiles, 32 groups of 4 rows), 4 warps, float4 of the 128 columns per lane.
+// grid = (units, 1, 4 groups of 4 rows), 4 warps, float4 of the 128 columns per lane.
 __global__ void __launch_bounds__(128) combine_many_kernel(const TcParams p) {
-  const long long u = combine_unit(p);
-  if (u < 0) return;
-  const int t = blockIdx.y;
+  const long long u = blockIdx.x;
   const long long c_first = (u * p.ncf) / p.per, c_last = ((u + 1) * p.ncf - 1) / p.per;
   const UnitInfo ui = decode_unit(p, u);
-  if (c_first == c_last && !ui.split) return;  // the unit was produced whole by one CTA
-  if (t >= ui.tiles) return;
-  // parts of this (unit, row tile): one per CTA that worked on the unit -- two per CTA, the half-streams, for a
-  // unit with one row tile -- each in its partial slot
-  const int n_parts = (int)(c_last - c_first + 1) * (ui.split ? 2 : 1);
-  auto slot_of = [&](int k) -> long long {
-    const long long c = c_first + (ui.split ? k >> 1 : k);
-    const long long base = p.per == p.ncf ? (long long)ui.srank : c + u;
-    return base * 2 + (ui.split ? (k & 1) : t);
-  };
+  if (c_first == c_last) return;  // the unit was produced whole by one CTA
+  const int n_parts = (int)(c_last - c_first + 1);  // one per CTA that worked on the unit, each in its partial slot
+  auto slot_of = [&](int k) -> long long { return (c_first + k + u) * 2; };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // The block joins four rows.  Each warp takes every fourth part of all four rows -- up to six parts of four rows
   // in flight per lane, so that a unit of two dozen parts is one or two rounds of loads deep instead of six -- and
@@ -123,7 +84,7 @@ __global__ void __launch_bounds__(128) combine_many_kernel(const TcParams p) {
   __shared__ float s_m[4][4], s_den[4][4];
   grid_dep_wait();
   const int r0 = blockIdx.z * 4;
-  const int rr0 = ui.m0 + t * 128 + r0;
+  const int rr0 = r0;
   if (rr0 >= ui.rows_q) return;  // (the whole block)
   {
     float M[4], den[4];

@@ -381,3 +381,90 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) attend_decode_kernel(const TcP
 }
 
 }  // namespace rekv_att
+
+namespace {
+size_t decode_smem(int Nf) {
+  const int npad = (Nf + 15) & ~15;
+  return std::max((size_t)4 * 2 * npad * 128, (size_t)rekv_att::DEC_SCRATCH) + 64 + 1024;
+}
+}  // namespace
+
+// Decode-shaped batches (at most 16 query rows per KV head in every question) take the kernel that is built around the
+// loads; it needs two whole frames of one KV head in shared memory.
+bool rekv_decode_shaped(const rekv_ctx* c, const QBatch& qb, int ncf, int nl) {
+  for (int i = 0; i < qb.nQ; ++i)
+    if ((qb.cu[i + 1] - qb.cu[i]) * c->sv.G > 16) return false;
+  return ncf > 0 && decode_smem(c->sv.Nf) <= 227 * 1024 && (size_t)nl * c->sv.Hkv * qb.nQ <= c->part_units;
+}
+
+cudaError_t rekv_launch_attend_decode(rekv_ctx* c, const void* q, const QBatch& qb, int ncf, int layer0, int layer1,
+                                      void* out, cudaStream_t st, bool timed, const AttendFullArgs* full) {
+  using namespace rekv_att;
+  const StoreView& s = c->sv;
+  TcParams p;
+  p.tbl_k = full ? full->tbl_k : nullptr;
+  p.self_o = full ? full->self_o : nullptr;
+  p.self_ml = full ? full->self_ml : nullptr;
+  p.q = (const __nv_bfloat16*)q;
+  p.out = (__nv_bfloat16*)out;
+  p.tbl = c->ctx_tbl;
+  p.part_o = c->part_o;
+  p.part_ml = c->part_ml;
+  p.unit_cnt = c->unit_cnt;
+  p.status = c->status;
+  p.qb = qb;
+  p.Hq = s.Hq;
+  p.Hkv = s.Hkv;
+  p.G = s.G;
+  p.Nf = s.Nf;
+  p.Npad = (s.Nf + 15) & ~15;
+  p.wait_limit = c->test_wait_limit;
+  p.skip_copy_entry = c->test_skip_copy_entry;
+  p.ncf = ncf;
+  p.layer0 = layer0;
+  p.scale_log2 = 1.4426950408889634f / sqrtf(128.f);
+  p.MP = qb.nQ;  // one unit per question
+  const long long units = (long long)(layer1 - layer0) * s.Hkv * p.MP;
+  p.total = units * ncf;
+  const int n_sm = rekv_sm_count();
+  long long grid;
+  if (units >= 4 * n_sm || (size_t)(n_sm + units) * 2 > c->part_units) {
+    grid = units;  // enough units to fill the machine: one whole unit per CTA, no partials
+    p.per = ncf;
+  } else {
+    grid = p.total < n_sm ? p.total : n_sm;
+    p.per = (int)((p.total + grid - 1) / grid);
+    // a small launch (one layer): four frames per CTA amortise its fixed cost
+    if (p.per < 4) p.per = ncf < 4 ? ncf : 4;
+    grid = (p.total + p.per - 1) / p.per;
+  }
+  static PerDeviceOnce dec_attr;
+  cudaError_t e = dec_attr.run([] {
+    return cudaFuncSetAttribute(attend_decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  });
+  if (e != cudaSuccess) return e;
+  // A unit cut into a few parts is merged by the CTA that finishes its last part (no further launch); when a
+  // launch has few units and therefore many parts per unit (one layer at a time), the merge kernel's
+  // parallelism is worth its launch.
+  if ((ncf + p.per - 1) / p.per + 1 > 4) p.unit_cnt = nullptr;
+  if (timed) cudaEventRecord(c->ev_t0, st);
+  e = rekv_launch_pdl(attend_decode_kernel, dim3((unsigned)grid), dim3(DEC_THREADS), decode_smem(s.Nf), st, p);
+  if (e != cudaSuccess) return e;
+  if (timed) {
+    cudaEventRecord(c->ev_t1, st);
+    c->timing_valid = true;
+    c->merge_timed = false;
+  }
+  c->launches += 1;
+  if (p.per != ncf && !p.unit_cnt) {
+    const bool many = (ncf + p.per - 1) / p.per + 1 > 8;  // parts per unit
+    e = rekv_launch_pdl(many ? combine_many_kernel : combine_tc5_kernel, dim3((unsigned)units, 1, 4), dim3(128), 0, st, p);
+    if (e != cudaSuccess) return e;
+    c->launches += 1;
+    if (timed) {
+      cudaEventRecord(c->ev_t2, st);
+      c->merge_timed = true;
+    }
+  }
+  return cudaGetLastError();
+}

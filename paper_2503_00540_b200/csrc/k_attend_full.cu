@@ -59,23 +59,47 @@ __device__ __forceinline__ int find_question(const QBatch& qb, int n) {
   return qi;
 }
 
-// grid = (ceil(sum_Nq * H_q / 32), L), 256 threads: 8 threads per (token, head) row, one 16-byte chunk of
-// each half per thread
-__global__ void __launch_bounds__(256) rope_q_kernel(const uint4* __restrict__ q, uint4* __restrict__ q_rot, QBatch qb,
-                                                     QBatch sb, int Hq, int n_ctx_tokens,
-                                                     const float2* __restrict__ tab, int layer0) {
+// Queries rotated into q_rot, and X's K/V into the pages' layout behind the context's token stream: per (layer, KV head,
+// K/V, 64-dim half) x_rows rows of 128 bytes with the 16-byte chunks XOR-swizzled by (row & 7), question i's tokens from row
+// round8(cu_self[i]) + 8 i on; K rotated on the way.  grid = (ceil(rows / 32), layers), 256 threads: 8 threads per row, one
+// 16-byte chunk of each half per thread.  Rows: with rotary embedding the sum_Nq * H_q query rows, then (x_kv != null) the
+// sum_Ns * H_kv rows of K and as many of V.
+__global__ void __launch_bounds__(256) stage_x_kernel(const uint4* __restrict__ q, uint4* __restrict__ q_rot,
+                                                      const uint4* __restrict__ k_self, const uint4* __restrict__ v_self,
+                                                      char* __restrict__ x_kv, long long x_rows, QBatch qb, QBatch sb, int Hq,
+                                                      int Hkv, int n_ctx_tokens, const float2* __restrict__ tab, int layer0) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int l = layer0 + blockIdx.y;
-  const int row = blockIdx.x * 32 + (threadIdx.x >> 3), c = threadIdx.x & 7;
-  if (row >= qb.sumNq * Hq) return;
-  const int n = row / Hq;
-  const int qi = find_question(qb, n);
-  const int nq = qb.cu[qi + 1] - qb.cu[qi], ns = sb.cu[qi + 1] - sb.cu[qi];
-  const int pos = n_ctx_tokens + (ns - nq) + (n - qb.cu[qi]);
-  const long long base = ((long long)l * qb.sumNq * Hq + row) * 16;  // 16 chunks of 16 bytes per row
-  uint4 lo = q[base + c], hi = q[base + 8 + c];
-  rotate_chunk(lo, hi, tab + (long long)pos * 64 + c * 8);
-  q_rot[base + c] = lo;
-  q_rot[base + 8 + c] = hi;
+  const int c = threadIdx.x & 7;
+  int row = blockIdx.x * 32 + (threadIdx.x >> 3);
+  const int q_rows = tab ? qb.sumNq * Hq : 0, x_n = x_kv ? sb.sumNq * Hkv : 0;
+  if (row < q_rows) {
+    const int n = row / Hq;
+    const int qi = find_question(qb, n);
+    const int nq = qb.cu[qi + 1] - qb.cu[qi], ns = sb.cu[qi + 1] - sb.cu[qi];
+    const int pos = n_ctx_tokens + (ns - nq) + (n - qb.cu[qi]);
+    const long long base = ((long long)l * qb.sumNq * Hq + row) * 16;  // 16 chunks of 16 bytes per row
+    uint4 lo = q[base + c], hi = q[base + 8 + c];
+    rotate_chunk(lo, hi, tab + (long long)pos * 64 + c * 8);
+    q_rot[base + c] = lo;
+    q_rot[base + 8 + c] = hi;
+    return;
+  }
+  row -= q_rows;
+  const int kv = row >= x_n ? 1 : 0;
+  row -= kv * x_n;
+  if (row >= x_n) return;
+  const int tok = row / Hkv, g = row - tok * Hkv;
+  const int qi = find_question(sb, tok);
+  const int s = tok - sb.cu[qi];
+  const uint4* src = (kv ? v_self : k_self) + ((long long)l * sb.sumNq * Hkv + row) * 16;
+  uint4 lo = src[c], hi = src[8 + c];
+  if (!kv && tab) rotate_chunk(lo, hi, tab + (long long)(n_ctx_tokens + s) * 64 + c * 8);
+  const int r = ((sb.cu[qi] + 7) & ~7) + 8 * qi + s;
+  char* dst = x_kv + (((long long)(l * Hkv + g) * 2 + kv) * 2 * x_rows + r) * 128 + ((c ^ (r & 7)) << 4);
+  *reinterpret_cast<uint4*>(dst) = lo;
+  *reinterpret_cast<uint4*>(dst + x_rows * 128) = hi;
 }
 
 // Rotated copies of the context's K tiles.  grid = (ncf, nQ, L), 256 threads.  A K tile of one KV head is
@@ -292,23 +316,6 @@ __global__ void __launch_bounds__(256) self_attend_kernel(const __nv_bfloat16* _
   }
 }
 
-// No retrieved context at all (nothing visible but X): the output is the normalised self part.
-__global__ void __launch_bounds__(256) self_finalize_kernel(const float* __restrict__ self_o,
-                                                            const float* __restrict__ self_ml,
-                                                            __nv_bfloat16* __restrict__ out, long long row0,
-                                                            long long rows) {
-  const long long row = row0 + (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= row0 + rows) return;
-  const float l = self_ml[row * 2 + 1];
-  const float inv = l > 0.f ? 1.f / l : 0.f;
-  const float4 o = *reinterpret_cast<const float4*>(self_o + row * 128 + lane * 4);
-  uint2 packed;
-  packed.x = pack_bf16(o.x * inv, o.y * inv);
-  packed.y = pack_bf16(o.z * inv, o.w * inv);
-  *reinterpret_cast<uint2*>(out + row * 128 + lane * 4) = packed;
-}
-
 }  // namespace
 
 cudaError_t rekv_launch_rope_table(rekv_ctx* c, cudaStream_t st) {
@@ -318,11 +325,12 @@ cudaError_t rekv_launch_rope_table(rekv_ctx* c, cudaStream_t st) {
 }
 
 // What the attention kernel needs for Eq. 3 in full, in two halves.
-// First half, independent of the retrieval: rotated queries (with rotary embedding) and the partial over the tokens
-// of X.  Layers [layer0, layer1): q, k_self, v_self are indexed with the absolute layer (a caller that holds one
-// layer's rows passes pointers moved back by layer0 layers), as the library's own buffers are.  The part over X
-// (latency-bound) goes to the internal stream when something runs beside it on the caller's: the pass over the
-// context's keys (consecutive positions), or -- early -- the layer's retrieval kernels.
+// First half, independent of the retrieval: rotated queries (with rotary embedding), and X's K/V: staged behind the
+// context's token stream for the tensor-core kernel, or, for decode-shaped batches, as the partial over the tokens of X.
+// Layers [layer0, layer1): q, k_self, v_self are indexed with the absolute layer (a caller that holds one layer's rows
+// passes pointers moved back by layer0 layers), as the library's own buffers are.  The partial over X (latency-bound)
+// goes to the internal stream when something runs beside it on the caller's: the pass over the context's keys
+// (consecutive positions), or -- early -- the layer's retrieval kernels.
 cudaError_t rekv_launch_attend_full_self(rekv_ctx* c, const void* q, const void* k_self, const void* v_self,
                                          const QBatch& qb, const QBatch& sb, int ncf, cudaStream_t st, int layer0,
                                          int layer1, bool early) {
@@ -333,17 +341,21 @@ cudaError_t rekv_launch_attend_full_self(rekv_ctx* c, const void* q, const void*
   // at 0 -- its rotation is the identity, the stored keys are used as they are -- and token s of X at 1 + s
   const bool static_ctx = rope && (c->cfg.flags & REKV_FLAG_ROPE_STATIC) != 0;
   const int n_ctx_tokens = static_ctx ? 1 : ncf * s.Nf;   // position of X's first token
-  const __nv_bfloat16* q_eff = (const __nv_bfloat16*)q;
-  if (rope) {
-    dim3 grid((qb.sumNq * s.Hq + 31) / 32, nl);
-    rope_q_kernel<<<grid, 256, 0, st>>>((const uint4*)q, (uint4*)c->q_rot, qb, sb, s.Hq, n_ctx_tokens, c->rope_tab,
-                                        layer0);
-    c->launches += 1;
-    q_eff = c->q_rot;
-  }
-  const bool fork = (rope && !static_ctx && ncf > 0) || early;
-  cudaStream_t st_self = fork ? c->side : st;
+  const float2* tab = rope ? c->rope_tab : nullptr;
+  const bool decode = rekv_decode_shaped(c, qb, ncf, nl);
   cudaError_t e;
+  const int rows = (rope ? qb.sumNq * s.Hq : 0) + (decode ? 0 : 2 * sb.sumNq * s.Hkv);
+  if (rows > 0) {
+    e = rekv_launch_pdl(stage_x_kernel, dim3((rows + 31) / 32, nl), dim3(256), 0, st, (const uint4*)q, (uint4*)c->q_rot,
+                        (const uint4*)k_self, (const uint4*)v_self, decode ? nullptr : c->x_kv, c->x_rows, qb, sb, s.Hq,
+                        s.Hkv, n_ctx_tokens, tab, layer0);
+    if (e != cudaSuccess) return e;
+    c->launches += 1;
+  }
+  c->self_forked = false;
+  if (!decode) return cudaGetLastError();
+  const bool fork = (rope && !static_ctx) || early;
+  cudaStream_t st_self = fork ? c->side : st;
   if (fork) {
     if ((e = cudaEventRecord(c->ev_main, st)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(c->side, c->ev_main, 0)) != cudaSuccess) return e;
@@ -351,8 +363,8 @@ cudaError_t rekv_launch_attend_full_self(rekv_ctx* c, const void* q, const void*
   int max_nq = 1;
   for (int i = 0; i < qb.nQ; ++i) max_nq = std::max(max_nq, qb.cu[i + 1] - qb.cu[i]);
   self_attend_kernel<<<dim3((max_nq + 127) / 128, s.Hq, nl * qb.nQ), 256, 0, st_self>>>(
-      q_eff, (const __nv_bfloat16*)k_self, (const __nv_bfloat16*)v_self, qb, sb, s.Hq, s.Hkv, s.G, n_ctx_tokens,
-      rope ? c->rope_tab : nullptr, 1.4426950408889634f / sqrtf(128.f), c->self_o, c->self_ml, layer0);
+      rope ? c->q_rot : (const __nv_bfloat16*)q, (const __nv_bfloat16*)k_self, (const __nv_bfloat16*)v_self, qb, sb, s.Hq,
+      s.Hkv, s.G, n_ctx_tokens, tab, 1.4426950408889634f / sqrtf(128.f), c->self_o, c->self_ml, layer0);
   c->launches += 1;
   if (fork && (e = cudaEventRecord(c->ev_side, c->side)) != cudaSuccess) return e;
   c->self_forked = fork;
@@ -367,8 +379,9 @@ cudaError_t rekv_launch_attend_full_ctx(rekv_ctx* c, const QBatch& qb, int ncf, 
   const bool rope = c->cfg.rope_theta > 0.f;
   const bool static_ctx = rope && (c->cfg.flags & REKV_FLAG_ROPE_STATIC) != 0;
   if (rope && !static_ctx && ncf > 0) {
-    rope_stage_kernel<<<dim3(ncf, qb.nQ, layer1 - layer0), 256, 0, st>>>(c->ctx_tbl, c->tbl_k, c->k_rot, qb.nQ, ncf,
-                                                                        s.Hkv, s.Nf, c->rope_tab, layer0);
+    cudaError_t e = rekv_launch_pdl(rope_stage_kernel, dim3(ncf, qb.nQ, layer1 - layer0), dim3(256), 0, st, c->ctx_tbl,
+                                    c->tbl_k, c->k_rot, qb.nQ, ncf, s.Hkv, s.Nf, c->rope_tab, layer0);
+    if (e != cudaSuccess) return e;
     c->launches += 1;
   }
   if (c->self_forked) {
@@ -376,14 +389,5 @@ cudaError_t rekv_launch_attend_full_ctx(rekv_ctx* c, const QBatch& qb, int ncf, 
     cudaError_t e = cudaStreamWaitEvent(st, c->ev_side, 0);
     if (e != cudaSuccess) return e;
   }
-  return cudaGetLastError();
-}
-
-cudaError_t rekv_launch_self_finalize(rekv_ctx* c, const QBatch& qb, void* out, cudaStream_t st, int layer0,
-                                      int layer1) {
-  const long long per_layer = (long long)qb.sumNq * c->sv.Hq, rows = (layer1 - layer0) * per_layer;
-  self_finalize_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(c->self_o, c->self_ml, (__nv_bfloat16*)out,
-                                                                   layer0 * per_layer, rows);
-  c->launches += 1;
   return cudaGetLastError();
 }

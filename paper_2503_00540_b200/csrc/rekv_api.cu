@@ -69,6 +69,7 @@ void free_ctx(rekv_ctx* c) {
   cudaFree(c->ext_emb);
   cudaFree(c->self_o);
   cudaFree(c->self_ml);
+  cudaFree(c->x_kv);
   cudaFree(c->q_rot);
   cudaFree(c->rope_tab);
   cudaFree(c->k_rot);
@@ -177,6 +178,8 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
   c->self_o = c->self_ml = nullptr;
   c->ext_emb = nullptr;
   c->ext_frames = 0;
+  c->x_kv = nullptr;
+  c->x_rows = 0;
   c->q_rot = nullptr;
   c->rope_tab = nullptr;
   c->k_rot = nullptr;
@@ -244,6 +247,8 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
     const size_t rows = (size_t)s.L * c->cfg.max_q_tokens * s.Hq;
     CREATE_CUDA(cudaMalloc(&c->self_o, rows * 128 * sizeof(float)), "allocating the self-attention partials");
     CREATE_CUDA(cudaMalloc(&c->self_ml, rows * 2 * sizeof(float)), "allocating the self-attention partials");
+    c->x_rows = ((c->cfg.max_self_tokens + 7) & ~7) + 8ll * maxQ;  // every question starts on a multiple of 8 rows
+    CREATE_CUDA(cudaMalloc(&c->x_kv, (size_t)s.L * s.Hkv * 4 * c->x_rows * 128), "allocating the staged own keys and values");
     if (c->cfg.rope_theta > 0.f) {
       const bool static_ctx = (cfg->flags & REKV_FLAG_ROPE_STATIC) != 0;
       c->rope_positions = (static_ctx ? 1 : ctx_frames_max * s.Nf) + c->cfg.max_self_tokens;
@@ -687,16 +692,15 @@ int attend_full_range(rekv_ctx* c, int layer0, int layer1, const void* q, const 
   REKV_CUDA(c, rekv_launch_attend_full_ctx(c, qb, c->g_ncf, st, layer0, layer1));
   const bool rope = c->cfg.rope_theta > 0.f && !(c->cfg.flags & REKV_FLAG_ROPE_STATIC);  // rotated copies of the context's keys
   const bool rope_q = c->cfg.rope_theta > 0.f;
-  if (c->g_ncf == 0) {
-    REKV_CUDA(c, rekv_launch_self_finalize(c, qb, out, st, layer0, layer1));
-  } else {
-    AttendFullArgs fa;
-    fa.tbl_k = rope ? c->tbl_k : nullptr;
-    fa.self_o = c->self_o;
-    fa.self_ml = c->self_ml;
-    REKV_CUDA(c, rekv_launch_attend_tc5(c, rope_q ? (const void*)c->q_rot : q, qb, c->g_ncf, layer0, layer1, out, st,
-                                        (c->cfg.flags & REKV_FLAG_TIMING) != 0 && layer1 - layer0 == c->sv.L, &fa));
-  }
+  AttendFullArgs fa;
+  fa.tbl_k = rope && c->g_ncf > 0 ? c->tbl_k : nullptr;
+  fa.self_o = c->self_o;
+  fa.self_ml = c->self_ml;
+  fa.x_kv = c->x_kv;
+  fa.x_rows = c->x_rows;
+  fa.sb = &sb;
+  REKV_CUDA(c, rekv_launch_attend_tc5(c, rope_q ? (const void*)c->q_rot : q, qb, c->g_ncf, layer0, layer1, out, st,
+                                      (c->cfg.flags & REKV_FLAG_TIMING) != 0 && layer1 - layer0 == c->sv.L, &fa));
   if (c->gather_layerwise || (c->sv.tail > 0 && layer1 - layer0 < c->sv.L)) {
     // later appends (ring slots) and gathers (staging) on the side stream must not overtake this read
     REKV_CUDA(c, cudaEventRecord(c->ev_side, st));

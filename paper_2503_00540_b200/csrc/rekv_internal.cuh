@@ -127,6 +127,8 @@ struct rekv_ctx {
   // Eq. 3 in full (allocated when max_self_tokens > 0)
   float* self_o;                    // [L][max_q_tokens][H_q][128]
   float* self_ml;                   // [L][max_q_tokens][H_q][2]
+  char* x_kv;                       // [L][H_kv][K, V][half][x_rows][128 B] X's keys and values in the page layout
+  long long x_rows;
   __nv_bfloat16* q_rot;             // [L][max_q_tokens][H_q][128] rotated queries (rope_theta > 0)
   float2* rope_tab;                 // [rope_positions][64] (cos, sin)
   int rope_positions;
@@ -228,8 +230,11 @@ inline cudaError_t rekv_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 blo
 // Extra inputs of the attention kernel for Eq. 3 in full.
 struct AttendFullArgs {
   char* const* tbl_k;    // rotated K tiles per context slot (null without rotary embedding)
-  const float* self_o;   // [L][sum_Nq][H_q][128] partial numerators over the tokens of X
+  const float* self_o;   // decode-shaped batches: [L][sum_Nq][H_q][128] partial numerators over the tokens of X
   const float* self_ml;  // [L][sum_Nq][H_q][2] their (max, sum), log2 domain
+  const char* x_kv;      // the tensor-core kernel: X's K/V staged in the page layout (stage_x_kernel)
+  long long x_rows;      // its rows per (layer, kv head, K/V, half)
+  const QBatch* sb;      // X's lengths
 };
 
 // ---- kernel launchers (each returns the cudaError_t of its launches) -----------------------
@@ -251,6 +256,10 @@ cudaError_t rekv_launch_materialize(rekv_ctx* c, int nQ, int ncf, void* k_ctx, v
 // k_attend_tc5.cu
 cudaError_t rekv_launch_attend_tc5(rekv_ctx* c, const void* q, const QBatch& qb, int ncf, int layer0, int layer1,
                                    void* out, cudaStream_t st, bool timed, const AttendFullArgs* full = nullptr);
+// k_attend_decode.cu: questions of at most 16 rows per KV head
+bool rekv_decode_shaped(const rekv_ctx* c, const QBatch& qb, int ncf, int nl);
+cudaError_t rekv_launch_attend_decode(rekv_ctx* c, const void* q, const QBatch& qb, int ncf, int layer0, int layer1,
+                                      void* out, cudaStream_t st, bool timed, const AttendFullArgs* full);
 // k_attend_full.cu: the pieces of Eq. 3 in full around the attention kernel
 cudaError_t rekv_launch_rope_table(rekv_ctx* c, cudaStream_t st);
 cudaError_t rekv_launch_attend_full_self(rekv_ctx* c, const void* q, const void* k_self, const void* v_self,
@@ -258,5 +267,3 @@ cudaError_t rekv_launch_attend_full_self(rekv_ctx* c, const void* q, const void*
                                          int layer1, bool early);
 cudaError_t rekv_launch_attend_full_ctx(rekv_ctx* c, const QBatch& qb, int ncf, cudaStream_t st, int layer0,
                                         int layer1);
-cudaError_t rekv_launch_self_finalize(rekv_ctx* c, const QBatch& qb, void* out, cudaStream_t st, int layer0,
-                                      int layer1);
