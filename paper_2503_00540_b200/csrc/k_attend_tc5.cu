@@ -791,7 +791,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
           bool put = ok;
           if (ok && !safe && s_over[par] == segn + 1) {
             put = false;
-            if (boss) atomicOr(s_redo, redo_bit(si, e, pos));
+            if (boss) {
+              atomicOr(s_redo, redo_bit(si, e, pos));
+              if (CG == 2) fence_cluster();  // (the barrier at the end of the pass does not publish it)
+            }
           }
           if (safe && !(redo_mask(false) & redo_bit(si, e, pos))) put = false;  // (the pair's other CTA asked for it)
           const float x_l = s_l[par * 256 + 128 + row_e];
@@ -924,7 +927,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
         // every role and both CTAs of a pair have finished the range: is there anything to run again?
         __syncwarp();
         if constexpr (CG == 2)
-          cluster_sync_all();
+          cluster_sync_relaxed();
         else
           __syncthreads();
         if (redo_mask(true) == 0ull || *s_abort) break;
@@ -952,7 +955,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
   __syncwarp();
   tc_fence_before();
   if constexpr (CG == 2)
-    cluster_sync_all();
+    cluster_sync_relaxed();
   else
     __syncthreads();
   if (p.second) grid_dep_wait();
@@ -960,10 +963,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
 }
 
 // Joins the parts of units that were cut into more than MAX_PARTS_INSIDE (launches of few units, such as one layer).
-// grid = (units, CTAs of a pair, 32 column quads), 512 threads: a thread per (row, every fourth part), consecutive threads on
-// consecutive rows, so that a part is read in 2 KB runs and 32 parts are one round of loads deep; the four groups' results
-// meet in shared memory.  (With a thread walking all parts of a row the 19 parts of a layer were three rounds: 4.4 us.)
-constexpr int MERGE_GROUPS = 4;
+// grid = (units, CTAs of a pair, 32 column quads), 256 threads: a thread per (row, every second part), consecutive threads on
+// consecutive rows, so that a part is read in 2 KB runs and 16 parts are one round of loads deep; the two groups' results
+// meet in shared memory.  (28 layers, 28 heads, 72 frames, one layer at a time: 946 us; four groups 962; a thread walking all parts of a row,
+// three rounds for the 19 parts of a layer, about 1040.)
+constexpr int MERGE_GROUPS = 2;
 template <int CG>
 __global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __grid_constant__ Tc5Params p) {
   const int lh = (int)blockIdx.x / p.W, rank = blockIdx.y;  // blockIdx.x counts (layer, kv head) x row blocks; W = row blocks

@@ -6,62 +6,67 @@
 namespace {
 
 // ---- question vector: mean over the question's tokens and over the G query heads of each KV group
-// grid = (nQ, layers, H_kv), layer = layer0 + blockIdx.y; 1024 threads = 16 token slices x 64 dim pairs (a short
-// question is two or three rounds of loads deep): every load instruction of a warp
-// covers 128 contiguous bytes of one (token, head) row.  Writes the group's 128 dims of the question
-// vector and its partial sum of squares (the score kernel adds the H_kv partials).
-constexpr int QM_SLICES = 16;
-__global__ void __launch_bounds__(QM_SLICES * 64) qmean_kernel(const __nv_bfloat162* __restrict__ q, QBatch qb, int Hq, int Hkv,
-                                                    int G, float* __restrict__ qa, float* __restrict__ qsq,
-                                                    int maxQ, int layer0) {
+// grid = (nQ, layers, H_kv), layer = layer0 + blockIdx.y; 1024 threads = 64 row slots x 16 lanes of 16 bytes, four rows
+// per thread in flight: a question of 36 tokens at G = 7 is one round of loads deep (latency is all this kernel has).
+// Writes the group's 128 dims of the question vector and its partial sum of squares (the score kernel adds the H_kv partials).
+constexpr int QM_THREADS = 1024;
+__global__ void __launch_bounds__(QM_THREADS) qmean_kernel(const uint4* __restrict__ q, QBatch qb, int Hq, int Hkv, int G,
+                                                           float* __restrict__ qa, float* __restrict__ qsq, int maxQ,
+                                                           int layer0) {
   // launched with programmatic stream serialisation: its blocks are resident when the kernel before it ends (the
   // caller's, which wrote the queries, or the library's own), and wait here for that kernel's results
   rekv_ptx::grid_dep_wait();
   rekv_ptx::grid_dep_launch();
   const int qi = blockIdx.x, l = layer0 + blockIdx.y, g = blockIdx.z;
-  const int Dp = Hkv * 128;
-  const int n0 = qb.cu[qi], n1 = qb.cu[qi + 1];
-  const int d2 = threadIdx.x & 63, slice = threadIdx.x >> 6;
-  float sx = 0.f, sy = 0.f;
-  for (int n = n0 + slice; n < n1; n += QM_SLICES) {
-    const __nv_bfloat162* row = q + (((long long)l * qb.sumNq + n) * Hq + g * G) * 64 + d2;
-    for (int j0 = 0; j0 < G; j0 += 8) {  // up to eight independent loads in flight
-      __nv_bfloat162 v[8];
+  const int n0 = qb.cu[qi], rows = (qb.cu[qi + 1] - n0) * G;
+  const int c = threadIdx.x & 15, slot = threadIdx.x >> 4, lane = threadIdx.x & 31;
+  const uint4* base = q + (((long long)l * qb.sumNq + n0) * Hq + g * G) * 16 + c;
+  float acc[8];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (j0 + j < G) v[j] = row[(j0 + j) * 64];
+  for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+  for (int m0 = slot; m0 < rows; m0 += 256) {
+    uint4 x[4];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (j0 + j < G) {
-          float2 f = __bfloat1622float2(v[j]);
-          sx += f.x;
-          sy += f.y;
-        }
+    for (int u = 0; u < 4; ++u) {
+      const int m = m0 + 64 * u, n = m / G;
+      x[u] = m < rows ? __ldg(base + ((long long)n * Hq + (m - n * G)) * 16) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint32_t v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        acc[2 * i] += __uint_as_float(v[i] << 16);
+        acc[2 * i + 1] += __uint_as_float(v[i] & 0xFFFF0000u);
+      }
     }
   }
-  __shared__ float2 part[QM_SLICES][64];
-  __shared__ float red[2];
-  part[slice][d2] = make_float2(sx, sy);
-  __syncthreads();
-  if (threadIdx.x < 64) {
-    const float inv = (float)((n1 - n0) * G);
-    float ax = 0.f, ay = 0.f;
+  __shared__ float part[32][128];
+  __shared__ float part2[8][128];
+  __shared__ float red[4];
 #pragma unroll
-    for (int i = 0; i < QM_SLICES; i += 4) {  // fixed order
-      ax += (part[i][d2].x + part[i + 1][d2].x) + (part[i + 2][d2].x + part[i + 3][d2].x);
-      ay += (part[i][d2].y + part[i + 1][d2].y) + (part[i + 2][d2].y + part[i + 3][d2].y);
-    }
-    ax = __fdiv_rn(ax, inv);
-    ay = __fdiv_rn(ay, inv);
-    float* dst = qa + ((long long)l * maxQ + qi) * Dp + g * 128;
-    dst[2 * d2] = ax;
-    dst[2 * d2 + 1] = ay;
-    float sq = ax * ax + ay * ay;
+  for (int i = 0; i < 8; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+  if (lane < 16) {
+    float4* dst = reinterpret_cast<float4*>(&part[threadIdx.x >> 5][c * 8]);
+    dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+  }
+  __syncthreads();
+  const int d = threadIdx.x & 127, k = threadIdx.x >> 7;  // fixed order
+  part2[k][d] = (part[4 * k][d] + part[4 * k + 1][d]) + (part[4 * k + 2][d] + part[4 * k + 3][d]);
+  __syncthreads();
+  if (threadIdx.x < 128) {
+    float a = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) a += part2[i][d];
+    a = __fdiv_rn(a, (float)rows);
+    qa[((long long)l * maxQ + qi) * (Hkv * 128) + g * 128 + d] = a;
+    float sq = a * a;
     for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sq;
+    if (lane == 0) red[threadIdx.x >> 5] = sq;
   }
   __syncthreads();
-  if (threadIdx.x == 0) qsq[((long long)l * maxQ + qi) * Hkv + g] = red[0] + red[1];
+  if (threadIdx.x == 0) qsq[((long long)l * maxQ + qi) * Hkv + g] = (red[0] + red[1]) + (red[2] + red[3]);
 }
 
 // ---- cosine scores.  grid = (item chunks, L); an item is a frame, or with block retrieval a block of
@@ -72,7 +77,7 @@ __global__ void __launch_bounds__(QM_SLICES * 64) qmean_kernel(const __nv_bfloat
 // SCORE_MAX_V4 = float4 per lane (4: D' <= 512, 8: D' <= 1024); fpc = frames per CTA (a multiple of 16), chosen by
 // the launcher so that the whole grid is resident at once (no second, mostly empty wave).
 template <int SCORE_MAX_V4>
-__global__ void __launch_bounds__(256, SCORE_MAX_V4 <= 4 ? 4 : 2)
+__global__ void __launch_bounds__(256, SCORE_MAX_V4 <= 4 ? 3 : 2)
     score_kernel(const float* __restrict__ reps, const float* __restrict__ qa, const float* __restrict__ qsq, int nQ,
                  int maxQ, int Dp, int Hkv, int max_frames, int n_visible, int q_group, float* __restrict__ scores,
                  int block, int layer0, int fpc, int* __restrict__ status) {
@@ -178,10 +183,14 @@ __device__ __forceinline__ unsigned score_key(float s) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// grid = (nQ, L), 512 threads.  Candidates are frames [0, n_cand).  Four 8-bit radix passes over the
-// score keys find the k-th largest key T exactly, with the number of candidates above it; one
-// ordered compaction then emits, in ascending frame index, every frame above T and the lowest-index
-// frames equal to T that are still needed (ties go to the lower index).
+// grid = (nQ, L), 512 threads.  Candidates are frames [0, n_cand).  Up to 2048 of them keep their keys in registers, and one
+// histogram over 2048 equal steps between the smallest and the largest score finds the step that holds the k-th largest:
+// every candidate in a higher step is selected, and the few in that step are ranked exactly against each other (score, then
+// lower index).  Otherwise -- more candidates, a NaN among them, a step with more than TK_LIST members -- four 8-bit radix
+// passes over the score keys find the k-th largest key T exactly, with the number of candidates above it; one ordered
+// compaction then emits, in ascending frame index, every frame above T and the lowest-index frames equal to T that are
+// still needed (ties go to the lower index).  Latency is all: the radix passes took 4.3 us per launch of 1792 candidates
+// (their first pass puts all cosines into a few bins, whose atomics queue).
 // With block retrieval the candidates are blocks; a selected block b_i is written as its `block` frames
 // b_i*block .. b_i*block + block-1 (k_eff counts items, top_k counts output slots).
 // With tbl != null (cache all in HBM) the block also writes the context table of its (layer, question) -- the
@@ -193,24 +202,14 @@ struct TopkTable {
   long long page_bytes;
   int L, ncf, n_vis_frames;
 };
-__device__ __forceinline__ void topk_write_table(const TopkTable& t, const int32_t* out, int k_frames, int l, int qi,
-                                                 int nQ) {
-  if (!t.tbl) return;
-  __syncthreads();  // the block's writes of the selection are visible to all its threads
-  char** row = t.tbl + ((long long)l * nQ + qi) * t.ncf;
-  for (int j = threadIdx.x; j < t.ncf; j += blockDim.x) {
-    const int frame = j < k_frames ? out[j] : t.n_vis_frames - (t.ncf - k_frames) + (j - k_frames);
-    row[j] = t.hbm + ((long long)frame * t.L + l) * t.page_bytes;
-  }
-}
-
+constexpr int TK_BINS = 2048, TK_LIST = 64;
 __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ scores, int nQ, int n_visible,
                                                    int n_cand, int top_k, int k_eff, int32_t* __restrict__ idx_out,
-                                                   int block, int layer0, TopkTable tt, int* __restrict__ status) {
+                                                   int block, int layer0, TopkTable tt, int copies, int* __restrict__ status) {
   const int qi = blockIdx.x, l = layer0 + blockIdx.y;
   const float* s = scores + ((long long)l * nQ + qi) * n_visible;
   int32_t* out = idx_out + ((long long)l * nQ + qi) * top_k;
-  __shared__ unsigned hist[4 * 256];
+  __shared__ __align__(16) unsigned hist[TK_BINS];  // (the radix passes use its front)
   __shared__ unsigned s_prefix;
   __shared__ int s_krem;
   __shared__ int warp_gt[16], warp_eq[16];
@@ -219,11 +218,19 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
   rekv_ptx::grid_dep_wait();
   rekv_ptx::grid_dep_launch();
 
-  for (int j = k_eff * block + threadIdx.x; j < top_k; j += blockDim.x) out[j] = -1;
-  if (k_eff <= 0) {
-    topk_write_table(tt, out, 0, l, qi, nQ);
-    return;
-  }
+  // entry `at` of the selection, and with it the page of that context slot; `copies` layers get the same selection
+  char** row = tt.tbl ? tt.tbl + ((long long)l * nQ + qi) * tt.ncf : nullptr;
+  auto page_of = [&](int frame) { return tt.hbm + ((long long)frame * tt.L + l) * tt.page_bytes; };
+  auto emit_item = [&](int at, int frame) {
+    for (int r = 0; r < copies; ++r) out[(long long)r * nQ * top_k + at] = frame;
+    if (row) row[at] = page_of(frame);
+  };
+  const int k_frames = k_eff > 0 ? k_eff * block : 0;
+  for (int j = k_frames + threadIdx.x; j < top_k; j += blockDim.x)
+    for (int r = 0; r < copies; ++r) out[(long long)r * nQ * top_k + j] = -1;
+  if (row)  // the trailing frames
+    for (int j = k_frames + threadIdx.x; j < tt.ncf; j += blockDim.x) row[j] = page_of(tt.n_vis_frames - tt.ncf + j);
+  if (k_eff <= 0) return;
   // up to TK_CACHE * 512 candidates keep their keys in registers: one read of the scores instead of five.  A thread
   // holds TK_CACHE consecutive candidates, so that the ordered compaction at the end is one scan over the threads.
   constexpr int TK_CACHE = 4;
@@ -240,7 +247,113 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
     s_base_gt = 0;
     s_base_eq = 0;
   }
-  for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) hist[i] = 0;  // one histogram per pass, cleared once
+  *reinterpret_cast<uint4*>(hist + 4 * threadIdx.x) = make_uint4(0, 0, 0, 0);
+  if (cached) {
+    __shared__ unsigned w_lo[16], w_hi[16], w_cnt[16];
+    __shared__ unsigned l_key[TK_LIST];
+    __shared__ int l_idx[TK_LIST];
+    __shared__ int s_bin, s_need, s_members, s_n;
+    unsigned k_lo = 0xFFFFFFFFu, k_hi = 0u;
+#pragma unroll
+    for (int j = 0; j < TK_CACHE; ++j)
+      if ((int)threadIdx.x * TK_CACHE + j < n_cand) {
+        k_lo = min(k_lo, kc[j]);
+        k_hi = max(k_hi, kc[j]);
+      }
+    k_lo = __reduce_min_sync(0xffffffffu, k_lo);
+    k_hi = __reduce_max_sync(0xffffffffu, k_hi);
+    if (lane == 0) {
+      w_lo[warp] = k_lo;
+      w_hi[warp] = k_hi;
+    }
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    k_lo = __reduce_min_sync(0xffffffffu, w_lo[lane & 15]);
+    k_hi = __reduce_max_sync(0xffffffffu, w_hi[lane & 15]);
+    auto value = [](unsigned k) { return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k); };
+    const float lo = value(k_lo), width = value(k_hi) - lo;
+    // (an infinite or NaN score, equal scores, or a width that overflows: the radix passes)
+    if (width > 0.f && width < 3.0e38f) {
+      const float scale = (float)TK_BINS / width;
+      int bin[TK_CACHE];
+#pragma unroll
+      for (int j = 0; j < TK_CACHE; ++j) {  // monotone in the score
+        bin[j] = -1;
+        if ((int)threadIdx.x * TK_CACHE + j < n_cand) {
+          bin[j] = min((int)((value(kc[j]) - lo) * scale), TK_BINS - 1);
+          atomicAdd(&hist[bin[j]], 1u);
+        }
+      }
+      __syncthreads();
+      // thread t holds bins [4t, 4t + 4); inclusive suffix sums over the block
+      const uint4 h = *reinterpret_cast<const uint4*>(hist + 4 * threadIdx.x);
+      const int tot = (int)(h.x + h.y + h.z + h.w);
+      int suf = tot;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_down_sync(0xffffffffu, suf, o);
+        if (lane + o < 32) suf += v;
+      }
+      if (lane == 0) w_cnt[warp] = suf;
+      __syncthreads();
+      suf += __reduce_add_sync(0xffffffffu, lane < 16 && lane > warp ? (int)w_cnt[lane & 15] : 0);
+      if (suf >= k_eff && suf - tot < k_eff) {  // the k-th largest lies in this thread's bins
+        int above = suf - tot, d = 3;
+        const int b[4] = {(int)h.x, (int)h.y, (int)h.z, (int)h.w};
+        for (; d > 0 && above + b[d] < k_eff; --d) above += b[d];
+        s_bin = 4 * threadIdx.x + d;
+        s_need = k_eff - above;
+        s_members = b[d];
+      }
+      __syncthreads();
+      const int at = s_bin, need = s_need, members = s_members;
+      if (members <= TK_LIST) {  // (uniform)
+        bool sel[TK_CACHE];
+#pragma unroll
+        for (int j = 0; j < TK_CACHE; ++j) {
+          sel[j] = bin[j] > at || (bin[j] == at && need == members);
+          if (need != members && bin[j] == at) {
+            const int n = atomicAdd(&s_n, 1);
+            l_key[n] = kc[j];
+            l_idx[n] = threadIdx.x * TK_CACHE + j;
+          }
+        }
+        if (need != members) {
+          __syncthreads();
+#pragma unroll
+          for (int j = 0; j < TK_CACHE; ++j)
+            if (bin[j] == at) {
+              const int i = threadIdx.x * TK_CACHE + j;
+              int before = 0;
+              for (int n = 0; n < members; ++n) before += l_key[n] > kc[j] || (l_key[n] == kc[j] && l_idx[n] < i);
+              sel[j] = before < need;
+            }
+        }
+        // ordered compaction: an exclusive scan over the threads
+        int cnt = 0;
+#pragma unroll
+        for (int j = 0; j < TK_CACHE; ++j) cnt += sel[j];
+        int sc = cnt;
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, sc, o);
+          if (lane >= o) sc += v;
+        }
+        if (lane == 31) warp_gt[warp] = sc;
+        __syncthreads();
+        int pos = sc - cnt + __reduce_add_sync(0xffffffffu, lane < warp ? warp_gt[lane & 15] : 0);
+#pragma unroll
+        for (int j = 0; j < TK_CACHE; ++j)
+          if (sel[j]) {
+            const int i = threadIdx.x * TK_CACHE + j;
+            if (REKV_CHECK(pos < k_eff && i < n_cand, status, 21))
+              for (int jj = 0; jj < block; ++jj) emit_item(pos * block + jj, i * block + jj);
+            ++pos;
+          }
+        return;
+      }
+      __syncthreads();
+      *reinterpret_cast<uint4*>(hist + 4 * threadIdx.x) = make_uint4(0, 0, 0, 0);
+    }
+  }
   __syncthreads();
   for (int pass = 0; pass < 4; ++pass) {
     const int shift = 24 - 8 * pass;
@@ -334,7 +447,7 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
       if (gt) pos = og + min(oe, need_eq);
       if (eq && oe < need_eq) pos = og + oe;
       if (pos >= 0 && REKV_CHECK(pos < k_eff && i < n_cand, status, 21))
-        for (int jj = 0; jj < block; ++jj) out[pos * block + jj] = i * block + jj;
+        for (int jj = 0; jj < block; ++jj) emit_item(pos * block + jj, i * block + jj);
       og += gt;
       oe += eq;
     }
@@ -363,7 +476,6 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
       __syncthreads();
     }
   }
-  topk_write_table(tt, out, k_eff * block, l, qi, nQ);
 }
 
 // ---- external retrieval (Eq. 2 with its temperature): cosine of each question embedding with every frame
@@ -376,6 +488,8 @@ __global__ void __launch_bounds__(256) ext_score_kernel(const float* __restrict_
                                                         float* __restrict__ scores) {
   extern __shared__ float4 s_qe[];  // [q_group][E/4]
   __shared__ float s_qn[REKV_MAX_QUESTIONS];
+  rekv_ptx::grid_dep_wait();
+  rekv_ptx::grid_dep_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int item = blockIdx.x * 8 + warp;
   const int e4 = E / 4;
@@ -434,48 +548,54 @@ __global__ void __launch_bounds__(256) ext_score_kernel(const float* __restrict_
   }
 }
 
-// the external selection is the same in every layer: copies layer 0's [nQ][top_k] block to the others
-__global__ void replicate_idx_kernel(int32_t* __restrict__ idx, int per_layer, int L) {
-  rekv_ptx::grid_dep_wait();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= per_layer) return;
-  const int32_t v = idx[i];
-  for (int l = 1; l < L; ++l) idx[(long long)l * per_layer + i] = v;
-}
 
 // Launch of the score kernel over frames [0, n_scored) of nl layers.  Frames per CTA grow until the grid fits the
 // device in one wave at the kernel's occupancy.
+// What the score kernel needs besides the grid.
+struct ScoreArgs {
+  int nl, n_scored;
+  const float* reps;
+  const float* qa;
+  const float* qsq;
+  int nQ, maxQ, Dp, Hkv, max_frames;
+  float* scores;
+  int block, layer0;
+  int* status;
+};
 template <int V4>
-cudaError_t launch_score_v4(bool pdl, cudaStream_t st, size_t smem, int nl, int n_scored, const float* reps, const float* qa,
-                            const float* qsq, int nQ, int maxQ, int Dp, int Hkv, int max_frames, int q_group, float* scores,
-                            int block, int layer0, int* status) {
+cudaError_t launch_score_v4(const ScoreArgs& a, bool pdl, cudaStream_t st) {
+  int q_group = (int)((96 * 1024) / (a.Dp * sizeof(float)));
+  if (q_group > a.nQ) q_group = a.nQ;
+  const size_t smem = (size_t)q_group * a.Dp * sizeof(float);
   static PerDeviceOnce attr;
-  cudaError_t ea = attr.run([] {
+  cudaError_t e = attr.run([] {
     return cudaFuncSetAttribute(score_kernel<V4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
   });
-  if (ea != cudaSuccess) return ea;
-  const int sms = rekv_sm_count();
-  int occ = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, score_kernel<V4>, 256, smem) != cudaSuccess || occ < 1) occ = 1;
-  int per_layer = (sms * occ) / nl;
+  if (e != cudaSuccess) return e;
+  // blocks per SM by the dynamic shared memory in KB (asking the runtime on every call costs as much as a launch)
+  static int known[REKV_MAX_DEVICES][97] = {};
+  int dev = 0, occ = 0;
+  const int kb = (int)((smem + 1023) / 1024);
+  const bool cacheable = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < REKV_MAX_DEVICES && kb <= 96;
+  if (cacheable) occ = known[dev][kb];
+  if (occ < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, score_kernel<V4>, 256, smem) != cudaSuccess || occ < 1) occ = 1;
+    if (cacheable) known[dev][kb] = occ;
+  }
+  int per_layer = (rekv_sm_count() * occ) / a.nl;
   if (per_layer < 1) per_layer = 1;
-  int fpc = ((n_scored + per_layer - 1) / per_layer + 15) & ~15;
+  int fpc = ((a.n_scored + per_layer - 1) / per_layer + 15) & ~15;
   if (fpc < 16) fpc = 16;
-  dim3 grid((n_scored + fpc - 1) / fpc, nl);
+  const dim3 grid((a.n_scored + fpc - 1) / fpc, a.nl);
   if (pdl)
-    return rekv_launch_pdl(score_kernel<V4>, grid, dim3(256), smem, st, reps, qa, qsq, nQ, maxQ, Dp, Hkv, max_frames,
-                           n_scored, q_group, scores, block, layer0, fpc, status);
-  score_kernel<V4><<<grid, 256, smem, st>>>(reps, qa, qsq, nQ, maxQ, Dp, Hkv, max_frames, n_scored, q_group, scores, block,
-                                            layer0, fpc, status);
+    return rekv_launch_pdl(score_kernel<V4>, grid, dim3(256), smem, st, a.reps, a.qa, a.qsq, a.nQ, a.maxQ, a.Dp, a.Hkv,
+                           a.max_frames, a.n_scored, q_group, a.scores, a.block, a.layer0, fpc, a.status);
+  score_kernel<V4><<<grid, 256, smem, st>>>(a.reps, a.qa, a.qsq, a.nQ, a.maxQ, a.Dp, a.Hkv, a.max_frames, a.n_scored, q_group,
+                                            a.scores, a.block, a.layer0, fpc, a.status);
   return cudaGetLastError();
 }
-cudaError_t launch_score(bool pdl, cudaStream_t st, size_t smem, int nl, int n_scored, const float* reps, const float* qa,
-                         const float* qsq, int nQ, int maxQ, int Dp, int Hkv, int max_frames, int q_group, float* scores,
-                         int block, int layer0, int* status) {
-  return Dp <= 512 ? launch_score_v4<4>(pdl, st, smem, nl, n_scored, reps, qa, qsq, nQ, maxQ, Dp, Hkv, max_frames, q_group,
-                                        scores, block, layer0, status)
-                   : launch_score_v4<8>(pdl, st, smem, nl, n_scored, reps, qa, qsq, nQ, maxQ, Dp, Hkv, max_frames, q_group,
-                                        scores, block, layer0, status);
+cudaError_t launch_score(const ScoreArgs& a, bool pdl, cudaStream_t st) {
+  return a.Dp <= 512 ? launch_score_v4<4>(a, pdl, st) : launch_score_v4<8>(a, pdl, st);
 }
 
 }  // namespace
@@ -488,22 +608,19 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
   const StoreView& s = c->sv;
   const int maxQ = c->cfg.max_questions;
   const int nl = layer1 - layer0;
-  {
-    cudaError_t e0 = rekv_launch_pdl(qmean_kernel, dim3(qb.nQ, nl, s.Hkv), dim3(QM_SLICES * 64), 0, st,
-                                     (const __nv_bfloat162*)q, qb, s.Hq, s.Hkv, s.G, c->qa, c->qnorm, maxQ, layer0);
-    if (e0 != cudaSuccess) return e0;
-  }
-  int q_group = (int)((96 * 1024) / (s.Dp * sizeof(float)));
-  if (q_group > qb.nQ) q_group = qb.nQ;
-  size_t smem = (size_t)q_group * s.Dp * sizeof(float);
   // b = 1: every visible frame is scored (the window's scores are reported but not candidates);
   // b > 1: the complete candidate blocks are scored
   const int b = c->cfg.block_frames;
   const int n_scored = b == 1 ? n_visible : geom.n_items;
   if (n_scored > 0) {
-    cudaError_t e1 = launch_score(true, st, smem, nl, n_scored, s.reps, c->qa, c->qnorm, qb.nQ, maxQ, s.Dp, s.Hkv,
-                                  s.max_frames, q_group, scores, b, layer0, c->status);
-    if (e1 != cudaSuccess) return e1;
+    ScoreArgs a = {nl, n_scored, s.reps, c->qa, c->qnorm, qb.nQ, maxQ, s.Dp, s.Hkv, s.max_frames, scores, b, layer0, c->status};
+    cudaError_t e;
+    e = rekv_launch_pdl(qmean_kernel, dim3(qb.nQ, nl, s.Hkv), dim3(QM_THREADS), 0, st, (const uint4*)q, qb, s.Hq,
+                        s.Hkv, s.G, c->qa, c->qnorm, maxQ, layer0);
+    if (e != cudaSuccess) return e;
+    c->launches += 1;
+    e = launch_score(a, true, st);
+    if (e != cudaSuccess) return e;
     c->launches += 1;
   }
   if (top_k > 0) {
@@ -517,11 +634,10 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
       tt.n_vis_frames = n_visible;
     }
     cudaError_t e2 = rekv_launch_pdl(topk_kernel, dim3(qb.nQ, nl), dim3(512), 0, st, scores, qb.nQ, n_scored,
-                                     geom.n_items, top_k, geom.k_items, idx_out, b, layer0, tt, c->status);
+                                     geom.n_items, top_k, geom.k_items, idx_out, b, layer0, tt, 1, c->status);
     if (e2 != cudaSuccess) return e2;
     c->launches += 1;
   }
-  c->launches += 1;
   return cudaGetLastError();
 }
 
@@ -538,21 +654,16 @@ cudaError_t rekv_launch_retrieve_external(rekv_ctx* c, const float* q_emb, int n
   });
   if (ea != cudaSuccess) return ea;
   if (n_scored > 0) {
-    ext_score_kernel<<<(n_scored + 7) / 8, 256, (size_t)q_group * E * sizeof(float), st>>>(c->ext_emb, q_emb, nQ, E, n_scored,
-                                                                                         b, q_group, tau, scores);
+    cudaError_t e1 = rekv_launch_pdl(ext_score_kernel, dim3((n_scored + 7) / 8), dim3(256), (size_t)q_group * E * sizeof(float),
+                                     st, (const float*)c->ext_emb, q_emb, nQ, E, n_scored, b, q_group, tau, scores);
+    if (e1 != cudaSuccess) return e1;
     c->launches += 1;
   }
   if (top_k > 0) {
     cudaError_t e2 = rekv_launch_pdl(topk_kernel, dim3(nQ, 1), dim3(512), 0, st, (const float*)scores, nQ, n_scored,
-                                     geom.n_items, top_k, geom.k_items, idx_out, b, 0, TopkTable{}, c->status);
+                                     geom.n_items, top_k, geom.k_items, idx_out, b, 0, TopkTable{}, s.L, c->status);
     if (e2 != cudaSuccess) return e2;
-    const int per_layer = nQ * top_k;
-    if (s.L > 1) {
-      cudaError_t e3 = rekv_launch_pdl(replicate_idx_kernel, dim3((per_layer + 255) / 256), dim3(256), 0, st, idx_out,
-                                       per_layer, s.L);
-      if (e3 != cudaSuccess) return e3;
-    }
-    c->launches += 2;
+    c->launches += 1;
   }
   return cudaGetLastError();
 }
@@ -644,13 +755,10 @@ extern "C" int rekv_score_frames_static(const void* q, const int32_t* cu_q, int 
 
   const int Dp = n_kv_heads * REKV_HEAD_DIM, G = n_q_heads / n_kv_heads;
   cudaStream_t st = (cudaStream_t)stream;
-  qmean_kernel<<<dim3(nQ, 1, n_kv_heads), QM_SLICES * 64, 0, st>>>((const __nv_bfloat162*)q, qb, n_q_heads, n_kv_heads, G, qa, qsq,
+  qmean_kernel<<<dim3(nQ, 1, n_kv_heads), QM_THREADS, 0, st>>>((const uint4*)q, qb, n_q_heads, n_kv_heads, G, qa, qsq,
                                                          STATIC_MAX_QUESTIONS, 0);
-  // the question vectors of one call fit in 64 KB of dynamic shared memory only in groups
-  int q_group = (int)((96 * 1024) / (Dp * sizeof(float)));
-  if (q_group > nQ) q_group = nQ;
-  e = launch_score(false, st, (size_t)q_group * Dp * sizeof(float), 1, n_frames, reps, qa, qsq, nQ, STATIC_MAX_QUESTIONS, Dp,
-                   n_kv_heads, n_frames, q_group, scores_out, 1, 0, nullptr);
+  const ScoreArgs a = {1, n_frames, reps, qa, qsq, nQ, STATIC_MAX_QUESTIONS, Dp, n_kv_heads, n_frames, scores_out, 1, 0, nullptr};
+  e = launch_score(a, false, st);
   if (e != cudaSuccess) {
     rekv_set_error(nullptr, cudaGetErrorString(e));
     return REKV_ERR_CUDA;

@@ -1,0 +1,66 @@
+"""Step 3 at the sizes and score patterns where the selection kernel changes its way: up to 2048 candidates one histogram
+over equal score steps and an exact ranking inside the step that holds the k-th largest; radix passes beyond that, when the
+step has more than 64 members, and when a score is not finite.  The scores come back from the same call, so the selection has
+to match exactly what sorting them gives (score, then lower index; NaN last; ascending output)."""
+import pytest
+import torch
+
+from paper_2503_00540_b200 import rekv
+
+pytestmark = pytest.mark.gpu
+
+
+def _select(embs: torch.Tensor, k: int, W: int = 0, b: int = 1):
+    T = embs.shape[0]
+    g = rekv.ReKV(3, 4, 1, 128, 1, T, W, max_topk=k, block_frames=b, ext_embed_dim=embs.shape[1])
+    kv = torch.zeros((3, 1, 1, 128), dtype=torch.bfloat16, device="cuda")
+    for f in range(T):
+        g.append_frame(kv, kv)
+        g.set_frame_embedding(f, embs[f])
+    q = torch.zeros((1, embs.shape[1]), device="cuda")
+    q[0, 0] = 1.0
+    idx, k_eff, scores = g.retrieve_external(q, k, T, 1.0, want_scores=True)
+    n_scored = scores.shape[1]
+    g.check_status()
+    g.close()
+    n_cand = max(T - W, 0) if b == 1 else n_scored
+    s = scores[0, :n_cand].cpu()
+    s = torch.where(torch.isnan(s), torch.full_like(s, float("-inf")), s)
+    items = sorted(range(n_cand), key=lambda i: (-s[i].item(), i))[:k_eff // b]
+    want = [i * b + j for i in sorted(items) for j in range(b)]
+    for l in range(3):
+        assert idx[l, 0, :k_eff].tolist() == want, f"layer {l}"
+        assert (idx[l, 0, k_eff:] == -1).all()
+
+
+def _angles(n, seed):
+    gen = torch.Generator().manual_seed(seed)
+    a = torch.rand(n, generator=gen) * 3.0
+    return torch.stack([a.cos(), a.sin(), 0 * a, 0 * a], 1).cuda().contiguous()
+
+
+@pytest.mark.parametrize("T,k,W", [(1, 1, 0), (2, 1, 1), (65, 64, 0), (513, 8, 0), (2047, 64, 3), (2048, 64, 0),
+                                   (2049, 64, 0), (2600, 200, 8), (1800, 1800, 8)])
+def test_selection_at_the_edges_of_the_histogram_path(T, k, W):
+    _select(_angles(T, T), k, W)
+
+
+@pytest.mark.parametrize("pattern", ["all_equal", "pairs", "one_step", "nan", "zero_norm"])
+def test_selection_with_ties_crowded_steps_and_scores_that_are_not_numbers(pattern):
+    e = _angles(1500, 5)
+    if pattern == "all_equal":
+        e[:] = e[0]
+    elif pattern == "pairs":      # every score twice, 40 of them thirty times
+        e[1::2] = e[0::2]
+        e[300:330] = e[700]
+    elif pattern == "one_step":   # one far score; all others inside a single step
+        a = 1.0 + 1e-6 * torch.arange(1500)
+        e = torch.stack([a.cos(), a.sin(), 0 * a, 0 * a], 1).cuda().contiguous()
+        e[77] = torch.tensor([-1.0, 0, 0, 0])
+    elif pattern == "nan":
+        e[3] = float("nan")
+        e[900] = float("nan")
+    else:
+        e[10:50] = 0.0
+    _select(e, 64)
+    _select(e[:1496].contiguous(), 64, b=8)
