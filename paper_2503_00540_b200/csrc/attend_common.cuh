@@ -1,6 +1,6 @@
-// Shared by the decode-shaped attention kernel of step 5 (Eq. 3) and its merge kernels: the launch parameters and the
-// decoding of a unit index.  A unit is (layer, kv head, question); a launch covers units * ncf (unit, context frame)
-// steps, cut into contiguous ranges of `per` steps per CTA.
+// The decode-shaped attention kernel of step 5 (Eq. 3): the launch parameters and the decoding of a unit index.  A unit is
+// (layer, kv head, question); a launch covers units * steps steps -- a step is a context frame, or a tile of X's tokens --
+// cut into contiguous ranges of `per` steps per CTA.
 #pragma once
 
 #include "ptx_helpers.cuh"
@@ -12,22 +12,30 @@ struct TcParams {
   const __nv_bfloat16* q;
   __nv_bfloat16* out;
   char* const* tbl;
-  // Eq. 3 in full (FULL instantiation and the merge kernel only; null otherwise)
-  char* const* tbl_k;      // per context slot: rotated copy of the page's K tiles, or null = K from the page
-  const float* self_o;     // per output row: sum of p*v over the tokens of X the row sees, relative to self_ml[0]
-  const float* self_ml;    // per output row: (max, sum) of that part, log2 domain
+  // Eq. 3 in full: the own K/V of X, [L][sum_Ns][H_kv][128] as the caller passes them, and their lengths (nQ = 0: none)
+  const __nv_bfloat16* k_self;
+  const __nv_bfloat16* v_self;
+  QBatch sb;
+  // rotary embedding: (cos, sin) per [position][64], or null; context token j is at position j when rot_ctx is set (else it
+  // is not rotated), token s of X at pos_x + s
+  const float2* tab;
+  int n_pos, pos_x, rot_ctx;
   float* part_o;
   float* part_ml;
-  int* unit_cnt;     // per unit: parts finished so far (decode kernel: the last part merges; self-resetting)
+  int* unit_cnt;     // per unit: parts finished so far (the last part merges; self-resetting)
   int* status;
   QBatch qb;
   int Hq, Hkv, G, Nf, Npad, ncf, MP, layer0;
+  int early;         // the context table and its pages are complete whatever the kernels just before this launch do
+  int steps;         // steps of a unit: its context frames, then tiles of N_pad tokens of X
   // test-only knobs (0 = off): iteration limit of the bounded waits, and the frame whose copy CTA 0 leaves out so that a
   // wait runs out with nothing in flight
   unsigned wait_limit;
   int skip_copy_entry;
-  int per;          // (unit, frame) steps per CTA
-  long long total;  // units * ncf
+  int part_slots;    // capacity of part_o / part_ml in 16-row parts
+  int per;           // steps per CTA, when parts == 0
+  int parts;         // > 0: CTAs per unit, each with an even share of its steps
+  long long total;   // units * steps
   float scale_log2;
 };
 
@@ -50,10 +58,5 @@ __device__ __forceinline__ UnitInfo decode_unit(const TcParams& p, long long u) 
 // k_attend_decode.cu: the load-bound kernel for questions of at most 16 rows per KV head
 constexpr int DEC_THREADS = 256;
 constexpr int DEC_WARPS = 8;
-constexpr uint32_t DEC_SCRATCH = DEC_WARPS * 16 * (128 + 2) * 4;  // the warps' (O, max, sum) at the end of a range
-__global__ void attend_decode_kernel(const TcParams p);
-// k_attend_combine.cu: joins the (max, sum, O) partials of a unit's parts
-__global__ void combine_tc5_kernel(const TcParams p);
-__global__ void combine_many_kernel(const TcParams p);  // units of many parts (launches of few units)
-
+constexpr uint32_t DEC_SCRATCH = DEC_WARPS * 16 * (132 + 2) * 4;  // the warps' (O, max, sum) at the end of a range
 }  // namespace rekv_att

@@ -118,6 +118,12 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t& r0, uint32_t& r1, ui
                : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
                : "r"(addr));
 }
+// an 8x8 matrix of 16-bit values held as a fragment (row lane / 4, columns 2 (lane % 4) ..), transposed
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
+  uint32_t d;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
+  return d;
+}
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
@@ -138,6 +144,15 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return r;
 }
 
+
+// Rotary embedding of two pairs (x_i, y_i) held as bf16 in the halves of lo and hi; cs = (cos_0, sin_0, cos_1, sin_1).
+// (x, y) -> (x cos - y sin, y cos + x sin); each product rounded once into the sum, the result to bf16
+__device__ __forceinline__ void rotate_pair(uint32_t& lo, uint32_t& hi, const float4& cs) {
+  const float x0 = __uint_as_float(lo << 16), x1 = __uint_as_float(lo & 0xFFFF0000u);
+  const float y0 = __uint_as_float(hi << 16), y1 = __uint_as_float(hi & 0xFFFF0000u);
+  lo = pack_bf16(fmaf(x0, cs.x, -y0 * cs.y), fmaf(x1, cs.z, -y1 * cs.w));
+  hi = pack_bf16(fmaf(y0, cs.x, x0 * cs.y), fmaf(y1, cs.z, x1 * cs.w));
+}
 
 // ---- 5th-generation tensor cores: tensor memory (TMEM) and tcgen05.mma -------------------------
 // TMEM address: bits 31..16 lane, bits 15..0 column (one column = 32 bits per lane).

@@ -67,8 +67,6 @@ void free_ctx(rekv_ctx* c) {
   cudaFree(c->status);
   cudaFree(c->idx_own);
   cudaFree(c->ext_emb);
-  cudaFree(c->self_o);
-  cudaFree(c->self_ml);
   cudaFree(c->x_kv);
   cudaFree(c->q_rot);
   cudaFree(c->rope_tab);
@@ -103,6 +101,8 @@ int attend_one_layer(rekv_ctx* c, int layer, const void* q, const QBatch& qb, vo
   }
   REKV_CUDA(c, rekv_launch_attend_tc5(c, layer_view(q, layer, qb.sumNq * row_bytes), qb, c->g_ncf, layer, layer + 1,
                       layer_view(out, layer, qb.sumNq * row_bytes), st, false, nullptr));
+  c->ctx_settled = s.tail == 0;
+  c->ctx_stream = st;
   if (s.tail > 0) {
     // later appends (ring slots) and gathers (staging) on the side stream must not overtake this read
     REKV_CUDA(c, cudaEventRecord(c->ev_side, st));
@@ -175,7 +175,6 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
   c->status = nullptr;
   c->link_bytes = nullptr;
   c->idx_own = nullptr;
-  c->self_o = c->self_ml = nullptr;
   c->ext_emb = nullptr;
   c->ext_frames = 0;
   c->x_kv = nullptr;
@@ -245,8 +244,6 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
                 "allocating the embedding table");
   if (c->cfg.max_self_tokens > 0) {  // workspaces of rekv_attend_full
     const size_t rows = (size_t)s.L * c->cfg.max_q_tokens * s.Hq;
-    CREATE_CUDA(cudaMalloc(&c->self_o, rows * 128 * sizeof(float)), "allocating the self-attention partials");
-    CREATE_CUDA(cudaMalloc(&c->self_ml, rows * 2 * sizeof(float)), "allocating the self-attention partials");
     c->x_rows = ((c->cfg.max_self_tokens + 7) & ~7) + 8ll * maxQ;  // every question starts on a multiple of 8 rows
     CREATE_CUDA(cudaMalloc(&c->x_kv, (size_t)s.L * s.Hkv * 4 * c->x_rows * 128), "allocating the staged own keys and values");
     if (c->cfg.rope_theta > 0.f) {
@@ -427,6 +424,7 @@ int rekv_gather(rekv_ctx* c, const int32_t* idx, int nQ, int top_k, int n_visibl
   }
   c->gathered = true;
   c->layer_ctx_valid.assign(s.L, 1);
+  c->ctx_settled = false;
   c->g_nQ = nQ;
   c->g_ncf = ncf;
   c->g_keff = k_eff;
@@ -460,6 +458,8 @@ int rekv_attend(rekv_ctx* c, const void* q, const int32_t* cu_q, int nQ, void* o
   auto launch = rekv_launch_attend_tc5;
   if (!c->gather_layerwise) {
     REKV_CUDA(c, launch(c, q, qb, c->g_ncf, 0, s.L, out, st, (c->cfg.flags & REKV_FLAG_TIMING) != 0, nullptr));
+    c->ctx_settled = s.tail == 0;
+    c->ctx_stream = st;
   } else {
     for (int l = 0; l < s.L; ++l) {
       REKV_CUDA(c, cudaStreamWaitEvent(st, c->layer_events[l], 0));
@@ -506,6 +506,7 @@ int rekv_question(rekv_ctx* c, const void* q, const int32_t* cu_q, int nQ, int t
   c->pull_timed = false;
   c->gathered = true;
   c->layer_ctx_valid.assign(s.L, 1);
+  c->ctx_settled = false;
   c->gather_layerwise = false;
   c->g_nQ = nQ;
   c->g_ncf = geom.ncf;
@@ -518,7 +519,7 @@ int rekv_question(rekv_ctx* c, const void* q, const int32_t* cu_q, int nQ, int t
 
 namespace {
 int attend_full_range(rekv_ctx* c, int layer0, int layer1, const void* q, const void* k_self, const void* v_self,
-                      const QBatch& qb, const QBatch& sb, void* out, cudaStream_t st, bool self_done);
+                      const QBatch& qb, const QBatch& sb, void* out, cudaStream_t st);
 int build_self_batch(rekv_ctx* c, const QBatch& qb, const int32_t* cu_self, int nQ, QBatch* sb);
 }  // namespace
 
@@ -549,15 +550,6 @@ static int question_layer_impl(rekv_ctx* c, int layer, const void* q, const void
   const long long row_bytes = (long long)s.Hq * REKV_HEAD_DIM * 2;
   // the selection goes to the caller's buffer if there is one, else to the context's own
   int32_t* idx = idx_out ? layer_view(idx_out, layer, (long long)nQ * top_k * 4) : c->idx_own;
-  // Eq. 3 in full on an HBM-resident cache: the part over X needs nothing of the retrieval, so it starts on the internal
-  // stream now and runs beside the layer's retrieval kernels (it joins before the attention kernel)
-  const bool self_early = k_self != nullptr && s.tail == 0 && geom.ncf > 0;
-  if (self_early) {
-    const long long kv_layer = (long long)sb.sumNq * s.Hkv * REKV_HEAD_DIM * 2;
-    REKV_CUDA(c, rekv_launch_attend_full_self(c, layer_view(q, layer, qb.sumNq * row_bytes),
-                                              layer_view(k_self, layer, kv_layer), layer_view(v_self, layer, kv_layer),
-                                              qb, sb, geom.ncf, st, layer, layer + 1, true));
-  }
   // cache all in HBM: the selection kernel writes the layer's context table itself (top_k > 0 launches it)
   const bool fused_table = s.tail == 0 && top_k > 0;
   REKV_CUDA(c, rekv_launch_retrieve(c, layer_view(q, layer, qb.sumNq * row_bytes), qb, top_k, geom, n_visible, layer,
@@ -577,6 +569,7 @@ static int question_layer_impl(rekv_ctx* c, int layer, const void* q, const void
   // contexts the other layers built under the old one are gone
   if (!c->gathered || c->g_nQ != nQ || c->g_ncf != geom.ncf) c->layer_ctx_valid.assign(s.L, 0);
   c->layer_ctx_valid[layer] = 1;
+  c->ctx_settled = false;
   c->gathered = true;
   c->gather_layerwise = s.tail > 0;
   c->g_nQ = nQ;
@@ -588,7 +581,7 @@ static int question_layer_impl(rekv_ctx* c, int layer, const void* q, const void
     const long long kv_layer = (long long)sb.sumNq * s.Hkv * REKV_HEAD_DIM * 2;
     rc = attend_full_range(c, layer, layer + 1, layer_view(q, layer, qb.sumNq * row_bytes),
                            layer_view(k_self, layer, kv_layer), layer_view(v_self, layer, kv_layer), qb, sb,
-                           layer_view(out, layer, qb.sumNq * row_bytes), st, self_early);
+                           layer_view(out, layer, qb.sumNq * row_bytes), st);
     return rc ? rc : geom.ncf;
   }
   c->q_early_ok = fused_table;  // the selection kernel, which only reads Q, is directly before the attention
@@ -684,23 +677,23 @@ int build_self_batch(rekv_ctx* c, const QBatch& qb, const int32_t* cu_self, int 
 // Eq. 3 in full for layers [layer0, layer1).  q, k_self, v_self and out are indexed with the absolute layer: a caller
 // that holds one layer's rows passes pointers moved back by layer0 layers (layer_view).
 int attend_full_range(rekv_ctx* c, int layer0, int layer1, const void* q, const void* k_self, const void* v_self,
-                      const QBatch& qb, const QBatch& sb, void* out, cudaStream_t st, bool self_done) {
+                      const QBatch& qb, const QBatch& sb, void* out, cudaStream_t st) {
   // an offloaded context: the range's pages must have arrived before the keys are rotated
   if (c->gather_layerwise) REKV_CUDA(c, cudaStreamWaitEvent(st, c->layer_events[layer1 - 1], 0));
-  if (!self_done)
-    REKV_CUDA(c, rekv_launch_attend_full_self(c, q, k_self, v_self, qb, sb, c->g_ncf, st, layer0, layer1, false));
+  REKV_CUDA(c, rekv_launch_attend_full_self(c, q, k_self, v_self, qb, sb, c->g_ncf, st, layer0, layer1));
   REKV_CUDA(c, rekv_launch_attend_full_ctx(c, qb, c->g_ncf, st, layer0, layer1));
-  const bool rope = c->cfg.rope_theta > 0.f && !(c->cfg.flags & REKV_FLAG_ROPE_STATIC);  // rotated copies of the context's keys
-  const bool rope_q = c->cfg.rope_theta > 0.f;
   AttendFullArgs fa;
-  fa.tbl_k = rope && c->g_ncf > 0 ? c->tbl_k : nullptr;
-  fa.self_o = c->self_o;
-  fa.self_ml = c->self_ml;
+  fa.sb = &sb;
+  fa.tbl_k = rekv_rope_ctx(c) && c->g_ncf > 0 ? c->tbl_k : nullptr;
   fa.x_kv = c->x_kv;
   fa.x_rows = c->x_rows;
-  fa.sb = &sb;
-  REKV_CUDA(c, rekv_launch_attend_tc5(c, rope_q ? (const void*)c->q_rot : q, qb, c->g_ncf, layer0, layer1, out, st,
-                                      (c->cfg.flags & REKV_FLAG_TIMING) != 0 && layer1 - layer0 == c->sv.L, &fa));
+  fa.q = q;
+  fa.k_self = k_self;
+  fa.v_self = v_self;
+  REKV_CUDA(c, rekv_launch_attend_tc5(c, c->cfg.rope_theta > 0.f ? (const void*)c->q_rot : q, qb, c->g_ncf, layer0, layer1, out,
+                                      st, (c->cfg.flags & REKV_FLAG_TIMING) != 0 && layer1 - layer0 == c->sv.L, &fa));
+  c->ctx_settled = c->sv.tail == 0;
+  c->ctx_stream = st;
   if (c->gather_layerwise || (c->sv.tail > 0 && layer1 - layer0 < c->sv.L)) {
     // later appends (ring slots) and gathers (staging) on the side stream must not overtake this read
     REKV_CUDA(c, cudaEventRecord(c->ev_side, st));
@@ -727,7 +720,7 @@ int rekv_attend_full(rekv_ctx* c, const void* q, const void* k_self, const void*
   rc = build_self_batch(c, qb, cu_self, nQ, &sb);
   if (rc) return rc;
   DeviceGuard guard(c->device);
-  return attend_full_range(c, 0, c->sv.L, q, k_self, v_self, qb, sb, out, (cudaStream_t)stream, false);
+  return attend_full_range(c, 0, c->sv.L, q, k_self, v_self, qb, sb, out, (cudaStream_t)stream);
 }
 
 int rekv_attend_full_layer(rekv_ctx* c, int layer, const void* q, const void* k_self, const void* v_self,
@@ -751,7 +744,7 @@ int rekv_attend_full_layer(rekv_ctx* c, int layer, const void* q, const void* k_
   const long long kv_layer = (long long)sb.sumNq * s.Hkv * REKV_HEAD_DIM * 2;
   return attend_full_range(c, layer, layer + 1, layer_view(q, layer, q_layer), layer_view(k_self, layer, kv_layer),
                            layer_view(v_self, layer, kv_layer), qb, sb, layer_view(out, layer, q_layer),
-                           (cudaStream_t)stream, false);
+                           (cudaStream_t)stream);
 }
 
 int rekv_geometry(rekv_ctx* c, int n_visible, int top_k, int32_t* n_scored, int32_t* k_eff, int32_t* w_eff) {

@@ -125,8 +125,6 @@ struct rekv_ctx {
   int ext_frames;                   // embeddings are set for frames [0, ext_frames)
 
   // Eq. 3 in full (allocated when max_self_tokens > 0)
-  float* self_o;                    // [L][max_q_tokens][H_q][128]
-  float* self_ml;                   // [L][max_q_tokens][H_q][2]
   char* x_kv;                       // [L][H_kv][K, V][half][x_rows][128 B] X's keys and values in the page layout
   long long x_rows;
   __nv_bfloat16* q_rot;             // [L][max_q_tokens][H_q][128] rotated queries (rope_theta > 0)
@@ -139,8 +137,12 @@ struct rekv_ctx {
   // test-only knobs of the bounded device-side waits (rekv_test_set_wait_limit); 0 / -1 = off
   unsigned test_wait_limit;
   int test_skip_copy_entry;
-  bool self_forked = false;         // Eq. 3 in full: the part over X is on the internal stream, ev_side marks its end
   bool q_early_ok = false;          // the attention launch that follows is chained to the library's own selection kernels (which only read Q)
+
+  // An attention launch on ctx_stream has read the whole context table since it was last written (it waited for the table's
+  // writer): later launches on that stream may read the table and an HBM-resident cache's pages before their own wait.
+  bool ctx_settled = false;
+  cudaStream_t ctx_stream = nullptr;
 
   // state of the last gather.  The context table has one geometry (questions x context frames) for all layers; a
   // layer's context is valid while the table still has the geometry it was built with (layer_ctx_valid).
@@ -227,15 +229,22 @@ inline cudaError_t rekv_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 blo
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// Extra inputs of the attention kernel for Eq. 3 in full.
+// Extra inputs of the attention kernels for Eq. 3 in full.
 struct AttendFullArgs {
-  char* const* tbl_k;    // rotated K tiles per context slot (null without rotary embedding)
-  const float* self_o;   // decode-shaped batches: [L][sum_Nq][H_q][128] partial numerators over the tokens of X
-  const float* self_ml;  // [L][sum_Nq][H_q][2] their (max, sum), log2 domain
-  const char* x_kv;      // the tensor-core kernel: X's K/V staged in the page layout (stage_x_kernel)
-  long long x_rows;      // its rows per (layer, kv head, K/V, half)
   const QBatch* sb;      // X's lengths
+  // the tensor-core kernel
+  char* const* tbl_k;    // rotated K tiles per context slot (null without rotary embedding)
+  const char* x_kv;      // X's K/V staged in the page layout (stage_x_kernel)
+  long long x_rows;      // its rows per (layer, kv head, K/V, half)
+  // the decode-shaped kernel: as the caller passes them
+  const void* q;
+  const void* k_self;
+  const void* v_self;
 };
+// Positions (rotary embedding): context token j at j and token s of X at n_ctx + s; with REKV_FLAG_ROPE_STATIC every
+// context token at 0 -- its rotation is the identity, the stored keys are used as they are -- and token s of X at 1 + s.
+inline bool rekv_rope_ctx(const rekv_ctx* c) { return c->cfg.rope_theta > 0.f && !(c->cfg.flags & REKV_FLAG_ROPE_STATIC); }
+inline int rekv_pos_x(const rekv_ctx* c, int ncf) { return rekv_rope_ctx(c) ? ncf * c->sv.Nf : 1; }
 
 // ---- kernel launchers (each returns the cudaError_t of its launches) -----------------------
 // k_append.cu
@@ -264,6 +273,6 @@ cudaError_t rekv_launch_attend_decode(rekv_ctx* c, const void* q, const QBatch& 
 cudaError_t rekv_launch_rope_table(rekv_ctx* c, cudaStream_t st);
 cudaError_t rekv_launch_attend_full_self(rekv_ctx* c, const void* q, const void* k_self, const void* v_self,
                                          const QBatch& qb, const QBatch& sb, int ncf, cudaStream_t st, int layer0,
-                                         int layer1, bool early);
+                                         int layer1);
 cudaError_t rekv_launch_attend_full_ctx(rekv_ctx* c, const QBatch& qb, int ncf, cudaStream_t st, int layer0,
                                         int layer1);

@@ -171,7 +171,8 @@ class ReKV:
         return rc
 
     def _stream(self) -> int:
-        return torch.cuda.current_stream(self.device).cuda_stream
+        # the raw handle of torch's current stream, without building a Stream object for every call
+        return torch._C._cuda_getCurrentRawStream(self.device.index)
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
@@ -197,7 +198,7 @@ class ReKV:
                  want_scores: bool = False) -> Tuple[torch.Tensor, int, Optional[torch.Tensor]]:
         """q: bf16 [L][sum_Nq][H_q][D].  Returns (idx int32 [L][nQ][top_k], k_eff, scores or None)."""
         nQ = len(cu_q) - 1
-        if tuple(q.shape) != (self.L, cu_q[-1], self.Hq, self.D):
+        if q.shape != (self.L, cu_q[-1], self.Hq, self.D):
             raise ValueError("q must be [L][sum_Nq][H_q][D]")
         idx = torch.empty((self.L, nQ, max(top_k, 0)), dtype=torch.int32, device=self.device)
         n_scored = self.geometry(n_visible, top_k)[0]
@@ -238,7 +239,7 @@ class ReKV:
         a selection the caller passes."""
         nQ = len(cu_q) - 1
         if idx is None:
-            if tuple(q.shape) != (self.L, cu_q[-1], self.Hq, self.D):
+            if q.shape != (self.L, cu_q[-1], self.Hq, self.D):
                 raise ValueError("q must be [L][sum_Nq][H_q][D]")
             if out is None:
                 out = torch.empty_like(q)
@@ -269,7 +270,7 @@ class ReKV:
                     cu_self: Sequence[int], out: Optional[torch.Tensor] = None) -> torch.Tensor:
         """Eq. 3 in full over the gathered context followed by the questions' own K/V (causal).
         q: bf16 [L][sum_Nq][H_q][D]; k_self, v_self: bf16 [L][sum_Ns][H_kv][D] -> bf16 like q."""
-        if tuple(q.shape) != (self.L, cu_q[-1], self.Hq, self.D):
+        if q.shape != (self.L, cu_q[-1], self.Hq, self.D):
             raise ValueError("q must be [L][sum_Nq][H_q][D]")
         if tuple(k_self.shape) != (self.L, cu_self[-1], self.Hkv, self.D) or k_self.shape != v_self.shape:
             raise ValueError("k_self and v_self must be [L][sum_Ns][H_kv][D]")
@@ -285,7 +286,7 @@ class ReKV:
         """retrieve -> gather -> attend of one layer.  q: bf16 [sum_Nq][H_q][D] of that layer -> same shape.
         idx (optional, int32 [nQ][top_k]) receives the layer's selection."""
         nQ = len(cu_q) - 1
-        if tuple(q.shape) != (cu_q[-1], self.Hq, self.D):
+        if q.shape != (cu_q[-1], self.Hq, self.D):
             raise ValueError("q must be [sum_Nq][H_q][D]")
         if idx is not None and tuple(idx.shape) != (nQ, top_k):
             raise ValueError("idx must be [nQ][top_k]")
@@ -326,15 +327,15 @@ class ReKV:
         return out
 
     def _check_layer_full_shapes(self, q, k_self, v_self, cu_q, cu_self):
-        if tuple(q.shape) != (cu_q[-1], self.Hq, self.D):
+        if q.shape != (cu_q[-1], self.Hq, self.D):
             raise ValueError("q must be [sum_Nq][H_q][D]")
-        if tuple(k_self.shape) != (cu_self[-1], self.Hkv, self.D) or k_self.shape != v_self.shape:
+        if k_self.shape != (cu_self[-1], self.Hkv, self.D) or k_self.shape != v_self.shape:
             raise ValueError("k_self and v_self must be [sum_Ns][H_kv][D]")
 
     def attend_layer(self, layer: int, q: torch.Tensor, cu_q: Sequence[int],
                      out: Optional[torch.Tensor] = None) -> torch.Tensor:
         """Attention of one layer over the context its last question_layer (or gather) built."""
-        if tuple(q.shape) != (cu_q[-1], self.Hq, self.D):
+        if q.shape != (cu_q[-1], self.Hq, self.D):
             raise ValueError("q must be [sum_Nq][H_q][D]")
         if out is None:
             out = torch.empty_like(q)
