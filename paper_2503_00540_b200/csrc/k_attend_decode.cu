@@ -216,38 +216,37 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) attend_decode_kernel(const __g
 #pragma unroll 1
       for (int un = u0; un < u1 && ok; ++un) {
         const int t0 = un * 16;
-        uint32_t a[8][4];  // K: tokens lg (+ 8), dims 16 kb + 2 lt (+ 8)
-        {
-          const int tok = t0 + (lm & 1) * 8 + lr;
+        // S^T of the unit, two chains of four products.  K fragments: tokens lg (+ 8), dims 16 kb + 2 lt (+ 8); chunk
+        // 2 kb + (lm >> 1) of the row, swizzled with row & 7 = lr, so that the k-block only flips address bits 5 and 6
+        const uint32_t a0 = sK + (uint32_t)(t0 + (lm & 1) * 8 + lr) * 128u + (uint32_t)(((lm >> 1) ^ lr) << 4);
+        float sacc[NT][4], s2[NT][4];
 #pragma unroll
-          for (int kb = 0; kb < 8; ++kb) {
-            const int c = 2 * kb + (lm >> 1);
-            const uint32_t addr = sK + (c >> 3) * half_stride + tok * 128 + (((c & 7) ^ (tok & 7)) << 4);
-            a[kb][0] = a[kb][1] = a[kb][2] = a[kb][3] = 0;
-            if (DEC_GUARD(addr + 16 <= s_base + ring_bytes && (addr & 15) == 0, 3))
-              ldmatrix_x4(a[kb][0], a[kb][1], a[kb][2], a[kb][3], addr);
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) sacc[nt][e] = s2[nt][e] = 0.f;
+#pragma unroll
+        for (int kb = 0; kb < 4; ++kb) {
+          uint32_t a[4] = {0, 0, 0, 0}, b[4] = {0, 0, 0, 0};
+          const uint32_t addr = a0 ^ (uint32_t)(kb << 5);
+          if (DEC_GUARD(addr + half_stride + 16 <= s_base + ring_bytes && (addr & 15) == 0, 3)) {
+            ldmatrix_x4(a[0], a[1], a[2], a[3], addr);
+            ldmatrix_x4(b[0], b[1], b[2], b[3], addr + half_stride);
           }
-        }
-        if (rot) {
+          if (rot) {
 #pragma unroll
-          for (int kb = 0; kb < 4; ++kb)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) rotate_pair(a[kb][e], a[kb + 4][e], cs[kb][e]);
-          if (un + 1 < u1) ask_cs(un + 1);
-        }
-        float sacc[NT][4];
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          float s2[4] = {0.f, 0.f, 0.f, 0.f};  // two chains of four products
-          sacc[nt][0] = sacc[nt][1] = sacc[nt][2] = sacc[nt][3] = 0.f;
-#pragma unroll
-          for (int kb = 0; kb < 4; ++kb) {
-            mma_bf16_16816(sacc[nt], a[kb], qf[nt][kb][0], qf[nt][kb][1]);
-            mma_bf16_16816(s2, a[kb + 4], qf[nt][kb + 4][0], qf[nt][kb + 4][1]);
+            for (int e = 0; e < 4; ++e) rotate_pair(a[e], b[e], cs[kb][e]);
           }
 #pragma unroll
-          for (int e = 0; e < 4; ++e) sacc[nt][e] += s2[e];
+          for (int nt = 0; nt < NT; ++nt) {
+            mma_bf16_16816(sacc[nt], a, qf[nt][kb][0], qf[nt][kb][1]);
+            mma_bf16_16816(s2[nt], b, qf[nt][kb + 4][0], qf[nt][kb + 4][1]);
+          }
         }
+        if (rot && un + 1 < u1) ask_cs(un + 1);
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) sacc[nt][e] += s2[nt][e];
         uint32_t pf[NT][2];
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
@@ -281,11 +280,10 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) attend_decode_kernel(const __g
           pf[nt][0] = movmatrix_trans(pack_bf16(sacc[nt][0], sacc[nt][1]));
           pf[nt][1] = movmatrix_trans(pack_bf16(sacc[nt][2], sacc[nt][3]));
         }
-        const int tok = t0 + (lm >> 1) * 8 + lr;
+        const uint32_t v0 = sV + (uint32_t)(t0 + (lm >> 1) * 8 + lr) * 128u + (uint32_t)(((lm & 1) ^ lr) << 4);
 #pragma unroll
         for (int dm = 0; dm < 8; ++dm) {
-          const int c = 2 * dm + (lm & 1);
-          const uint32_t addr = sV + (c >> 3) * half_stride + tok * 128 + (((c & 7) ^ (tok & 7)) << 4);
+          const uint32_t addr = (v0 ^ (uint32_t)((dm & 3) << 5)) + (dm >= 4 ? half_stride : 0u);
           uint32_t v[4] = {0, 0, 0, 0};
           if (DEC_GUARD(addr + 16 <= s_base + ring_bytes && (addr & 15) == 0, 4)) ldmatrix_x4_trans(v[0], v[1], v[2], v[3], addr);
 #pragma unroll
@@ -383,8 +381,9 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) attend_decode_kernel(const __g
       if (s_last) {
         __threadfence();
         // a warp per row, a float4 of its 128 columns per lane; a lane's (max, sum) are those of parts k0 + lane and
-        // k0 + 32 + lane.  Twenty parts' rows are in flight: 37 parts (one layer) are two rounds deep.
-        constexpr int U = 20;
+        // k0 + 32 + lane.  The rows of U parts are in flight (28 layers, 37 parts each: twelve 575 us, twenty 612, whose
+        // registers spill).
+        constexpr int U = 12;
         for (int r = warp; r < ui.rows_q; r += DEC_WARPS) {
           const float2* ml_r = reinterpret_cast<const float2*>(p.part_ml) + part_of(u, c_first) * 16 + r;
           const float4* o_r = reinterpret_cast<const float4*>(p.part_o + (part_of(u, c_first) * 16 + r) * 128) + lane;
