@@ -1,18 +1,24 @@
 // Step 1: page a frame's K/V into the store and pool its keys into the frame representative
 // (internal retrieval: v = 1/N_f * sum_j k_j, heads concatenated), in one pass over the frame.
+#include "ptx_helpers.cuh"
 #include "rekv_internal.cuh"
 
 namespace {
 
-// grid = L * H_kv * 2 (K tiles pool, V tiles only move); 256 threads: 16 row groups x 16 chunks.
+// grid = L * H_kv * 2 (K tiles pool, V tiles only move); 512 threads: 32 row groups x 16 chunks, eight rows per thread in
+// flight, so that a frame of up to 256 tokens is one round of loads deep: a frame (22.5 MB read and written at 28 layers, 4 KV
+// heads, 196 tokens: 3.5 us) is over before a second round of latency would be.
 // Source rows are 256-byte segments (one head of one token), read as 16-byte chunks; the page is
 // written in the swizzled tile layout.  Pooling accumulates in fp32 in a fixed order.
-__global__ void __launch_bounds__(256) append_pool_kernel(const uint4* __restrict__ k_in,
+constexpr int AP_GROUPS = 32, AP_ROWS = 8;
+__global__ void __launch_bounds__(16 * AP_GROUPS) append_pool_kernel(const uint4* __restrict__ k_in,
                                                           const uint4* __restrict__ v_in, char* __restrict__ page0,
                                                           float* __restrict__ reps, int frame, int L, int Hkv,
                                                           int Nf, int max_frames, long long page_bytes,
                                                           long long store_bytes, char* __restrict__ store,
                                                           int* __restrict__ status) {
+  rekv_ptx::grid_dep_wait();
+  rekv_ptx::grid_dep_launch();
   const int kv = blockIdx.x & 1;
   const int h = (blockIdx.x >> 1) % Hkv;
   const int l = (blockIdx.x >> 1) / Hkv;
@@ -26,17 +32,16 @@ __global__ void __launch_bounds__(256) append_pool_kernel(const uint4* __restric
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0.f;
 
-  // four rows per thread in flight
-  for (int t0 = rg; t0 < Nf; t0 += 64) {
-    uint4 x[4];
+  for (int t0 = rg; t0 < Nf; t0 += AP_GROUPS * AP_ROWS) {
+    uint4 x[AP_ROWS];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int t = t0 + 16 * u;
-      if (t < Nf) x[u] = __ldg(src + (long long)t * Hkv * 16);
+    for (int u = 0; u < AP_ROWS; ++u) {
+      const int t = t0 + AP_GROUPS * u;
+      if (t < Nf) x[u] = __ldcs(src + (long long)t * Hkv * 16);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int t = t0 + 16 * u;
+    for (int u = 0; u < AP_ROWS; ++u) {
+      const int t = t0 + AP_GROUPS * u;
       if (t < Nf) {
         char* dst = tile + t * 128 + ((cc ^ (t & 7)) << 4);
         if (!REKV_CHECK(dst >= store && dst + 16 <= store + store_bytes && (reinterpret_cast<uintptr_t>(dst) & 15) == 0,
@@ -56,14 +61,14 @@ __global__ void __launch_bounds__(256) append_pool_kernel(const uint4* __restric
     }
   }
   if (kv == 0) {
-    __shared__ float red[16][129];
+    __shared__ float red[AP_GROUPS][129];
 #pragma unroll
     for (int i = 0; i < 8; ++i) red[rg][c * 8 + i] = acc[i];
     __syncthreads();
     if (threadIdx.x < 128) {
       float s = 0.f;
 #pragma unroll
-      for (int r = 0; r < 16; ++r) s += red[r][threadIdx.x];
+      for (int r = 0; r < AP_GROUPS; ++r) s += red[r][threadIdx.x];
       if (REKV_CHECK(frame >= 0 && frame < max_frames && l < L, status, 2))
         reps[((long long)l * max_frames + frame) * (Hkv * 128) + h * 128 + threadIdx.x] = __fdiv_rn(s, (float)Nf);
     }
@@ -92,10 +97,10 @@ __global__ void unswizzle_page_kernel(const char* __restrict__ page, uint4* __re
 cudaError_t rekv_launch_append(rekv_ctx* c, const void* k, const void* v, int frame, cudaStream_t st) {
   const StoreView& s = c->sv;
   char* page0 = s.hbm + rekv_hbm_page_offset(s, frame, 0);
-  append_pool_kernel<<<s.L * s.Hkv * 2, 256, 0, st>>>((const uint4*)k, (const uint4*)v, page0, s.reps, frame, s.L,
-                                                      s.Hkv, s.Nf, s.max_frames, s.page_bytes,
-                                                      (long long)(s.tail > 0 ? s.tail : s.max_frames) * s.L * s.page_bytes,
-                                                      s.hbm, c->status);
+  cudaError_t e = rekv_launch_pdl(append_pool_kernel, dim3(s.L * s.Hkv * 2), dim3(16 * AP_GROUPS), 0, st, (const uint4*)k,
+                                  (const uint4*)v, page0, s.reps, frame, s.L, s.Hkv, s.Nf, s.max_frames, s.page_bytes,
+                                  (long long)(s.tail > 0 ? s.tail : s.max_frames) * s.L * s.page_bytes, s.hbm, c->status);
+  if (e != cudaSuccess) return e;
   c->launches += 1;
   return cudaGetLastError();
 }

@@ -451,7 +451,7 @@ size_t decode_smem(int Nf) {
 bool rekv_decode_shaped(const rekv_ctx* c, const QBatch& qb, int ncf, int nl) {
   for (int i = 0; i < qb.nQ; ++i)
     if ((qb.cu[i + 1] - qb.cu[i]) * c->sv.G > 16) return false;
-  return ncf > 0 && decode_smem(c->sv.Nf) <= 227 * 1024 && (size_t)nl * c->sv.Hkv * qb.nQ <= c->part_units;
+  return ncf > 0 && decode_smem(c->sv.Nf) <= 227 * 1024 && (size_t)nl * c->sv.Hkv * qb.nQ <= c->cnt_units;
 }
 
 cudaError_t rekv_launch_attend_decode(rekv_ctx* c, const void* q, const QBatch& qb, int ncf, int layer0, int layer1,

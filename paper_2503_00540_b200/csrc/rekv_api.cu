@@ -52,27 +52,7 @@ int build_qbatch(rekv_ctx* c, const int32_t* cu_q, int nQ, QBatch* qb) {
 void free_ctx(rekv_ctx* c) {
   if (!c) return;
   cudaDeviceSynchronize();
-  cudaFree(c->sv.hbm);
-  cudaFree(c->sv.staging);
-  cudaFree(c->sv.q8_ring);
-  cudaFree(c->sv.reps);
-  cudaFree(c->d_host_arenas);
-  cudaFree(c->qa);
-  cudaFree(c->qnorm);
-  cudaFree(c->scores);
-  cudaFree(c->ctx_tbl);
-  cudaFree(c->part_o);
-  cudaFree(c->part_ml);
-  cudaFree(c->unit_cnt);
-  cudaFree(c->status);
-  cudaFree(c->idx_own);
-  cudaFree(c->ext_emb);
-  cudaFree(c->x_kv);
-  cudaFree(c->q_rot);
-  cudaFree(c->rope_tab);
-  cudaFree(c->k_rot);
-  cudaFree(c->tbl_k);
-  cudaFree(c->link_bytes);
+  cudaFree(c->block);
   for (char* a : c->host_arenas) cudaFreeHost(a);
   for (cudaEvent_t e : c->slot_events) cudaEventDestroy(e);
   for (cudaEvent_t e : c->layer_events) cudaEventDestroy(e);
@@ -162,6 +142,7 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
   c->ev_main = c->ev_side = nullptr;
   c->ev_t0 = c->ev_t1 = c->ev_t2 = c->ev_r0 = c->ev_r1 = c->ev_p0 = c->ev_p1 = nullptr;
   c->timing_valid = c->merge_timed = c->retrieve_timed = c->pull_timed = false;
+  c->block = nullptr;
   c->h_link_bytes = nullptr;
   c->d2h_pending = false;
   c->ring_reader_ev = nullptr;
@@ -218,62 +199,86 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
     }                                                                                                        \
   } while (0)
 
+  // All device memory is one allocation: a cudaMalloc and its cudaFree cost 0.3 ms each whatever their size, and a stream's
+  // context is created and destroyed in the course of a program.
+  struct Piece {
+    void** at;
+    size_t bytes;
+  };
+  std::vector<Piece> pieces;
+  auto want = [&](auto** at, size_t bytes) { pieces.push_back({(void**)at, (bytes + 1023) & ~(size_t)1023}); };
   const long long hbm_frames = s.tail > 0 ? s.tail : s.max_frames;
-  CREATE_CUDA(cudaMalloc(&s.hbm, (size_t)(hbm_frames * frame_bytes)), "allocating the HBM frame store");
-  CREATE_CUDA(cudaMalloc(&s.reps, (size_t)s.L * s.max_frames * s.Dp * sizeof(float)), "allocating the representative table");
   const int ctx_frames_max = cfg->max_topk + cfg->window_frames + cfg->block_frames - 1;
   const int maxQ = cfg->max_questions;
-  CREATE_CUDA(cudaMalloc(&c->qa, (size_t)s.L * maxQ * s.Dp * sizeof(float)), "allocating question vectors");
-  CREATE_CUDA(cudaMalloc(&c->qnorm, (size_t)s.L * maxQ * s.Hkv * sizeof(float)), "allocating question norms");
-  CREATE_CUDA(cudaMalloc(&c->scores, (size_t)s.L * maxQ * s.max_frames * sizeof(float)), "allocating the score buffer");
-  CREATE_CUDA(cudaMalloc(&c->ctx_tbl, (size_t)s.L * maxQ * (ctx_frames_max + 1) * sizeof(char*)), "allocating the context table");
-  // 2048 slots cover every launch whose units are cut at CTA boundaries; launches of many whole units park two
-  // half-stream partials per unit with a single row tile (at most one per layer, KV head and question), up to a cap
-  c->part_units = std::min<size_t>(8192, std::max<size_t>(2048, (size_t)2 * s.L * s.Hkv * maxQ + 16));
-  CREATE_CUDA(cudaMalloc(&c->part_o, c->part_units * 128 * 128 * sizeof(float)), "allocating split-KV partials");
-  CREATE_CUDA(cudaMalloc(&c->part_ml, c->part_units * 128 * 2 * sizeof(float)), "allocating split-KV partials");
-  CREATE_CUDA(cudaMalloc(&c->unit_cnt, c->part_units * sizeof(int)), "allocating split-KV counters");
-  CREATE_CUDA(cudaMemset(c->unit_cnt, 0, c->part_units * sizeof(int)), "clearing split-KV counters");
-  CREATE_CUDA(cudaMalloc(&c->status, sizeof(int)), "allocating the status word");
-  CREATE_CUDA(cudaMemset(c->status, 0, sizeof(int)), "clearing the status word");
-  CREATE_CUDA(cudaMalloc(&c->idx_own, (size_t)s.L * maxQ * (c->cfg.max_topk > 0 ? c->cfg.max_topk : 1) * sizeof(int32_t)),
-              "allocating the selection buffer");
+  const int n_arenas = s.tail > 0 ? (s.max_frames + s.frames_per_arena - 1) / s.frames_per_arena : 0;
+  const bool static_ctx = (cfg->flags & REKV_FLAG_ROPE_STATIC) != 0;
+  const bool rope = cfg->max_self_tokens > 0 && cfg->rope_theta > 0.f;
   c->ctx_frames_max = ctx_frames_max;
-  if (c->cfg.ext_embed_dim > 0)
-    CREATE_CUDA(cudaMalloc(&c->ext_emb, (size_t)s.max_frames * c->cfg.ext_embed_dim * sizeof(float)),
-                "allocating the embedding table");
-  if (c->cfg.max_self_tokens > 0) {  // workspaces of rekv_attend_full
-    const size_t rows = (size_t)s.L * c->cfg.max_q_tokens * s.Hq;
-    c->x_rows = ((c->cfg.max_self_tokens + 7) & ~7) + 8ll * maxQ;  // every question starts on a multiple of 8 rows
-    CREATE_CUDA(cudaMalloc(&c->x_kv, (size_t)s.L * s.Hkv * 4 * c->x_rows * 128), "allocating the staged own keys and values");
-    if (c->cfg.rope_theta > 0.f) {
-      const bool static_ctx = (cfg->flags & REKV_FLAG_ROPE_STATIC) != 0;
-      c->rope_positions = (static_ctx ? 1 : ctx_frames_max * s.Nf) + c->cfg.max_self_tokens;
-      CREATE_CUDA(cudaMalloc(&c->q_rot, rows * 128 * sizeof(__nv_bfloat16)), "allocating rotated queries");
-      CREATE_CUDA(cudaMalloc(&c->rope_tab, (size_t)c->rope_positions * 64 * sizeof(float2)), "allocating the rotary table");
-      if (!static_ctx) {
-        CREATE_CUDA(cudaMalloc(&c->k_rot, (size_t)s.L * maxQ * ctx_frames_max * (s.page_bytes / 2)),
-                    "allocating rotated key tiles");
-        CREATE_CUDA(cudaMalloc(&c->tbl_k, (size_t)s.L * maxQ * (ctx_frames_max + 1) * sizeof(char*)),
-                    "allocating the rotated-key table");
-      }
-      CREATE_CUDA(rekv_launch_rope_table(c, 0), "building the rotary table");
-      CREATE_CUDA(cudaDeviceSynchronize(), "building the rotary table");
+  // partial results: at most four 128-row slots per worker of the tensor-core kernel, twice (two launches side by side); the
+  // decode-shaped kernel takes eight parts of 16 rows per slot
+  c->part_units = 1024;
+  c->cnt_units = std::max<size_t>(c->part_units, (size_t)s.L * s.Hkv * maxQ);
+  // counters first: they are cleared together
+  want(&c->unit_cnt, c->cnt_units * sizeof(int));
+  want(&c->status, sizeof(int));
+  want(&c->link_bytes, sizeof(unsigned long long));
+  size_t clear_bytes = 0;
+  for (const Piece& x : pieces) clear_bytes += x.bytes;
+  want(&s.hbm, (size_t)(hbm_frames * frame_bytes));
+  want(&s.reps, (size_t)s.L * s.max_frames * s.Dp * sizeof(float));
+  want(&c->qa, (size_t)s.L * maxQ * s.Dp * sizeof(float));
+  want(&c->qnorm, (size_t)s.L * maxQ * s.Hkv * sizeof(float));
+  want(&c->scores, (size_t)s.L * maxQ * s.max_frames * sizeof(float));
+  want(&c->ctx_tbl, (size_t)s.L * maxQ * (ctx_frames_max + 1) * sizeof(char*));
+  want(&c->part_o, c->part_units * 128 * 128 * sizeof(float));
+  want(&c->part_ml, c->part_units * 128 * 2 * sizeof(float));
+  want(&c->idx_own, (size_t)s.L * maxQ * std::max(cfg->max_topk, 1) * sizeof(int32_t));
+  if (cfg->ext_embed_dim > 0) want(&c->ext_emb, (size_t)s.max_frames * cfg->ext_embed_dim * sizeof(float));
+  if (cfg->max_self_tokens > 0) {  // workspaces of rekv_attend_full
+    c->x_rows = ((cfg->max_self_tokens + 7) & ~7) + 8ll * maxQ;  // every question starts on a multiple of 8 rows
+    want(&c->x_kv, (size_t)s.L * s.Hkv * 4 * c->x_rows * 128);
+  }
+  if (rope) {
+    c->rope_positions = (static_ctx ? 1 : ctx_frames_max * s.Nf) + cfg->max_self_tokens;
+    want(&c->q_rot, (size_t)s.L * cfg->max_q_tokens * s.Hq * 128 * sizeof(__nv_bfloat16));
+    want(&c->rope_tab, (size_t)c->rope_positions * 64 * sizeof(float2));
+    if (!static_ctx) {
+      want(&c->k_rot, (size_t)s.L * maxQ * ctx_frames_max * (s.page_bytes / 2));
+      want(&c->tbl_k, (size_t)s.L * maxQ * (ctx_frames_max + 1) * sizeof(char*));
     }
   }
-  CREATE_CUDA(cudaMalloc(&c->link_bytes, sizeof(unsigned long long)), "allocating counters");
-  CREATE_CUDA(cudaMemset(c->link_bytes, 0, sizeof(unsigned long long)), "clearing counters");
+  if (s.tail > 0) {
+    want(&c->d_host_arenas, n_arenas * sizeof(char*));
+    want(&s.staging, (size_t)s.L * maxQ * ctx_frames_max * s.page_bytes);
+    if (s.host_fp8) want(&s.q8_ring, (size_t)s.tail * host_frame_bytes);
+  }
+  size_t total = 0;
+  for (const Piece& x : pieces) total += x.bytes;
+  char what[96];
+  snprintf(what, sizeof(what), "allocating %zu MB of device memory (frame store and workspaces)", total >> 20);
+  CREATE_CUDA(cudaMalloc(&c->block, total), what);
+  {
+    char* at = c->block;
+    for (const Piece& x : pieces) {
+      *x.at = at;
+      at += x.bytes;
+    }
+  }
+  CREATE_CUDA(cudaMemset(c->unit_cnt, 0, clear_bytes), "clearing counters");
+  if (rope) {
+    CREATE_CUDA(rekv_launch_rope_table(c, 0), "building the rotary table");
+    CREATE_CUDA(cudaDeviceSynchronize(), "building the rotary table");
+  }
   CREATE_CUDA(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking), "creating the side stream");
   CREATE_CUDA(cudaEventCreateWithFlags(&c->ev_main, cudaEventDisableTiming), "creating events");
   CREATE_CUDA(cudaEventCreateWithFlags(&c->ev_side, cudaEventDisableTiming), "creating events");
   for (cudaEvent_t* e : {&c->ev_t0, &c->ev_t1, &c->ev_t2, &c->ev_r0, &c->ev_r1, &c->ev_p0, &c->ev_p1})
     CREATE_CUDA(cudaEventCreate(e), "creating events");
-  CREATE_CUDA(cudaHostAlloc((void**)&c->h_link_bytes, sizeof(unsigned long long), cudaHostAllocDefault), "allocating counters");
-  *c->h_link_bytes = 0;
 
   if (s.tail > 0) {
+    CREATE_CUDA(cudaHostAlloc((void**)&c->h_link_bytes, sizeof(unsigned long long), cudaHostAllocDefault), "allocating counters");
+    *c->h_link_bytes = 0;
     // pinned-host tier: arenas of whole frames, allocated up front so that append never blocks
-    const int n_arenas = (s.max_frames + s.frames_per_arena - 1) / s.frames_per_arena;
     for (int a = 0; a < n_arenas; ++a) {
       int fr = s.max_frames - a * s.frames_per_arena;
       if (fr > s.frames_per_arena) fr = s.frames_per_arena;
@@ -290,13 +295,9 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
       }
       c->host_arenas.push_back(p);
     }
-    CREATE_CUDA(cudaMalloc(&c->d_host_arenas, n_arenas * sizeof(char*)), "allocating the arena table");
     CREATE_CUDA(cudaMemcpy(c->d_host_arenas, c->host_arenas.data(), n_arenas * sizeof(char*), cudaMemcpyHostToDevice),
                 "uploading the arena table");
     s.host_arenas = c->d_host_arenas;
-    CREATE_CUDA(cudaMalloc(&s.staging, (size_t)s.L * maxQ * ctx_frames_max * s.page_bytes), "allocating gather staging");
-    if (s.host_fp8)
-      CREATE_CUDA(cudaMalloc(&s.q8_ring, (size_t)s.tail * host_frame_bytes), "allocating the quantised write-through ring");
     c->slot_events.resize(s.tail);
     c->slot_event_valid.assign(s.tail, 0);
     for (int i = 0; i < s.tail; ++i)
@@ -402,7 +403,6 @@ int rekv_gather(rekv_ctx* c, const int32_t* idx, int nQ, int top_k, int n_visibl
     REKV_CUDA(c, rekv_launch_page_table(c, idx, nQ, top_k, geom, n_visible, 0, s.L, c->frames, st));
     c->gather_layerwise = false;
     c->pull_timed = false;
-    *c->h_link_bytes = 0;
   } else {
     // host tier: the pulls run layer by layer on the side stream (behind every write-through that is
     // still in flight there); attention of layer l only waits for layer l's event
@@ -773,7 +773,7 @@ int rekv_stats(rekv_ctx* c, rekv_stats_t* out) {
   out->kv_bytes_logical = 2ll * s.L * c->frames * s.Nf * s.Hkv * REKV_HEAD_DIM * 2;
   out->rep_bytes = (long long)s.L * c->frames * s.Dp * (long long)sizeof(float);
   // nothing here waits for the device: counters and timings are those of the work that has completed
-  out->last_link_bytes = (int64_t)*c->h_link_bytes;
+  out->last_link_bytes = c->h_link_bytes ? (int64_t)*c->h_link_bytes : 0;
   auto elapsed_us = [](cudaEvent_t a, cudaEvent_t b) -> double {
     float ms = 0.f;
     if (cudaEventQuery(b) != cudaSuccess || cudaEventElapsedTime(&ms, a, b) != cudaSuccess) {
@@ -818,7 +818,7 @@ int rekv_check_status(rekv_ctx* c, void* stream) {
   REKV_CUDA(c, cudaMemcpy(&st, c->status, sizeof(int), cudaMemcpyDeviceToHost));
   if (st != 0) {
     REKV_CUDA(c, cudaMemset(c->status, 0, sizeof(int)));
-    REKV_CUDA(c, cudaMemset(c->unit_cnt, 0, c->part_units * sizeof(int)));  // a kernel that gave up may have left counts
+    REKV_CUDA(c, cudaMemset(c->unit_cnt, 0, c->cnt_units * sizeof(int)));  // a kernel that gave up may have left counts
     if (st == REKV_ERR_TIMEOUT) REKV_FAIL(c, REKV_ERR_TIMEOUT, "a device-side wait expired");
     REKV_FAIL(c, st, "a kernel reported error %d (an index outside the visible frames?)", st);
   }

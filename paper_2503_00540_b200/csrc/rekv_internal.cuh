@@ -107,6 +107,8 @@ struct rekv_ctx {
   bool timing_valid, merge_timed, retrieve_timed, pull_timed;
   unsigned long long* h_link_bytes; // pinned host mirror of link_bytes, refreshed (asynchronously) after each gather
 
+  char* block;                      // the one device allocation that everything below (and the store) lies in
+
   // scratch (device)
   float* qa;                        // [L][max_questions][Dp] fp32 question vectors
   float* qnorm;                     // [L][max_questions][H_kv] partial sums of squares of the question vector
@@ -115,7 +117,8 @@ struct rekv_ctx {
   float* part_o;                    // split-KV partial outputs
   float* part_ml;                   // split-KV partial (max, sum)
   size_t part_units;                // capacity in (unit) entries of 128 rows
-  int* unit_cnt;                    // [part_units] parts finished per unit (zero between launches)
+  int* unit_cnt;                    // [cnt_units] parts finished per unit (zero between launches)
+  size_t cnt_units;
   int* status;                      // device status word
   unsigned long long* link_bytes;   // device counter: bytes pulled over the host link
   int32_t* idx_own;                 // [L][max_questions][max_topk]: selections of the layer-sequential calls
