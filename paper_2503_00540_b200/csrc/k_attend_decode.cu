@@ -498,7 +498,10 @@ cudaError_t rekv_launch_attend_decode(rekv_ctx* c, const void* q, const QBatch& 
   p.parts = 0;
   // One layer: every unit gets CTAs of its own, since a CTA with parts of two units pays the end of a range twice.
   if (units * 4 <= n_sm && p.steps > 1) {
+    // ... as few as the longest of them allows (24 steps on 18 CTAs are two steps each: twelve CTAs, twelve parts to join)
     p.parts = (int)std::min<long long>(n_sm / units, p.steps);
+    const int longest = (p.steps + p.parts - 1) / p.parts;
+    p.parts = (p.steps + longest - 1) / longest;
     p.per = p.steps;
     grid = units * p.parts;
   } else if (units >= 4 * n_sm || n_sm + units > p.part_slots) {

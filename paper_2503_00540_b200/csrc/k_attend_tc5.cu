@@ -179,7 +179,7 @@ __device__ __forceinline__ Seg decode_seg(const Tc5Params& p, int pos, int end) 
   return s;
 }
 __device__ __forceinline__ int worker_of(const Tc5Params& p, int c) {
-  return (int)(((long long)(c + 1) * p.W - 1) / p.total);
+  return (int)((long long)c * p.W / p.total);
 }
 
 __device__ __forceinline__ float max3(float a, float b, float c) {
@@ -294,8 +294,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
     return false;
   };
 
-  const int range0 = (int)((long long)worker * p.total / p.W);
-  const int range1 = (int)((long long)(worker + 1) * p.total / p.W);
+  const int range0 = (int)(((long long)worker * p.total + p.W - 1) / p.W);
+  const int range1 = (int)(((long long)(worker + 1) * p.total + p.W - 1) / p.W);
   const int Rc = p.ncf * p.Ns;                              // stream rows of the context
   const uint32_t page_half = (uint32_t)p.Nf * 128u;         // one 64-dim half of a head tile in a page
   // the bit of a segment in the run-again mask: the first and the last segment of a range (the only ones that can be
@@ -981,7 +981,7 @@ __global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __g
   const int nch = stream_chunks(p, qi);
   c0 += mp * nch;
   const int W = p.merge_inside;  // (this kernel's copy of the parameters: the attention launch's workers)
-  auto worker_at = [&](int c) { return (int)(((long long)(c + 1) * W - 1) / p.total); };
+  auto worker_at = [&](int c) { return (int)((long long)c * W / p.total); };
   const int w0 = worker_at(c0), n_parts = worker_at(c0 + nch - 1) - w0 + 1;
   const int row = threadIdx.x & 127, grp = threadIdx.x >> 7, quad = blockIdx.z;
   const int rows_q = (p.qb.cu[qi + 1] - p.qb.cu[qi]) * p.G;
@@ -1095,24 +1095,35 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
   if (e != cudaSuccess) return e;
   p.per_lh = 0;
   int blocks = 0, max_ch = 1;
+  bool equal = true;  // every unit has max_ch chunks
   for (int i = 0; i < p.qb.nQ; ++i) {
     const int nb = row_blocks<CG>(p, i), nc = stream_chunks(p, i);
     p.per_lh += nb * nc;
     blocks += nb;
-    max_ch = std::max(max_ch, nc);
+    equal = equal && (nb == 0 || blocks == nb || nc == max_ch);
+    if (nb > 0) max_ch = std::max(max_ch, nc);
   }
   const long long total = (long long)p.per_lh * p.Hkv * p.nl;
   if (total > 0x7fffffff / 2) return cudaErrorInvalidValue;
   p.total = (int)total;
-  // A range has a fixed cost (Q, the first tiles' latency, the result) of a few chunks' time: no shorter ranges than that.
-  constexpr int MIN_CHUNKS = 4;
-  const int units = p.nl * p.Hkv * blocks;
-  p.W = std::min(max_workers<CG>(), std::max(units, p.total / MIN_CHUNKS));
-  // Many workers per unit: whole workers per unit (equal units then start at a range's start), since a range with parts of
-  // two units pays a second Q, result and pipeline start.
-  if (p.W >= 4 * units) p.W -= p.W % units;
-  const int parts = (max_ch - 1) / std::max(1, p.total / p.W) + 2;  // of a unit, at most
-  p.merge_inside = parts <= MAX_PARTS_INSIDE;
+  // How many workers.  Long ranges: all there are, ranges cut where they fall.  A launch of few units (one layer) is a trade
+  // between chunks one after the other (0.8 us each), a range with parts of two units (a second Q, result and pipeline start:
+  // whole workers per unit avoid it), and joining parts.  The merge launch costs such a launch about 2 us, a join inside the
+  // kernel 4 to 6 (fence, counter and the parts' latency, one after the other, at its very end).  28 layers one at a time,
+  // 113 chunks, 4 units (us): 1 worker per unit 3268, 2, 3, 4 joined inside 2096, 1672, 1490, 6, 9, 18 with the merge launch
+  // 1112, 978, 918; 11 chunks, 8 units, 9 layers: 322, 300, 288, 295, 255, 264.
+  const int units = p.nl * p.Hkv * blocks, max_w = max_workers<CG>();
+  p.W = std::min(max_w, p.total);
+  p.merge_inside = (max_ch - 1) / std::max(1, p.total / p.W) + 2 <= MAX_PARTS_INSIDE;   // parts of a unit, at most
+  float best = 0.8f * (float)((p.total + p.W - 1) / p.W) + (units % p.W ? 9.f : 0.f);
+  for (int k = 1; (k == 1 || k < max_ch) && units * k <= max_w; ++k) {  // (two chunks at least in the longer ranges)
+    const float t = 0.8f * (float)((max_ch + k - 1) / k) + (k == 1 ? 0.f : 2.f + 0.05f * (float)k);
+    if (t < best) {
+      best = t;
+      p.W = units * k;
+      p.merge_inside = k == 1 && equal;
+    }
+  }
   if (p.split_rem && !p.merge_inside) {  // (no merge launch between or after the two: fewer workers, whole units each)
     p.W = std::min(p.W, units);
     p.merge_inside = 1;
