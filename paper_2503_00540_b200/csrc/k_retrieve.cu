@@ -203,11 +203,10 @@ struct TopkTable {
   int L, ncf, n_vis_frames;
 };
 constexpr int TK_BINS = 2048, TK_LIST = 64;
-__global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ scores, int nQ, int n_visible,
-                                                   int n_cand, int top_k, int k_eff, int32_t* __restrict__ idx_out,
-                                                   int block, int layer0, TopkTable tt, int copies, int* __restrict__ status) {
-  const int qi = blockIdx.x, l = layer0 + blockIdx.y;
-  const float* s = scores + ((long long)l * nQ + qi) * n_visible;
+// s: the question's scores (global or shared memory), complete for the calling block of 512 threads
+__device__ __forceinline__ void select_topk(const float* s, int qi, int l, int nQ, int n_cand, int top_k, int k_eff,
+                                            int32_t* __restrict__ idx_out, int block, const TopkTable& tt, int copies,
+                                            int* __restrict__ status) {
   int32_t* out = idx_out + ((long long)l * nQ + qi) * top_k;
   __shared__ __align__(16) unsigned hist[TK_BINS];  // (the radix passes use its front)
   __shared__ unsigned s_prefix;
@@ -215,8 +214,6 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
   __shared__ int warp_gt[16], warp_eq[16];
   __shared__ int s_base_gt, s_base_eq;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  rekv_ptx::grid_dep_wait();
-  rekv_ptx::grid_dep_launch();
 
   // entry `at` of the selection, and with it the page of that context slot; `copies` layers get the same selection
   char** row = tt.tbl ? tt.tbl + ((long long)l * nQ + qi) * tt.ncf : nullptr;
@@ -478,6 +475,218 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
   }
 }
 
+__global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ scores, int nQ, int n_visible,
+                                                   int n_cand, int top_k, int k_eff, int32_t* __restrict__ idx_out,
+                                                   int block, int layer0, TopkTable tt, int copies, int* __restrict__ status) {
+  const int qi = blockIdx.x, l = layer0 + blockIdx.y;
+  rekv_ptx::grid_dep_wait();
+  rekv_ptx::grid_dep_launch();
+  select_topk(scores + ((long long)l * nQ + qi) * n_visible, qi, l, nQ, n_cand, top_k, k_eff, idx_out, block, tt, copies, status);
+}
+
+// ---- steps 2-3 of a layer in one launch: question vectors, scores and selection by one cluster per layer.  Three launches
+// pass 4 us from one to the next, whatever little they do; here the CTAs exchange what they have through distributed shared
+// memory: every CTA sums a share of the query rows and sends its partial sum to all, scores a share of the items -- whose
+// first rows have been on their way since the start -- and sends the scores to the CTA that selects for the question.
+// grid = (CTAs per cluster, layers), 512 threads; RB rows of float4 x V4 per lane are in flight per warp.
+constexpr int RK_MAX_Q = 4;          // questions
+constexpr int RK_MAX_ITEMS = 2048;   // items scored (the selection's histogram path)
+struct RetrieveArgs {
+  const uint4* q;
+  const float* reps;
+  float* scores;                     // [L][nQ][n_scored], or null
+  int32_t* idx_out;
+  int* status;
+  TopkTable tt;
+  int Hq, Hkv, max_frames, n_scored, n_cand, top_k, k_eff, block, layer0, CL;
+  QBatch qb;
+};
+template <int V4, int RB>
+__global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(const __grid_constant__ RetrieveArgs p) {
+  using namespace rekv_ptx;
+  extern __shared__ __align__(16) float rk_smem[];
+  const int Dp = p.Hkv * 128, nQ = p.qb.nQ, CL = p.CL;
+  const int cpg = CL / p.Hkv;                                   // CTAs that sum the rows of one KV group
+  float* s_vec = rk_smem;                                       // [nQ][Hkv * cpg][128] partial sums, from all CTAs
+  float* s_q = s_vec + nQ * p.Hkv * cpg * 128;                  // [nQ][Dp] question vectors
+  float* s_score = s_q + nQ * Dp;                               // [n_scored] of the question this CTA selects for
+  __shared__ float s_part[16][128];
+  __shared__ float s_red[RK_MAX_Q][16];
+  __shared__ __align__(8) unsigned long long s_bar[2];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = (int)cluster_ctarank(), l = p.layer0 + blockIdx.y;
+  const uint32_t bar_vec = smem_u32(&s_bar[0]), bar_score = smem_u32(&s_bar[1]);
+  if (tid == 0) {
+    mbar_init(bar_vec, 1);
+    mbar_init(bar_score, 1);
+    fence_barrier_init();
+    mbar_expect_tx(bar_vec, (uint32_t)(nQ * p.Hkv * cpg * 512));
+    if (rank < nQ) mbar_expect_tx(bar_score, (uint32_t)p.n_scored * 4u);
+  }
+  __syncthreads();
+  cluster_sync_all();
+  grid_dep_wait();
+  grid_dep_launch();
+  auto wait = [&](uint32_t bar) {
+    if (mbar_wait_cluster_bounded(bar, 0)) return true;
+    atomicExch(p.status, REKV_ERR_TIMEOUT);
+    return false;
+  };
+
+  // the first items' rows: asked for now, used when the question vectors are there
+  const int per = (p.n_scored + CL - 1) / CL;
+  const int f0 = rank * per, f1 = min(f0 + per, p.n_scored);
+  const float4* reps_l = reinterpret_cast<const float4*>(p.reps + (long long)l * p.max_frames * Dp) + lane;
+  float4 r[RB][V4];
+  auto load_rows = [&](int f) {
+#pragma unroll
+    for (int b = 0; b < RB; ++b) {
+      const float4* row = reps_l + (long long)min(f + b, f1 - 1) * p.block * (Dp / 4);
+#pragma unroll
+      for (int i = 0; i < V4; ++i)
+        if (i < p.Hkv) r[b][i] = __ldg(row + i * 32);
+    }
+  };
+  int f = f0 + warp * RB;
+  if (f < f1) load_rows(f);
+
+  // ---- question vectors: mean over the question's tokens and the G query heads of each KV group
+  const int G = p.Hq / p.Hkv, g = rank / cpg;
+  for (int qi = 0; qi < nQ; ++qi) {
+    const int n0 = p.qb.cu[qi], rows = (p.qb.cu[qi + 1] - n0) * G;
+    if (g < p.Hkv) {
+      const int c = tid & 15, slots = 32 * cpg;
+      const uint4* base = p.q + (((long long)l * p.qb.sumNq + n0) * p.Hq + g * G) * 16 + c;
+      float acc[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+      for (int m0 = (rank - g * cpg) * 32 + (tid >> 4); m0 < rows; m0 += 4 * slots) {
+        uint4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int m = m0 + u * slots, n = m / G;
+          x[u] = m < rows ? __ldg(base + ((long long)n * p.Hq + (m - n * G)) * 16) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const uint32_t v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            acc[2 * i] += __uint_as_float(v[i] << 16);
+            acc[2 * i + 1] += __uint_as_float(v[i] & 0xFFFF0000u);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
+      if (lane < 16) {
+        float4* dst = reinterpret_cast<float4*>(&s_part[warp][c * 8]);
+        dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+      }
+      __syncthreads();
+      // thread t sends columns 4 (t & 31) .. of the CTA's sum to CTA t / 32 (every thread adds its columns up itself)
+      if (warp < CL) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int w = 0; w < 16; ++w) {
+          const float4 x = *reinterpret_cast<const float4*>(&s_part[w][lane * 4]);
+          a.x += x.x;
+          a.y += x.y;
+          a.z += x.z;
+          a.w += x.w;
+        }
+        const uint32_t dst = smem_u32(s_vec + ((qi * p.Hkv * cpg + rank) * 128 + lane * 4));
+        st_async_v4(mapa(dst, (uint32_t)warp), a, mapa(bar_vec, (uint32_t)warp));
+      }
+      __syncthreads();  // (s_part is written again for the next question)
+    }
+  }
+  bool ok = wait(bar_vec);
+  for (int qi = 0; qi < nQ; ++qi) {
+    const float inv = (float)((p.qb.cu[qi + 1] - p.qb.cu[qi]) * G);
+    float sq = 0.f;
+    for (int d = tid; d < Dp; d += 512) {
+      float a = 0.f;
+      for (int k = 0; k < cpg; ++k) a += s_vec[((qi * p.Hkv + (d >> 7)) * cpg + k) * 128 + (d & 127)];
+      a = __fdiv_rn(a, inv);
+      s_q[qi * Dp + d] = a;
+      sq += a * a;
+    }
+    for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) s_red[qi][warp] = sq;
+  }
+  __syncthreads();
+
+  // ---- scores: every lane holds its part of RB rows; dot products and norms by shuffles
+  const float eps = 1e-8f;
+  const float4* s_q4 = reinterpret_cast<const float4*>(s_q) + lane;
+  while (f < f1) {
+    if (p.block > 1) {  // block vector = mean of the block's frame vectors
+      const float fb = (float)p.block;
+#pragma unroll
+      for (int b = 0; b < RB; ++b) {
+        const float4* row = reps_l + (long long)min(f + b, f1 - 1) * p.block * (Dp / 4);
+        for (int j = 1; j < p.block; ++j)
+#pragma unroll
+          for (int i = 0; i < V4; ++i)
+            if (i < p.Hkv) {
+              const float4 x = __ldg(row + (long long)j * (Dp / 4) + i * 32);
+              r[b][i].x += x.x; r[b][i].y += x.y; r[b][i].z += x.z; r[b][i].w += x.w;
+            }
+#pragma unroll
+        for (int i = 0; i < V4; ++i)
+          if (i < p.Hkv) {
+            r[b][i].x = __fdiv_rn(r[b][i].x, fb); r[b][i].y = __fdiv_rn(r[b][i].y, fb);
+            r[b][i].z = __fdiv_rn(r[b][i].z, fb); r[b][i].w = __fdiv_rn(r[b][i].w, fb);
+          }
+      }
+    }
+    float rn[RB];
+#pragma unroll
+    for (int b = 0; b < RB; ++b) {
+      float n = 0.f;
+#pragma unroll
+      for (int i = 0; i < V4; ++i)
+        if (i < p.Hkv) n += r[b][i].x * r[b][i].x + r[b][i].y * r[b][i].y + r[b][i].z * r[b][i].z + r[b][i].w * r[b][i].w;
+      for (int o = 16; o; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+      rn[b] = fmaxf(__fsqrt_rn(n), eps);
+    }
+    for (int qi = 0; qi < nQ; ++qi) {
+      float qn = 0.f;
+#pragma unroll
+      for (int w = 0; w < 16; ++w) qn += s_red[qi][w];
+      qn = fmaxf(__fsqrt_rn(qn), eps);
+      float d[RB];
+#pragma unroll
+      for (int b = 0; b < RB; ++b) d[b] = 0.f;
+#pragma unroll
+      for (int i = 0; i < V4; ++i)
+        if (i < p.Hkv) {
+          const float4 a = s_q4[qi * (Dp / 4) + i * 32];
+#pragma unroll
+          for (int b = 0; b < RB; ++b) d[b] += r[b][i].x * a.x + r[b][i].y * a.y + r[b][i].z * a.z + r[b][i].w * a.w;
+        }
+#pragma unroll
+      for (int b = 0; b < RB; ++b) {
+        for (int o = 16; o; o >>= 1) d[b] += __shfl_xor_sync(0xffffffffu, d[b], o);
+        const float sc = __fdiv_rn(d[b], qn * rn[b]);
+        if (lane == b && f + b < f1 && REKV_CHECK((long long)(f + b + 1) * p.block <= p.max_frames, p.status, 11)) {
+          st_async_f32(mapa(smem_u32(s_score + f + b), (uint32_t)qi), sc, mapa(bar_score, (uint32_t)qi));
+          if (p.scores) p.scores[((long long)l * nQ + qi) * p.n_scored + f + b] = sc;
+        }
+      }
+    }
+    f += 16 * RB;
+    if (f < f1) load_rows(f);
+  }
+  // ---- selection: CTA qi for question qi
+  if (rank < nQ) {
+    ok = wait(bar_score) && ok;
+    if (ok) select_topk(s_score, rank, l, nQ, p.n_cand, p.top_k, p.k_eff, p.idx_out, p.block, p.tt, 1, p.status);
+  }
+}
+
 // ---- external retrieval (Eq. 2 with its temperature): cosine of each question embedding with every frame
 // embedding (or with the mean of a block's frame embeddings), divided by tau.  grid = ceil(items / 8), 256
 // threads, a warp per item: the item's vector is read once into registers (float4 per lane, coalesced) and
@@ -598,6 +807,44 @@ cudaError_t launch_score(const ScoreArgs& a, bool pdl, cudaStream_t st) {
   return a.Dp <= 512 ? launch_score_v4<4>(a, pdl, st) : launch_score_v4<8>(a, pdl, st);
 }
 
+// CTAs per cluster of the one-launch retrieval, or 0 where the three launches are better: every warp has to hold all of its
+// rows at once (one round of loads).  28 layers of 1800 frames, 4 KV heads, one at a time: two rounds on 16 CTAs, 994 us
+// against 919 with the scores spread over 113 blocks; 9 layers of 439 frames, 8 KV heads: 229 against 253; 1 layer of 64
+// frames: 17.1 against 19.2.
+int retrieve_cluster(const QBatch& qb, const StoreView& s, int nl, int n_scored, int block, int top_k, int* rows) {
+  if (qb.nQ > RK_MAX_Q || top_k <= 0 || n_scored <= 0 || (long long)qb.sumNq * s.Hq * 256 > (1 << 20)) return 0;
+  const bool few = nl * 16 <= rekv_sm_count();   // 16 CTAs per layer with up to 16 float4 per lane, or 8 with 8 (two CTAs per SM)
+  const int cl = few ? 16 : 8, most = (few ? 16 : 8) / (s.Hkv <= 4 ? 4 : 8);
+  const long long frames = (long long)n_scored * block;
+  // the fewest rows per warp that do it: short code, which every launch fetches anew
+  for (*rows = 1; *rows < most && frames > (long long)cl * 16 * *rows;) *rows *= 2;
+  return n_scored <= RK_MAX_ITEMS && frames <= (long long)cl * 16 * *rows ? cl : 0;
+}
+template <int V4, int RB>
+cudaError_t launch_retrieve_kernel(const RetrieveArgs& a, int nl, cudaStream_t st) {
+  static PerDeviceOnce attr;
+  cudaError_t e = attr.run([] {
+    cudaError_t e0 = cudaFuncSetAttribute(retrieve_kernel<V4, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+    if (e0 != cudaSuccess) return e0;
+    return cudaFuncSetAttribute(retrieve_kernel<V4, RB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)a.CL, (unsigned)nl);
+  cfg.blockDim = dim3(512);
+  cfg.dynamicSmemBytes = ((size_t)a.qb.nQ * (a.Hkv * (a.CL / a.Hkv) + a.Hkv) * 128 + a.n_scored) * sizeof(float);
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)a.CL;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, retrieve_kernel<V4, RB>, a);
+}
+
 }  // namespace
 
 cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, int top_k, const CtxGeom& geom,
@@ -612,6 +859,46 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
   // b > 1: the complete candidate blocks are scored
   const int b = c->cfg.block_frames;
   const int n_scored = b == 1 ? n_visible : geom.n_items;
+  TopkTable tt = {};
+  if (write_table) {  // HBM-resident cache: the context table comes out of the same launch
+    tt.tbl = c->ctx_tbl;
+    tt.hbm = s.hbm;
+    tt.page_bytes = s.page_bytes;
+    tt.L = s.L;
+    tt.ncf = geom.ncf;
+    tt.n_vis_frames = n_visible;
+  }
+  int rk_rows = 0;
+  if (const int cl = retrieve_cluster(qb, s, nl, n_scored, b, top_k, &rk_rows)) {
+    RetrieveArgs a;
+    a.q = (const uint4*)q;
+    a.reps = s.reps;
+    a.scores = scores == c->scores ? nullptr : scores;
+    a.idx_out = idx_out;
+    a.status = c->status;
+    a.tt = tt;
+    a.Hq = s.Hq;
+    a.Hkv = s.Hkv;
+    a.max_frames = s.max_frames;
+    a.n_scored = n_scored;
+    a.n_cand = geom.n_items;
+    a.top_k = top_k;
+    a.k_eff = geom.k_items;
+    a.block = b;
+    a.layer0 = layer0;
+    a.qb = qb;
+    a.CL = cl;
+    cudaError_t e;
+    if (s.Hkv <= 4)
+      e = rk_rows == 4   ? launch_retrieve_kernel<4, 4>(a, nl, st)
+          : rk_rows == 2 ? launch_retrieve_kernel<4, 2>(a, nl, st)
+                         : launch_retrieve_kernel<4, 1>(a, nl, st);
+    else
+      e = rk_rows == 2 ? launch_retrieve_kernel<8, 2>(a, nl, st) : launch_retrieve_kernel<8, 1>(a, nl, st);
+    if (e != cudaSuccess) return e;
+    c->launches += 1;
+    return cudaGetLastError();
+  }
   if (n_scored > 0) {
     ScoreArgs a = {nl, n_scored, s.reps, c->qa, c->qnorm, qb.nQ, maxQ, s.Dp, s.Hkv, s.max_frames, scores, b, layer0, c->status};
     cudaError_t e;
@@ -624,15 +911,6 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
     c->launches += 1;
   }
   if (top_k > 0) {
-    TopkTable tt = {};
-    if (write_table) {  // HBM-resident cache: the context table comes out of the same launch
-      tt.tbl = c->ctx_tbl;
-      tt.hbm = s.hbm;
-      tt.page_bytes = s.page_bytes;
-      tt.L = s.L;
-      tt.ncf = geom.ncf;
-      tt.n_vis_frames = n_visible;
-    }
     cudaError_t e2 = rekv_launch_pdl(topk_kernel, dim3(qb.nQ, nl), dim3(512), 0, st, scores, qb.nQ, n_scored,
                                      geom.n_items, top_k, geom.k_items, idx_out, b, layer0, tt, 1, c->status);
     if (e2 != cudaSuccess) return e2;

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 from paper_2503_00540_b200 import rekv
+from tests import harness as H
 
 pytestmark = pytest.mark.gpu
 
@@ -64,3 +65,34 @@ def test_selection_with_ties_crowded_steps_and_scores_that_are_not_numbers(patte
         e[10:50] = 0.0
     _select(e, 64)
     _select(e[:1496].contiguous(), 64, b=8)
+
+
+@pytest.mark.parametrize("L,Hkv,T,b,lengths", [
+    (1, 2, 256, 1, [3]), (1, 2, 1025, 1, [3]),        # 16 CTAs per layer, one row per warp at most; beyond four
+    (9, 4, 1024, 1, [5, 1]), (10, 4, 256, 1, [5]),    # ... 9 layers at most; 8 CTAs per layer from the tenth on
+    (10, 4, 257, 1, [5]), (2, 8, 512, 1, [2, 7, 1, 4]), (12, 8, 128, 1, [2]), (12, 8, 129, 1, [2]),
+    (2, 3, 40, 1, [6]), (2, 4, 515, 8, [6]), (1, 1, 7, 1, [1] * 5)])   # idle CTAs, blocks, more than four questions
+def test_one_launch_retrieval_and_the_sizes_around_it(L, Hkv, T, b, lengths):
+    """Question vector, scores and selection in one launch (clusters) and just beyond the sizes it takes: the scores against
+    64-bit sums over the same representatives to 1e-4 (two orders above what fp32 sums lose), the selection exactly what those
+    scores give."""
+    s = H.Shape(L=L, Hq=2 * Hkv, Hkv=Hkv, Nf=2, T=T, W=3, k=8, seed=7, b=b)
+    g = H.build_gpu(s, max_questions=len(lengths), max_q_tokens=sum(lengths))
+    q, cu = H.questions(s, lengths, device="cuda")
+    idx, k_eff, scores = g.retrieve(q, cu, 8, T, want_scores=True)
+    idx2, _, _ = g.retrieve(q, cu, 8, T)
+    g.check_status()
+    assert torch.equal(idx, idx2)
+    n_cand = max(T - 3, 0) // b
+    for l in range(L):
+        reps = g.get_reps(l, T).double()
+        if b > 1:
+            reps = reps[:n_cand * b].reshape(n_cand, b, -1).mean(1)
+        for i in range(len(lengths)):
+            v = q[l, cu[i]:cu[i + 1]].double().reshape(-1, Hkv, 2, 128).mean((0, 2)).reshape(-1)
+            ref = (reps @ v) / (reps.norm(dim=1).clamp_min(1e-8) * v.norm().clamp_min(1e-8))
+            row = scores[l, i].cpu()
+            H.assert_close_rel(row[None], ref.cpu()[None], f"scores of layer {l}, question {i}")
+            items = sorted(sorted(range(n_cand), key=lambda f: (-row[f].item(), f))[:k_eff // b])
+            assert idx[l, i, :k_eff].tolist() == [f * b + j for f in items for j in range(b)]
+    g.close()
