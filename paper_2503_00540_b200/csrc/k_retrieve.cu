@@ -150,7 +150,39 @@ __global__ void __launch_bounds__(256, SCORE_MAX_V4 <= 4 ? 3 : 2)
       }
       n0 = fmaxf(__fsqrt_rn(n0), eps);
       n1 = fmaxf(__fsqrt_rn(n1), eps);
-      for (int qi = 0; qi < qn; ++qi) {
+      // Eight questions' dot products with both items are reduced together: at every step a lane hands over the half of its
+      // sums that the other lane keeps, 16 shuffles for 16 sums instead of 80.
+      int q0 = 0;
+      for (; q0 + 4 <= qn; q0 += 8) {
+        float d[16];  // [item][question]
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          d[j] = d[8 + j] = 0.f;
+          if (q0 + j < qn) {
+#pragma unroll
+            for (int i = 0; i < SCORE_MAX_V4; ++i)
+              if (i < nv4) {
+                const float4 a = s_q[(q0 + j) * (Dp / 4) + i * 32 + lane];
+                d[j] += r0[i].x * a.x + r0[i].y * a.y + r0[i].z * a.z + r0[i].w * a.w;
+                d[8 + j] += r1[i].x * a.x + r1[i].y * a.y + r1[i].z * a.z + r1[i].w * a.w;
+              }
+          }
+        }
+#pragma unroll
+        for (int n = 8, o = 16; n >= 1; n >>= 1, o >>= 1) {
+          const bool up = (lane & o) != 0;
+#pragma unroll
+          for (int i = 0; i < n; ++i) {
+            const float send = up ? d[i] : d[i + n], keep = up ? d[i + n] : d[i];
+            d[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+          }
+        }
+        const float sum = d[0] + __shfl_xor_sync(0xffffffffu, d[0], 1);
+        const int item = lane >> 4, j = q0 + ((lane >> 1) & 7);  // lane bits 4..1 are the sum's index
+        if (!(lane & 1) && j < qn && (item == 0 || two))
+          scores[((long long)l * nQ + qg0 + j) * n_visible + f + item] = __fdiv_rn(sum, s_qn[qg0 + j] * (item ? n1 : n0));
+      }
+      for (int qi = q0; qi < qn; ++qi) {
         float d0 = 0.f, d1 = 0.f;
 #pragma unroll
         for (int i = 0; i < SCORE_MAX_V4; ++i)

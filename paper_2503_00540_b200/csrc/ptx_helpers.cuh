@@ -159,6 +159,22 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+// two fp32 operations in one instruction: (x0, x1) = (x0, x1) * a + b, and (s0, s1) += (x0, x1)
+__device__ __forceinline__ void fma_f32x2(float& x0, float& x1, float a, float b) {
+  asm("{\n\t.reg .b64 x, m, c;\n\t"
+      "mov.b64 x, {%0, %1};\n\tmov.b64 m, {%2, %2};\n\tmov.b64 c, {%3, %3};\n\t"
+      "fma.rn.f32x2 x, x, m, c;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(x0), "+f"(x1)
+      : "f"(a), "f"(b));
+}
+__device__ __forceinline__ void add_f32x2(float& s0, float& s1, float x0, float x1) {
+  asm("{\n\t.reg .b64 s, x;\n\t"
+      "mov.b64 s, {%0, %1};\n\tmov.b64 x, {%2, %3};\n\t"
+      "add.rn.f32x2 s, s, x;\n\tmov.b64 {%0, %1}, s;\n\t}"
+      : "+f"(s0), "+f"(s1)
+      : "f"(x0), "f"(x1));
+}
+
 // two floats -> packed bf16x2 (lo in the low half), round to nearest even
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   uint32_t r;

@@ -71,7 +71,8 @@ def test_selection_with_ties_crowded_steps_and_scores_that_are_not_numbers(patte
     (1, 2, 256, 1, [3]), (1, 2, 1025, 1, [3]),        # 16 CTAs per layer, one row per warp at most; beyond four
     (9, 4, 1024, 1, [5, 1]), (10, 4, 256, 1, [5]),    # ... 9 layers at most; 8 CTAs per layer from the tenth on
     (10, 4, 257, 1, [5]), (2, 8, 512, 1, [2, 7, 1, 4]), (12, 8, 128, 1, [2]), (12, 8, 129, 1, [2]),
-    (2, 3, 40, 1, [6]), (2, 4, 515, 8, [6]), (1, 1, 7, 1, [1] * 5)])   # idle CTAs, blocks, more than four questions
+    (2, 3, 40, 1, [6]), (2, 4, 515, 8, [6]),           # idle CTAs; blocks
+    (1, 1, 7, 1, [1] * 5), (2, 4, 51, 1, [1] * 7), (1, 8, 33, 1, [2] * 11), (2, 2, 50, 1, [1] * 20)])  # eight at a time, and the rest
 def test_one_launch_retrieval_and_the_sizes_around_it(L, Hkv, T, b, lengths):
     """Question vector, scores and selection in one launch (clusters) and just beyond the sizes it takes: the scores against
     64-bit sums over the same representatives to 1e-4 (two orders above what fp32 sums lose), the selection exactly what those
