@@ -36,7 +36,7 @@ WORKLOADS = {
     # decode-shaped question (one token): the HBM-bound end of Eq. 3
     "7b_hbm_decode_1tok": dict(L=28, Hq=28, Hkv=4, D=128, Nf=196, T=1800, W=8, k=64, Nq=1, seed=2503, off_scale=0.5,
                                tail=0, nQ=1, appends_per_step=1),
-    # a short question (10 tokens = 70 rows per KV head): one row tile per unit, run as two half-streams
+    # a short question (10 tokens = 70 rows per KV head): one row tile per unit, single CTAs
     "7b_hbm_short_q10": dict(L=28, Hq=28, Hkv=4, D=128, Nf=196, T=1800, W=8, k=64, Nq=10, seed=2503, off_scale=0.5,
                              tail=0, nQ=1, appends_per_step=1),
     # block retrieval (Eq. 2 paragraph, b = 8): 8 blocks of 8 consecutive frames instead of 64 frames
@@ -155,7 +155,7 @@ class ClockSampler:
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one attention launch from the committed ncu capture
 # (profiles/), scaled to the full workload by the layers processed; None where no capture exists.
-TRAFFIC_NCU = {"7b_hbm_1800f": 848.2e6, "7b_hbm_decode_1tok": 825.0e6}
+TRAFFIC_NCU = {"7b_hbm_1800f": 850.2e6, "7b_hbm_decode_1tok": 826.4e6}
 
 
 def algorithmic_bytes(w, sum_nq=None, nQ=1):
