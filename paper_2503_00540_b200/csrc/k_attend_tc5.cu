@@ -1065,6 +1065,14 @@ __global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __g
   *reinterpret_cast<uint2*>(p.out + ((((long long)l * p.qb.sumNq + p.qb.cu[qi] + n) * p.Hq + g * p.G + j) * 128 + quad * 4)) = packed;
 }
 
+template <int CG>
+cudaError_t prepare_tc5() {  // the kernel's shared-memory limit, once per device
+  static PerDeviceOnce attr;
+  return attr.run([] {
+    return cudaFuncSetAttribute(attend_tc5_kernel<CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+  });
+}
+
 // workers that can run at once: CTA pairs (clusters of two), or CTAs
 template <int CG>
 int max_workers() {
@@ -1086,7 +1094,10 @@ int max_workers() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int m = 0;
-    if (cudaOccupancyMaxActiveClusters(&m, attend_tc5_kernel<2>, &cfg) == cudaSuccess && m > 0) n = std::min(n, m);
+    if (prepare_tc5<CG>() == cudaSuccess && cudaOccupancyMaxActiveClusters(&m, attend_tc5_kernel<CG>, &cfg) == cudaSuccess && m > 0)
+      n = std::min(n, m);
+    else
+      cudaGetLastError();
   }
   if (cacheable) known[dev] = n;
   return n;
@@ -1094,10 +1105,7 @@ int max_workers() {
 
 template <int CG>
 cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
-  static PerDeviceOnce attr;
-  cudaError_t e = attr.run([] {
-    return cudaFuncSetAttribute(attend_tc5_kernel<CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
-  });
+  cudaError_t e = prepare_tc5<CG>();
   if (e != cudaSuccess) return e;
   p.per_lh = 0;
   int blocks = 0, max_ch = 1;
