@@ -49,6 +49,7 @@
 #include <type_traits>
 
 #include "attend_common.cuh"
+#include "attend_plan.h"
 
 using namespace rekv_ptx;
 using namespace rekv_att;
@@ -64,7 +65,7 @@ constexpr uint32_t TMEM_COLS = 512;                    // O [0,128), S/P [128,51
 constexpr uint32_t Q_TILE_BYTES = 128 * 256;           // 128 rows x 128 dims bf16
 constexpr uint32_t RING_BYTES = 160 * 1024;            // K and V tiles in flight
 constexpr float RESCALE_SUM_LIMIT = 1.152921504606846976e18f;  // 2^60
-constexpr int MAX_PARTS_INSIDE = 4;
+constexpr int MAX_PARTS_INSIDE = REKV_MAX_PARTS_INSIDE;
 constexpr uint32_t WAIT_LIMIT = 1u << 22;
 // P is cut (not rounded) to bf16: a value with mantissa m in [1, 2) loses u * 2^-7 / m of itself, u uniform in [0, 1).
 // The mantissa of 2^x is log-uniform, E[1/m] = 1 / (2 ln 2), so the mean loss is 0.7213 * 2^-8 of the value, and scaling
@@ -1120,28 +1121,10 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
   const long long total = (long long)p.per_lh * p.Hkv * p.nl;
   if (total > 0x7fffffff / 2) return cudaErrorInvalidValue;
   p.total = (int)total;
-  // How many workers.  Long ranges: all there are, ranges cut where they fall.  A launch of few units (one layer) is a trade
-  // between chunks one after the other (0.8 us each), a range with parts of two units (a second Q, result and pipeline start:
-  // whole workers per unit avoid it), and joining parts.  The merge launch costs such a launch about 2 us, a join inside the
-  // kernel 4 to 6 (fence, counter and the parts' latency, one after the other, at its very end).  28 layers one at a time,
-  // 113 chunks, 4 units (us): 1 worker per unit 3268, 2, 3, 4 joined inside 2096, 1672, 1490, 6, 9, 18 with the merge launch
-  // 1112, 978, 918; 11 chunks, 8 units, 9 layers: 322, 300, 288, 295, 255, 264.
-  const int units = p.nl * p.Hkv * blocks, max_w = max_workers<CG>();
-  p.W = std::min(max_w, p.total);
-  p.merge_inside = (max_ch - 1) / std::max(1, p.total / p.W) + 2 <= MAX_PARTS_INSIDE;   // parts of a unit, at most
-  float best = 0.8f * (float)((p.total + p.W - 1) / p.W) + (units % p.W ? 9.f : 0.f);
-  for (int k = 1; (k == 1 || k < max_ch) && units * k <= max_w; ++k) {  // (two chunks at least in the longer ranges)
-    const float t = 0.8f * (float)((max_ch + k - 1) / k) + (k == 1 ? 0.f : 2.f + 0.05f * (float)k);
-    if (t < best) {
-      best = t;
-      p.W = units * k;
-      p.merge_inside = k == 1 && equal;
-    }
-  }
-  if (p.split_rem && !p.merge_inside) {  // (no merge launch between or after the two: fewer workers, whole units each)
-    p.W = std::min(p.W, units);
-    p.merge_inside = 1;
-  }
+  // (split launches: no merge launch between or after the two)
+  const AttendPlan plan = rekv_attend_plan(p.total, p.nl * p.Hkv * blocks, max_ch, equal, max_workers<CG>(), !p.split_rem);
+  p.W = plan.workers;
+  p.merge_inside = plan.merge_inside;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(p.W * CG));
   cfg.blockDim = dim3(TC_THREADS);

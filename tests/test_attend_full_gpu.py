@@ -82,6 +82,17 @@ def test_units_cut_in_two_or_three_are_finished_in_the_kernel_with_the_part_over
 
 
 @pytest.mark.parametrize("theta", THETAS)
+@pytest.mark.parametrize("Hkv,nq,ns", [
+    (2, [20, 20, 20], [20, 20, 1200]),             # single CTAs, one layer: units of 1, 1 and 10 chunks
+    (1, [40, 40, 40], [40, 41, 1200]),             # CTA pairs
+    (4, [20, 20, 20, 20], [90, 90, 100, 2400])])   # single CTAs again: 2, 2, 2 and 20 chunks
+def test_one_long_history_among_short_questions_in_a_launch_of_few_units(Hkv, nq, ns, theta):
+    """A launch of one layer whose units differ much in length: workers by the longest unit's chunks would be more than there
+    are chunks."""
+    _run(H.Shape(L=1, Hq=4 * Hkv, Hkv=Hkv, Nf=16, T=12, W=2, k=2, seed=7), nq, ns, theta)
+
+
+@pytest.mark.parametrize("theta", THETAS)
 def test_many_units_take_the_whole_unit_path(theta):
     """Enough (layer, head, question) units that every unit is produced whole by one CTA."""
     s = H.Shape(L=8, Hq=16, Hkv=8, Nf=64, T=12, W=2, k=4)
