@@ -34,8 +34,11 @@ inline AttendPlan rekv_attend_plan(int total, int units, int max_ch, bool equal,
       p.merge_inside = k == 1 && equal;
     }
   }
-  if (!may_merge && !p.merge_inside) {  // fewer workers, whole units each
-    p.workers = std::min(p.workers, units);
+  if (!may_merge && !p.merge_inside) {
+    // Fewer workers: whole units each where all are equally long; where one is much longer than the rest, ranges of more than
+    // a third of it, so that it falls into four at most.
+    const int range = (max_ch - 1) / (REKV_MAX_PARTS_INSIDE - 1) + 1;
+    p.workers = std::min({p.workers, units, total / range});
     p.merge_inside = true;
   }
   return p;

@@ -92,6 +92,15 @@ def test_one_long_history_among_short_questions_in_a_launch_of_few_units(Hkv, nq
     _run(H.Shape(L=1, Hq=4 * Hkv, Hkv=Hkv, Nf=16, T=12, W=2, k=2, seed=7), nq, ns, theta)
 
 
+@pytest.mark.parametrize("nq,ns", [
+    ([32] * 8 + [8] * 5, [32] * 8 + [8] * 4 + [8008]),     # 153 pair chunks, 8 layers x 4 heads: split; units of 7 and 69 chunks
+    ([32] * 8 + [8] * 5, [8008] + [32] * 7 + [8] * 5)])    # the long one among the full pairs
+def test_one_long_history_in_a_batch_of_two_launches(nq, ns):
+    """Full pairs of row tiles in one launch and the remainders in another beside it, neither followed by a merge launch: the
+    long unit has to be cut into no more parts than the kernel joins."""
+    _run(H.Shape(L=8, Hq=28, Hkv=4, Nf=64, T=20, W=4, k=8, seed=2503), nq, ns, 0.0)
+
+
 @pytest.mark.parametrize("theta", THETAS)
 def test_many_units_take_the_whole_unit_path(theta):
     """Enough (layer, head, question) units that every unit is produced whole by one CTA."""

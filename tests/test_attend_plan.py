@@ -1,6 +1,7 @@
 """The rule that deals a launch's chunks to the workers of the tensor-core attention kernel (csrc/attend_plan.h, plain host
 code), walked over batches of equal and very unequal units: no worker is left without a chunk -- it would read the queries of
-a unit beyond the last, and be counted as a part that nobody writes."""
+a unit beyond the last, and be counted as a part that nobody writes -- and no unit whose parts the kernel joins itself has more
+than the four it can join."""
 import ctypes
 import os
 import random
@@ -51,8 +52,9 @@ def _batches(n):
                 x = rng.choice([4, 10, 20, 69, 200])
             chunks += [max(1, context + x)] * rng.randint(1, 4)
         yield chunks, rng.choice([1, 2, 4, 8, 16, 28 * 4, 80 * 8]), rng.choice([1, 2, 66, 74, 132, 148])
-    for chunks, lh in ([1, 1, 10], 1), ([2, 2, 10], 4), ([2, 2, 2, 20], 4):
-        yield chunks, lh, 74
+    for chunks, lh, max_w in ([1, 1, 10], 1, 74), ([2, 2, 10], 4, 74), ([2, 2, 2, 20], 4, 148), ([7] * 4 + [69], 32, 148), \
+            ([15] * 7 + [200], 16, 148):
+        yield chunks, lh, max_w
 
 
 def test_every_worker_has_a_chunk(plan):
@@ -60,3 +62,18 @@ def test_every_worker_has_a_chunk(plan):
         for may_merge in (True, False):
             w, _ = plan(chunks, lh, max_w, may_merge)
             assert 1 <= w <= min(max_w, sum(chunks) * lh), (chunks, lh, max_w, may_merge, w)
+
+
+def test_units_joined_in_the_kernel_have_at_most_four_parts(plan):
+    for chunks, lh, max_w in _batches(4000):
+        total = sum(chunks) * lh
+        for may_merge in (True, False):
+            w, inside = plan(chunks, lh, max_w, may_merge)
+            assert inside or may_merge
+            if not inside:
+                continue
+            at = 0
+            for n in chunks * min(lh, 64):
+                parts = (at + n - 1) * w // total - at * w // total + 1
+                assert parts <= 4, (chunks, lh, max_w, may_merge, w)
+                at += n
