@@ -279,8 +279,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
   if constexpr (CG == 2) cluster_sync_all();  // the peer's barriers are initialised before anything arrives there
   tc_fence_after();
   const uint32_t tmem = *s_tmem_slot;
-  if (!p.second && !(p.early_q && warp >= SM_WARP0)) grid_dep_wait();  // (the softmax warps load the first Q tile before that)
-  grid_dep_launch();
+  // (With early_q the softmax warps load the first Q tile before their wait.)  No warp releases the next launch before its own
+  // wait: one thread's release counts for its CTA, and the next launch may take what this one's predecessors wrote as complete.
+  const bool waits_later = p.early_q && warp >= SM_WARP0;
+  if (!waits_later) {
+    if (!p.second) grid_dep_wait();
+    grid_dep_launch();
+  }
 
   const uint32_t wait_limit = p.wait_limit ? p.wait_limit : WAIT_LIMIT;
   auto try_wait = [&](int b, uint32_t parity) -> bool {
@@ -337,7 +342,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
   if (warp >= SM_WARP0) {  // the first segment's Q
     load_q(decode_seg<CG>(p, range0, range1), 0, (warp - SM_WARP0) * 16, std::integral_constant<int, 8>{});
     if (lane == 0) mbar_arrive(bar(B_QFULL));
-    if (p.early_q) grid_dep_wait();
+    if (waits_later) {
+      grid_dep_wait();
+      grid_dep_launch();
+    }
   }
 
   // The roles run the same range loop with the role as a compile-time constant, so that each side of the register

@@ -142,8 +142,9 @@ struct rekv_ctx {
   int test_skip_copy_entry;
   bool q_early_ok = false;          // the attention launch that follows is chained to the library's own selection kernels (which only read Q)
 
-  // An attention launch on ctx_stream has read the whole context table since it was last written (it waited for the table's
-  // writer): later launches on that stream may read the table and an HBM-resident cache's pages before their own wait.
+  // An attention launch on ctx_stream follows the table's writer, and released its successor only after its own wait for that
+  // writer (every kernel here releases after its wait): later launches on that stream may read the table and an HBM-resident
+  // cache's pages before their own wait.
   bool ctx_settled = false;
   cudaStream_t ctx_stream = nullptr;
 

@@ -193,3 +193,52 @@ def test_a_layer_context_built_under_another_geometry_is_refused():
     assert torch.equal(out0, out0b)
     H.assert_attention(out0b[None], ref["out"][0:1], "layer 0 gathered again")
     g.close()
+
+
+@pytest.mark.parametrize("k", [4, 12, 28])
+@pytest.mark.parametrize("full", [False, True])
+def test_a_token_directly_behind_the_question_of_its_layer(k, full):
+    """question_layer and at once a one-token step over the context it builds, nothing between them, another question every
+    time: contexts of one, two and four chunks, whose attention is one launch, so that the decode launch -- which asks for its
+    first frames before its dependency wait -- follows it directly.  The same bits as with a synchronisation between the two,
+    and those against the oracle."""
+    s = H.Shape(L=3, Hq=8, Hkv=2, Nf=16, T=64, W=4, k=k, seed=540)
+    extra = dict(max_self_tokens=8, rope_theta=1e6) if full else {}
+    g = H.build_gpu(s, max_questions=1, max_q_tokens=16, **extra)
+    o = H.build_oracle(s)
+    n = 6
+    qs = [H.questions(s, [16], device="cuda", first_id=10 * i)[0] for i in range(n)]
+    toks = [H.questions(s, [1], device="cuda", first_id=10 * i + 5)[0] for i in range(n)]
+    ks, vs, cus = H.self_kv(s, [8], device="cuda")
+
+    def run(sync):
+        out, outd = [torch.zeros_like(q) for q in qs], [torch.zeros_like(t) for t in toks]
+        idx = torch.zeros((n, s.L, 1, k), dtype=torch.int32, device="cuda")
+        torch.cuda.synchronize()
+        for i in range(n):
+            for l in range(s.L):
+                g.question_layer(l, qs[i][l], [0, 16], k, s.T, out=out[i][l], idx=idx[i, l])
+                if sync:
+                    torch.cuda.synchronize()
+                if full:
+                    g.attend_full_layer(l, toks[i][l], ks[l], vs[l], [0, 1], cus, out=outd[i][l])
+                else:
+                    g.attend_layer(l, toks[i][l], [0, 1], out=outd[i][l])
+                if sync:
+                    torch.cuda.synchronize()
+        g.check_status()
+        return out, outd, idx
+
+    out0, outd0, idx0 = run(True)
+    out1, outd1, idx1 = run(False)
+    assert torch.equal(idx0, idx1)
+    for i in range(n):
+        assert torch.equal(out0[i], out1[i]) and torch.equal(outd0[i], outd1[i]), f"question {i}"
+        ref = o.question(qs[i].cpu(), k, s.T)
+        for l in range(s.L):
+            if torch.equal(idx0[i, l, 0].cpu(), ref["idx"][l]):
+                H.assert_attention(out0[i][l:l + 1], ref["out"][l:l + 1], f"question {i} layer {l}")
+                if not full:
+                    refd, _ = o.attend(toks[i].cpu(), ref["k_ctx"], ref["v_ctx"])
+                    H.assert_attention(outd0[i][l:l + 1], refd[l:l + 1], f"token {i} layer {l}")
+    g.close()
