@@ -308,6 +308,13 @@ int rekv_check_status(rekv_ctx* ctx, void* stream);
  * Host-side only; returns REKV_OK. */
 int rekv_test_set_wait_limit(rekv_ctx* ctx, unsigned iterations, int skip_copy_entry);
 
+/* TEST-ONLY.  What the retrieval of small tables does from now on (0 = as always):
+ *   REKV_TEST_RETRIEVE_NO_CLUSTER  as on a device, or a partition of one, where no thread-block cluster of the size that the
+ *                                  one-launch retrieval takes can be resident: three launches
+ * Host-side only; returns REKV_OK. */
+enum { REKV_TEST_RETRIEVE_NO_CLUSTER = 1 };
+int rekv_test_set_retrieve(rekv_ctx* ctx, int mode);
+
 /* Message of the last failure on this context (or of the last failed rekv_create when ctx is NULL).
  * The pointer stays valid until the next failing call. */
 const char* rekv_last_error(rekv_ctx* ctx);

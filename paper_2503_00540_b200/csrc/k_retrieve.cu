@@ -522,6 +522,7 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
 // first rows have been on their way since the start -- and sends the scores to the CTA that selects for the question.
 // grid = (CTAs per cluster, layers), 512 threads; RB rows of float4 x V4 per lane are in flight per warp.
 constexpr int RK_MAX_Q = 4;          // questions
+constexpr int RK_MAX_CL = 16;        // CTAs per cluster
 constexpr int RK_MAX_ITEMS = 2048;   // items scored (the selection's histogram path)
 struct RetrieveArgs {
   const uint4* q;
@@ -852,8 +853,11 @@ int retrieve_cluster(const QBatch& qb, const StoreView& s, int nl, int n_scored,
   for (*rows = 1; *rows < most && frames > (long long)cl * 16 * *rows;) *rows *= 2;
   return n_scored <= RK_MAX_ITEMS && frames <= (long long)cl * 16 * *rows ? cl : 0;
 }
+// *launched: false where no cluster of that size can be resident -- 16 CTAs are beyond the portable size, and a partition of the
+// device may have no 16 SMs of one GPC -- and nothing was launched.
 template <int V4, int RB>
-cudaError_t launch_retrieve_kernel(const RetrieveArgs& a, int nl, cudaStream_t st) {
+cudaError_t launch_retrieve_kernel(const RetrieveArgs& a, int nl, bool no_cluster, cudaStream_t st, bool* launched) {
+  *launched = false;
   static PerDeviceOnce attr;
   cudaError_t e = attr.run([] {
     cudaError_t e0 = cudaFuncSetAttribute(retrieve_kernel<V4, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
@@ -874,6 +878,18 @@ cudaError_t launch_retrieve_kernel(const RetrieveArgs& a, int nl, cudaStream_t s
   at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
+  // clusters that can be resident, asked once per device and size: 0 unknown, 1 some, 2 none
+  static char known[REKV_MAX_DEVICES][RK_MAX_CL + 1] = {};
+  int dev = 0, n = 0;
+  const bool cacheable = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < REKV_MAX_DEVICES;
+  char state = cacheable ? known[dev][a.CL] : 0;
+  if (!state) {
+    state = cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<V4, RB>, &cfg) == cudaSuccess && n > 0 ? 1 : 2;
+    if (state == 2) cudaGetLastError();
+    if (cacheable) known[dev][a.CL] = state;
+  }
+  if (state == 2 || no_cluster) return cudaSuccess;
+  *launched = true;
   return cudaLaunchKernelEx(&cfg, retrieve_kernel<V4, RB>, a);
 }
 
@@ -921,15 +937,20 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
     a.qb = qb;
     a.CL = cl;
     cudaError_t e;
+    const bool off = (c->test_retrieve & REKV_TEST_RETRIEVE_NO_CLUSTER) != 0;
+    bool launched = false;
     if (s.Hkv <= 4)
-      e = rk_rows == 4   ? launch_retrieve_kernel<4, 4>(a, nl, st)
-          : rk_rows == 2 ? launch_retrieve_kernel<4, 2>(a, nl, st)
-                         : launch_retrieve_kernel<4, 1>(a, nl, st);
+      e = rk_rows == 4   ? launch_retrieve_kernel<4, 4>(a, nl, off, st, &launched)
+          : rk_rows == 2 ? launch_retrieve_kernel<4, 2>(a, nl, off, st, &launched)
+                         : launch_retrieve_kernel<4, 1>(a, nl, off, st, &launched);
     else
-      e = rk_rows == 2 ? launch_retrieve_kernel<8, 2>(a, nl, st) : launch_retrieve_kernel<8, 1>(a, nl, st);
+      e = rk_rows == 2 ? launch_retrieve_kernel<8, 2>(a, nl, off, st, &launched)
+                       : launch_retrieve_kernel<8, 1>(a, nl, off, st, &launched);
     if (e != cudaSuccess) return e;
-    c->launches += 1;
-    return cudaGetLastError();
+    if (launched) {
+      c->launches += 1;
+      return cudaGetLastError();
+    }
   }
   if (n_scored > 0) {
     ScoreArgs a = {nl, n_scored, s.reps, c->qa, c->qnorm, qb.nQ, maxQ, s.Dp, s.Hkv, s.max_frames, scores, b, layer0, c->status};

@@ -809,6 +809,12 @@ int rekv_test_set_wait_limit(rekv_ctx* c, unsigned iterations, int skip_copy_ent
   return REKV_OK;
 }
 
+int rekv_test_set_retrieve(rekv_ctx* c, int mode) {
+  if (!c) return REKV_ERR_ARG;
+  c->test_retrieve = mode;
+  return REKV_OK;
+}
+
 int rekv_check_status(rekv_ctx* c, void* stream) {
   if (!c) return REKV_ERR_ARG;
   DeviceGuard guard(c->device);

@@ -140,6 +140,7 @@ struct rekv_ctx {
   // test-only knobs of the bounded device-side waits (rekv_test_set_wait_limit); 0 / -1 = off
   unsigned test_wait_limit;
   int test_skip_copy_entry;
+  int test_retrieve = 0;            // REKV_TEST_RETRIEVE_* (rekv_test_set_retrieve)
   bool q_early_ok = false;          // the attention launch that follows is chained to the library's own selection kernels (which only read Q)
 
   // An attention launch on ctx_stream follows the table's writer, and released its successor only after its own wait for that

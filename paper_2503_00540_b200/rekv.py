@@ -19,6 +19,7 @@ OK, ERR_ARG, ERR_FULL, ERR_EMPTY, ERR_ALLOC, ERR_CUDA, ERR_TIMEOUT, ERR_STATE = 
 FLAG_TIMING = 1 << 2
 FLAG_HOST_FP8 = 1 << 3
 FLAG_ROPE_STATIC = 1 << 4
+TEST_RETRIEVE_NO_CLUSTER = 1
 
 
 class RekvError(RuntimeError):
@@ -49,7 +50,7 @@ EXPORTS = ("rekv_create", "rekv_destroy", "rekv_append_frame", "rekv_retrieve", 
            "rekv_question_layer_full", "rekv_attend_full_layer",
            "rekv_set_frame_embedding", "rekv_retrieve_external", "rekv_question",
            "rekv_save", "rekv_load", "rekv_set_timing", "rekv_geometry",
-           "rekv_test_set_wait_limit")
+           "rekv_test_set_wait_limit", "rekv_test_set_retrieve")
 
 _lib = None
 
@@ -85,6 +86,7 @@ def lib() -> ctypes.CDLL:
         L.rekv_check_status.argtypes = [vp, vp]
         L.rekv_set_timing.argtypes = [vp, i32]
         L.rekv_test_set_wait_limit.argtypes = [vp, ctypes.c_uint, i32]
+        L.rekv_test_set_retrieve.argtypes = [vp, i32]
         L.rekv_geometry.argtypes = [vp, i32, i32, ip, ip, ip]
         L.rekv_last_error.argtypes = [vp]
         L.rekv_last_error.restype = ctypes.c_char_p
@@ -359,6 +361,10 @@ class ReKV:
     def test_set_wait_limit(self, iterations: int, skip_copy_entry: int = -1) -> None:
         """Test-only: shortens the kernels' bounded waits and makes one tile copy go missing (rekv_test_set_wait_limit)."""
         self._check(lib().rekv_test_set_wait_limit(self._h, iterations, skip_copy_entry))
+
+    def test_set_retrieve(self, mode: int) -> None:
+        """Test-only: what the retrieval of small tables does from now on (rekv_test_set_retrieve)."""
+        self._check(lib().rekv_test_set_retrieve(self._h, mode))
 
     def launch_count(self) -> int:
         return int(lib().rekv_launch_count(self._h))

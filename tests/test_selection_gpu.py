@@ -97,3 +97,29 @@ def test_one_launch_retrieval_and_the_sizes_around_it(L, Hkv, T, b, lengths):
             items = sorted(sorted(range(n_cand), key=lambda f: (-row[f].item(), f))[:k_eff // b])
             assert idx[l, i, :k_eff].tolist() == [f * b + j for f in items for j in range(b)]
     g.close()
+
+
+@pytest.mark.parametrize("L,T,lengths", [(1, 64, [16]), (12, 60, [5, 9])])  # clusters of 16 and of 8 CTAs
+def test_retrieval_without_room_for_a_cluster_takes_the_three_launches(L, T, lengths):
+    s = H.Shape(L=L, Hq=8, Hkv=2, Nf=2, T=T, W=3, k=8, seed=7)
+    g = H.build_gpu(s, max_questions=len(lengths), max_q_tokens=sum(lengths))
+    q, cu = H.questions(s, lengths, device="cuda")
+
+    def retrieve():
+        n = g.launch_count()
+        idx, _, scores = g.retrieve(q, cu, 8, T, want_scores=True)
+        return idx, scores, g.launch_count() - n
+
+    idx1, scores1, n1 = retrieve()
+    g.test_set_retrieve(rekv.TEST_RETRIEVE_NO_CLUSTER)
+    idx3, scores3, n3 = retrieve()
+    out3 = g.question(q, cu, 8, T)
+    g.check_status()
+    assert (n1, n3) == (1, 3)
+    for l in range(L):
+        H.assert_close_rel(scores3[l], scores1[l], f"scores of layer {l}")
+    assert torch.equal(idx3, idx1)
+    g.test_set_retrieve(0)
+    assert torch.equal(g.question(q, cu, 8, T), out3)
+    g.check_status()
+    g.close()
