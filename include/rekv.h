@@ -300,7 +300,7 @@ int rekv_check_status(rekv_ctx* ctx, void* stream);
 /* TEST-ONLY.  The kernels' device-side waits (on a copy, a matrix product, another warp) are bounded: when a
  * wait runs out of iterations the kernel writes REKV_ERR_TIMEOUT to the status word, releases what it holds
  * and returns, and the context stays usable.  This call makes that path reachable without a fault:
- *   iterations       limit of every bounded wait of the attention kernels launched from now on (0 = the
+ *   iterations       limit of every bounded wait of the kernels launched from now on (0 = the
  *                    built-in limit, about a third of a second)
  *   skip_copy_entry  >= 0: the copy producer of the attention kernel's first CTA leaves out the K/V tile copy
  *                    with this sequence number, so that the wait for it expires with nothing in flight; -1 = off
@@ -311,8 +311,11 @@ int rekv_test_set_wait_limit(rekv_ctx* ctx, unsigned iterations, int skip_copy_e
 /* TEST-ONLY.  What the retrieval of small tables does from now on (0 = as always):
  *   REKV_TEST_RETRIEVE_NO_CLUSTER  as on a device, or a partition of one, where no thread-block cluster of the size that the
  *                                  one-launch retrieval takes can be resident: three launches
+ *   REKV_TEST_RETRIEVE_SKIP_SUM, REKV_TEST_RETRIEVE_SKIP_SCORE  the one launch leaves out the first layer's first CTA's part of
+ *                                  the question vectors, or its first score: the wait for it runs out (give it a short limit
+ *                                  with rekv_test_set_wait_limit first)
  * Host-side only; returns REKV_OK. */
-enum { REKV_TEST_RETRIEVE_NO_CLUSTER = 1 };
+enum { REKV_TEST_RETRIEVE_NO_CLUSTER = 1, REKV_TEST_RETRIEVE_SKIP_SUM = 2, REKV_TEST_RETRIEVE_SKIP_SCORE = 4 };
 int rekv_test_set_retrieve(rekv_ctx* ctx, int mode);
 
 /* Message of the last failure on this context (or of the last failed rekv_create when ctx is NULL).

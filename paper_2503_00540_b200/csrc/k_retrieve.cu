@@ -532,8 +532,18 @@ struct RetrieveArgs {
   int* status;
   TopkTable tt;
   int Hq, Hkv, max_frames, n_scored, n_cand, top_k, k_eff, block, layer0, CL;
+  unsigned wait_limit;               // test-only knobs (0 = off), see rekv_test_set_wait_limit, rekv_test_set_retrieve
+  int test;
   QBatch qb;
 };
+// A wait ran out (the status word says so).  No selection, but a list and a table that are safe to follow: what comes next in the
+// stream reads them before anyone has read the status.  (Out of line: the launch fetches its code anew every time.)
+__device__ __noinline__ void retrieve_failed(const RetrieveArgs& p, int qi, int l) {
+  const long long row = (long long)l * p.qb.nQ + qi;
+  for (int j = threadIdx.x; j < p.top_k; j += blockDim.x) p.idx_out[row * p.top_k + j] = -1;
+  if (p.tt.tbl)
+    for (int j = threadIdx.x; j < p.tt.ncf; j += blockDim.x) p.tt.tbl[row * p.tt.ncf + j] = p.tt.hbm + (long long)l * p.tt.page_bytes;  // frame 0
+}
 template <int V4, int RB>
 __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(const __grid_constant__ RetrieveArgs p) {
   using namespace rekv_ptx;
@@ -561,7 +571,7 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
   grid_dep_wait();
   grid_dep_launch();
   auto wait = [&](uint32_t bar) {
-    if (mbar_wait_cluster_bounded(bar, 0)) return true;
+    if (mbar_wait_cluster_bounded(bar, 0, p.wait_limit ? p.wait_limit : 1u << 22)) return true;
     atomicExch(p.status, REKV_ERR_TIMEOUT);
     return false;
   };
@@ -630,7 +640,8 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
           a.w += x.w;
         }
         const uint32_t dst = smem_u32(s_vec + ((qi * p.Hkv * cpg + rank) * 128 + lane * 4));
-        st_async_v4(mapa(dst, (uint32_t)warp), a, mapa(bar_vec, (uint32_t)warp));
+        if (!((p.test & REKV_TEST_RETRIEVE_SKIP_SUM) && rank == 0 && blockIdx.y == 0))
+          st_async_v4(mapa(dst, (uint32_t)warp), a, mapa(bar_vec, (uint32_t)warp));
       }
       __syncthreads();  // (s_part is written again for the next question)
     }
@@ -705,7 +716,8 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
         for (int o = 16; o; o >>= 1) d[b] += __shfl_xor_sync(0xffffffffu, d[b], o);
         const float sc = __fdiv_rn(d[b], qn * rn[b]);
         if (lane == b && f + b < f1 && REKV_CHECK((long long)(f + b + 1) * p.block <= p.max_frames, p.status, 11)) {
-          st_async_f32(mapa(smem_u32(s_score + f + b), (uint32_t)qi), sc, mapa(bar_score, (uint32_t)qi));
+          if (!((p.test & REKV_TEST_RETRIEVE_SKIP_SCORE) && f + b == 0 && blockIdx.y == 0))
+            st_async_f32(mapa(smem_u32(s_score + f + b), (uint32_t)qi), sc, mapa(bar_score, (uint32_t)qi));
           if (p.scores) p.scores[((long long)l * nQ + qi) * p.n_scored + f + b] = sc;
         }
       }
@@ -716,8 +728,15 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
   // ---- selection: CTA qi for question qi
   if (rank < nQ) {
     ok = wait(bar_score) && ok;
-    if (ok) select_topk(s_score, rank, l, nQ, p.n_cand, p.top_k, p.k_eff, p.idx_out, p.block, p.tt, 1, p.status);
+    ok = __syncthreads_and(ok);
+    if (ok) {
+      select_topk(s_score, rank, l, nQ, p.n_cand, p.top_k, p.k_eff, p.idx_out, p.block, p.tt, 1, p.status);
+      return;
+    }
+    retrieve_failed(p, rank, l);
   }
+  // a thread whose wait ran out stays until the others are done or here too: they may still send into this CTA's shared memory
+  if (!ok) cluster_sync_threads();
 }
 
 // ---- external retrieval (Eq. 2 with its temperature): cosine of each question embedding with every frame
@@ -936,6 +955,8 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
     a.layer0 = layer0;
     a.qb = qb;
     a.CL = cl;
+    a.wait_limit = c->test_wait_limit;
+    a.test = c->test_retrieve;
     cudaError_t e;
     const bool off = (c->test_retrieve & REKV_TEST_RETRIEVE_NO_CLUSTER) != 0;
     bool launched = false;

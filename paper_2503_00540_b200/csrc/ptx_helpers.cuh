@@ -65,6 +65,9 @@ __device__ __forceinline__ void cluster_sync_all() {  // every thread of every C
 __device__ __forceinline__ void cluster_sync_relaxed() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
+__device__ __forceinline__ void cluster_sync_threads() {  // any threads: waits for those of the cluster that have not exited
+  asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+}
 __device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 __device__ __forceinline__ uint32_t mapa(uint32_t smem_addr, uint32_t rank) {  // the same offset in another CTA
   uint32_t r;

@@ -19,7 +19,7 @@ OK, ERR_ARG, ERR_FULL, ERR_EMPTY, ERR_ALLOC, ERR_CUDA, ERR_TIMEOUT, ERR_STATE = 
 FLAG_TIMING = 1 << 2
 FLAG_HOST_FP8 = 1 << 3
 FLAG_ROPE_STATIC = 1 << 4
-TEST_RETRIEVE_NO_CLUSTER = 1
+TEST_RETRIEVE_NO_CLUSTER, TEST_RETRIEVE_SKIP_SUM, TEST_RETRIEVE_SKIP_SCORE = 1, 2, 4
 
 
 class RekvError(RuntimeError):

@@ -64,3 +64,39 @@ def test_decode_kernel_gives_up_when_a_frame_never_arrives():
     """One query token (4 rows per KV head): the load-bound decode kernel."""
     s = H.Shape(L=4, Hq=8, Hkv=2, Nf=48, T=60, W=4, k=36, seed=7)
     _expire_then_recover(s, [1], 0)
+
+
+@pytest.mark.parametrize("L,lengths", [(1, [16]), (12, [5, 3, 4])])  # clusters of 16 and of 8 CTAs
+@pytest.mark.parametrize("mode", [rekv.TEST_RETRIEVE_SKIP_SUM, rekv.TEST_RETRIEVE_SKIP_SCORE])
+def test_one_launch_retrieval_gives_up_when_a_part_never_arrives(L, lengths, mode):
+    """A CTA of the first layer's cluster leaves out its part of the question vectors (every CTA of the cluster waits for it)
+    or a score (the CTA that selects waits): the launch returns, the layer's list is empty and its context table safe to
+    follow, and the next question is answered as before."""
+    s = H.Shape(L=L, Hq=8, Hkv=2, Nf=16, T=60, W=4, k=8, seed=7)
+    g = H.build_gpu(s, max_questions=len(lengths), max_q_tokens=sum(lengths))
+    q, cu = H.questions(s, lengths, device="cuda")
+    idx0, _, _ = g.retrieve(q, cu, s.k, s.T)
+    out0 = g.question(q, cu, s.k, s.T)
+    g.check_status()
+    g.test_set_wait_limit(20000)
+    g.test_set_retrieve(mode)
+    idx = torch.full_like(idx0, -7)
+    for l in range(L):
+        g.question_layer(l, q[l], cu, s.k, s.T, idx=idx[l])
+    with pytest.raises(rekv.RekvError) as e:
+        g.check_status()
+    assert e.value.code == rekv.ERR_TIMEOUT
+    idx_r, _, _ = g.retrieve(q, cu, s.k, s.T)
+    g.question(q, cu, s.k, s.T)
+    with pytest.raises(rekv.RekvError) as e:
+        g.check_status()
+    assert e.value.code == rekv.ERR_TIMEOUT
+    g.check_status()
+    assert (idx_r[0, 0] == -1).all() and torch.equal(idx_r[1:], idx0[1:])
+    assert (idx[:, 0] == -1).all()
+    g.test_set_wait_limit(0)
+    g.test_set_retrieve(0)
+    assert torch.equal(g.retrieve(q, cu, s.k, s.T)[0], idx0)
+    assert torch.equal(g.question(q, cu, s.k, s.T), out0)
+    g.check_status()
+    g.close()
