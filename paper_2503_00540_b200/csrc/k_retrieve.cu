@@ -5,6 +5,22 @@
 
 namespace {
 
+// The arithmetic of the scores, for the three launches and the one-launch form alike: a score has the same bits whichever
+// of them a call takes (a layer at a time or all layers, and rekv_score_frames_static), and so has the selection.  Fixed
+// orders, and no product left to the compiler to contract:
+//   question vector  64 partial sums, row r of the question in sum r mod 64, joined pairwise as a binary tree
+//   its square norm  32-dim blocks by butterflies, four of them per KV group, groups in order
+//   dot, row norm    per lane float4 by float4, then a butterfly over the lanes
+constexpr int Q_SLOTS = 64;
+__device__ __forceinline__ float add_dot4(float acc, const float4& a, const float4& b) {
+  return __fadd_rn(acc, __fmaf_rn(a.w, b.w, __fmaf_rn(a.z, b.z, __fmaf_rn(a.y, b.y, __fmul_rn(a.x, b.x)))));
+}
+__device__ __forceinline__ float square_norm_of_warp(float a) {  // of the warp's 32 dims
+  float sq = __fmul_rn(a, a);
+  for (int o = 16; o; o >>= 1) sq = __fadd_rn(sq, __shfl_xor_sync(0xffffffffu, sq, o));
+  return sq;
+}
+
 // ---- question vector: mean over the question's tokens and over the G query heads of each KV group
 // grid = (nQ, layers, H_kv), layer = layer0 + blockIdx.y; 1024 threads = 64 row slots x 16 lanes of 16 bytes, four rows
 // per thread in flight: a question of 36 tokens at G = 7 is one round of loads deep (latency is all this kernel has).
@@ -52,17 +68,15 @@ __global__ void __launch_bounds__(QM_THREADS) qmean_kernel(const uint4* __restri
     dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
   }
   __syncthreads();
-  const int d = threadIdx.x & 127, k = threadIdx.x >> 7;  // fixed order
+  const int d = threadIdx.x & 127, k = threadIdx.x >> 7;
   part2[k][d] = (part[4 * k][d] + part[4 * k + 1][d]) + (part[4 * k + 2][d] + part[4 * k + 3][d]);
   __syncthreads();
   if (threadIdx.x < 128) {
-    float a = 0.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) a += part2[i][d];
+    float a = ((part2[0][d] + part2[1][d]) + (part2[2][d] + part2[3][d])) +
+              ((part2[4][d] + part2[5][d]) + (part2[6][d] + part2[7][d]));
     a = __fdiv_rn(a, (float)rows);
     qa[((long long)l * maxQ + qi) * (Hkv * 128) + g * 128 + d] = a;
-    float sq = a * a;
-    for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    const float sq = square_norm_of_warp(a);
     if (lane == 0) red[threadIdx.x >> 5] = sq;
   }
   __syncthreads();
@@ -141,8 +155,8 @@ __global__ void __launch_bounds__(256, SCORE_MAX_V4 <= 4 ? 3 : 2)
 #pragma unroll
       for (int i = 0; i < SCORE_MAX_V4; ++i)
         if (i < nv4) {
-          n0 += r0[i].x * r0[i].x + r0[i].y * r0[i].y + r0[i].z * r0[i].z + r0[i].w * r0[i].w;
-          n1 += r1[i].x * r1[i].x + r1[i].y * r1[i].y + r1[i].z * r1[i].z + r1[i].w * r1[i].w;
+          n0 = add_dot4(n0, r0[i], r0[i]);
+          n1 = add_dot4(n1, r1[i], r1[i]);
         }
       for (int o = 16; o; o >>= 1) {
         n0 += __shfl_xor_sync(0xffffffffu, n0, o);
@@ -163,8 +177,8 @@ __global__ void __launch_bounds__(256, SCORE_MAX_V4 <= 4 ? 3 : 2)
             for (int i = 0; i < SCORE_MAX_V4; ++i)
               if (i < nv4) {
                 const float4 a = s_q[(q0 + j) * (Dp / 4) + i * 32 + lane];
-                d[j] += r0[i].x * a.x + r0[i].y * a.y + r0[i].z * a.z + r0[i].w * a.w;
-                d[8 + j] += r1[i].x * a.x + r1[i].y * a.y + r1[i].z * a.z + r1[i].w * a.w;
+                d[j] = add_dot4(d[j], r0[i], a);
+                d[8 + j] = add_dot4(d[8 + j], r1[i], a);
               }
           }
         }
@@ -188,8 +202,8 @@ __global__ void __launch_bounds__(256, SCORE_MAX_V4 <= 4 ? 3 : 2)
         for (int i = 0; i < SCORE_MAX_V4; ++i)
           if (i < nv4) {
             const float4 a = s_q[qi * (Dp / 4) + i * 32 + lane];
-            d0 += r0[i].x * a.x + r0[i].y * a.y + r0[i].z * a.z + r0[i].w * a.w;
-            d1 += r1[i].x * a.x + r1[i].y * a.y + r1[i].z * a.z + r1[i].w * a.w;
+            d0 = add_dot4(d0, r0[i], a);
+            d1 = add_dot4(d1, r1[i], a);
           }
         for (int o = 16; o; o >>= 1) {
           d0 += __shfl_xor_sync(0xffffffffu, d0, o);
@@ -519,8 +533,9 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
 // ---- steps 2-3 of a layer in one launch: question vectors, scores and selection by one cluster per layer.  Three launches
 // pass 4 us from one to the next, whatever little they do; here the CTAs exchange what they have through distributed shared
 // memory: every CTA sums a share of the query rows and sends its partial sum to all, scores a share of the items -- whose
-// first rows have been on their way since the start -- and sends the scores to the CTA that selects for the question.
-// grid = (CTAs per cluster, layers), 512 threads; RB rows of float4 x V4 per lane are in flight per warp.
+// first rows are on their way while the sums are exchanged -- and sends the scores to the CTA that selects for the question.
+// grid = (CTAs per cluster, layers), 512 threads; RB rows of float4 x V4 per lane are in flight per warp; CPG CTAs (1, 2, 4, 8) sum
+// the rows of one KV group.
 constexpr int RK_MAX_Q = 4;          // questions
 constexpr int RK_MAX_CL = 16;        // CTAs per cluster
 constexpr int RK_MAX_ITEMS = 2048;   // items scored (the selection's histogram path)
@@ -544,17 +559,16 @@ __device__ __noinline__ void retrieve_failed(const RetrieveArgs& p, int qi, int 
   if (p.tt.tbl)
     for (int j = threadIdx.x; j < p.tt.ncf; j += blockDim.x) p.tt.tbl[row * p.tt.ncf + j] = p.tt.hbm + (long long)l * p.tt.page_bytes;  // frame 0
 }
-template <int V4, int RB>
+template <int V4, int RB, int CPG>
 __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(const __grid_constant__ RetrieveArgs p) {
   using namespace rekv_ptx;
   extern __shared__ __align__(16) float rk_smem[];
   const int Dp = p.Hkv * 128, nQ = p.qb.nQ, CL = p.CL;
-  const int cpg = CL / p.Hkv;                                   // CTAs that sum the rows of one KV group
-  float* s_vec = rk_smem;                                       // [nQ][Hkv * cpg][128] partial sums, from all CTAs
-  float* s_q = s_vec + nQ * p.Hkv * cpg * 128;                  // [nQ][Dp] question vectors
+  float* s_vec = rk_smem;                                       // [nQ][Hkv][CPG][128] partial sums, from all CTAs
+  float* s_q = s_vec + nQ * p.Hkv * CPG * 128;                  // [nQ][Dp] question vectors
   float* s_score = s_q + nQ * Dp;                               // [n_scored] of the question this CTA selects for
-  __shared__ float s_part[16][128];
-  __shared__ float s_red[RK_MAX_Q][16];
+  __shared__ __align__(16) float s_part[Q_SLOTS / 2][128];
+  __shared__ __align__(16) float s_red[RK_MAX_Q][32];            // square norms of the 32-dim blocks
   __shared__ __align__(8) unsigned long long s_bar[2];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int rank = (int)cluster_ctarank(), l = p.layer0 + blockIdx.y;
@@ -563,7 +577,7 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
     mbar_init(bar_vec, 1);
     mbar_init(bar_score, 1);
     fence_barrier_init();
-    mbar_expect_tx(bar_vec, (uint32_t)(nQ * p.Hkv * cpg * 512));
+    mbar_expect_tx(bar_vec, (uint32_t)(nQ * p.Hkv * CPG * 512));
     if (rank < nQ) mbar_expect_tx(bar_score, (uint32_t)p.n_scored * 4u);
   }
   __syncthreads();
@@ -576,7 +590,6 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
     return false;
   };
 
-  // the first items' rows: asked for now, used when the question vectors are there
   const int per = (p.n_scored + CL - 1) / CL;
   const int f0 = rank * per, f1 = min(f0 + per, p.n_scored);
   const float4* reps_l = reinterpret_cast<const float4*>(p.reps + (long long)l * p.max_frames * Dp) + lane;
@@ -591,74 +604,89 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
     }
   };
   int f = f0 + warp * RB;
-  if (f < f1) load_rows(f);
 
   // ---- question vectors: mean over the question's tokens and the G query heads of each KV group
-  const int G = p.Hq / p.Hkv, g = rank / cpg;
+  // (each CTA of a group's CPG takes Q_SLOTS / CPG of the sums, a slot -- two with CPG = 1 -- per 16 lanes of 16 bytes)
+  constexpr int slots = Q_SLOTS / CPG, TURNS = CPG == 1 ? 2 : 1;
+  const int G = p.Hq / p.Hkv, g = rank / CPG;
   for (int qi = 0; qi < nQ; ++qi) {
     const int n0 = p.qb.cu[qi], rows = (p.qb.cu[qi + 1] - n0) * G;
     if (g < p.Hkv) {
-      const int c = tid & 15, slots = 32 * cpg;
+      const int c = tid & 15;
       const uint4* base = p.q + (((long long)l * p.qb.sumNq + n0) * p.Hq + g * G) * 16 + c;
-      float acc[8];
+      const int sl = tid >> 4;
+      if (sl < slots) {
+        float acc[TURNS][8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i] = 0.f;
-      for (int m0 = (rank - g * cpg) * 32 + (tid >> 4); m0 < rows; m0 += 4 * slots) {
-        uint4 x[4];
+        for (int w = 0; w < TURNS; ++w)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int m = m0 + u * slots, n = m / G;
-          x[u] = m < rows ? __ldg(base + ((long long)n * p.Hq + (m - n * G)) * 16) : make_uint4(0, 0, 0, 0);
+          for (int i = 0; i < 8; ++i) acc[w][i] = 0.f;
+        for (int m0 = (rank - g * CPG) * slots + sl; m0 < rows; m0 += 4 * Q_SLOTS) {
+          uint4 x[TURNS][4];
+#pragma unroll
+          for (int w = 0; w < TURNS; ++w)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const int m = m0 + 32 * w + u * Q_SLOTS, n = m / G;
+              x[w][u] = m < rows ? __ldg(base + ((long long)n * p.Hq + (m - n * G)) * 16) : make_uint4(0, 0, 0, 0);
+            }
+#pragma unroll
+          for (int w = 0; w < TURNS; ++w)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const uint32_t v[4] = {x[w][u].x, x[w][u].y, x[w][u].z, x[w][u].w};
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                acc[w][2 * i] += __uint_as_float(v[i] << 16);
+                acc[w][2 * i + 1] += __uint_as_float(v[i] & 0xFFFF0000u);
+              }
+            }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const uint32_t v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+        for (int w = 0; w < TURNS; ++w) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            acc[2 * i] += __uint_as_float(v[i] << 16);
-            acc[2 * i + 1] += __uint_as_float(v[i] & 0xFFFF0000u);
+          for (int i = 0; i < 8; ++i) acc[w][i] += __shfl_xor_sync(0xffffffffu, acc[w][i], 16);
+          if (lane < 16) {
+            float4* dst = reinterpret_cast<float4*>(&s_part[warp + 16 * w][c * 8]);
+            dst[0] = make_float4(acc[w][0], acc[w][1], acc[w][2], acc[w][3]);
+            dst[1] = make_float4(acc[w][4], acc[w][5], acc[w][6], acc[w][7]);
           }
         }
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], 16);
-      if (lane < 16) {
-        float4* dst = reinterpret_cast<float4*>(&s_part[warp][c * 8]);
-        dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-        dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
       }
       __syncthreads();
       // thread t sends columns 4 (t & 31) .. of the CTA's sum to CTA t / 32 (every thread adds its columns up itself)
       if (warp < CL) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int w = 0; w < 16; ++w) {
-          const float4 x = *reinterpret_cast<const float4*>(&s_part[w][lane * 4]);
-          a.x += x.x;
-          a.y += x.y;
-          a.z += x.z;
-          a.w += x.w;
-        }
-        const uint32_t dst = smem_u32(s_vec + ((qi * p.Hkv * cpg + rank) * 128 + lane * 4));
+        auto add4 = [](const float4& a, const float4& b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); };
+        auto quad = [&](int k) {
+          const float4* x = reinterpret_cast<const float4*>(&s_part[4 * k][lane * 4]);
+          return add4(add4(x[0], x[32]), add4(x[64], x[96]));
+        };
+        float4 a = quad(0);
+        if (CPG <= 4) a = add4(a, quad(1));
+        if (CPG <= 2) a = add4(a, add4(quad(2), quad(3)));
+        if (CPG <= 1) a = add4(a, add4(add4(quad(4), quad(5)), add4(quad(6), quad(7))));
+        const uint32_t dst = smem_u32(s_vec + ((qi * p.Hkv * CPG + rank) * 128 + lane * 4));
         if (!((p.test & REKV_TEST_RETRIEVE_SKIP_SUM) && rank == 0 && blockIdx.y == 0))
           st_async_v4(mapa(dst, (uint32_t)warp), a, mapa(bar_vec, (uint32_t)warp));
       }
       __syncthreads();  // (s_part is written again for the next question)
     }
   }
+  if (f < f1) load_rows(f);  // the first items' rows arrive while the sums are exchanged
   bool ok = wait(bar_vec);
   for (int qi = 0; qi < nQ; ++qi) {
-    const float inv = (float)((p.qb.cu[qi + 1] - p.qb.cu[qi]) * G);
-    float sq = 0.f;
+    const float rows = (float)((p.qb.cu[qi + 1] - p.qb.cu[qi]) * G);
     for (int d = tid; d < Dp; d += 512) {
-      float a = 0.f;
-      for (int k = 0; k < cpg; ++k) a += s_vec[((qi * p.Hkv + (d >> 7)) * cpg + k) * 128 + (d & 127)];
-      a = __fdiv_rn(a, inv);
+      const float* v = s_vec + (qi * p.Hkv + (d >> 7)) * CPG * 128 + (d & 127);
+      float a = v[0];
+      if (CPG >= 2) a += v[128];
+      if (CPG >= 4) a += v[256] + v[384];
+      if (CPG >= 8) a += (v[512] + v[640]) + (v[768] + v[896]);
+      a = __fdiv_rn(a, rows);
       s_q[qi * Dp + d] = a;
-      sq += a * a;
+      const float sq = square_norm_of_warp(a);
+      if (lane == 0) s_red[qi][d >> 5] = sq;
     }
-    for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if (lane == 0) s_red[qi][warp] = sq;
   }
   __syncthreads();
 
@@ -692,14 +720,18 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
       float n = 0.f;
 #pragma unroll
       for (int i = 0; i < V4; ++i)
-        if (i < p.Hkv) n += r[b][i].x * r[b][i].x + r[b][i].y * r[b][i].y + r[b][i].z * r[b][i].z + r[b][i].w * r[b][i].w;
+        if (i < p.Hkv) n = add_dot4(n, r[b][i], r[b][i]);
       for (int o = 16; o; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
       rn[b] = fmaxf(__fsqrt_rn(n), eps);
     }
     for (int qi = 0; qi < nQ; ++qi) {
       float qn = 0.f;
 #pragma unroll
-      for (int w = 0; w < 16; ++w) qn += s_red[qi][w];
+      for (int k = 0; k < V4; ++k)
+        if (k < p.Hkv) {
+          const float4 x = *reinterpret_cast<const float4*>(&s_red[qi][4 * k]);
+          qn += (x.x + x.y) + (x.z + x.w);
+        }
       qn = fmaxf(__fsqrt_rn(qn), eps);
       float d[RB];
 #pragma unroll
@@ -709,7 +741,7 @@ __global__ void __launch_bounds__(512, V4 * RB <= 8 ? 2 : 1) retrieve_kernel(con
         if (i < p.Hkv) {
           const float4 a = s_q4[qi * (Dp / 4) + i * 32];
 #pragma unroll
-          for (int b = 0; b < RB; ++b) d[b] += r[b][i].x * a.x + r[b][i].y * a.y + r[b][i].z * a.z + r[b][i].w * a.w;
+          for (int b = 0; b < RB; ++b) d[b] = add_dot4(d[b], r[b][i], a);
         }
 #pragma unroll
       for (int b = 0; b < RB; ++b) {
@@ -874,20 +906,20 @@ int retrieve_cluster(const QBatch& qb, const StoreView& s, int nl, int n_scored,
 }
 // *launched: false where no cluster of that size can be resident -- 16 CTAs are beyond the portable size, and a partition of the
 // device may have no 16 SMs of one GPC -- and nothing was launched.
-template <int V4, int RB>
+template <int V4, int RB, int CPG>
 cudaError_t launch_retrieve_kernel(const RetrieveArgs& a, int nl, bool no_cluster, cudaStream_t st, bool* launched) {
   *launched = false;
   static PerDeviceOnce attr;
   cudaError_t e = attr.run([] {
-    cudaError_t e0 = cudaFuncSetAttribute(retrieve_kernel<V4, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+    cudaError_t e0 = cudaFuncSetAttribute(retrieve_kernel<V4, RB, CPG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
     if (e0 != cudaSuccess) return e0;
-    return cudaFuncSetAttribute(retrieve_kernel<V4, RB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return cudaFuncSetAttribute(retrieve_kernel<V4, RB, CPG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   });
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)a.CL, (unsigned)nl);
   cfg.blockDim = dim3(512);
-  cfg.dynamicSmemBytes = ((size_t)a.qb.nQ * (a.Hkv * (a.CL / a.Hkv) + a.Hkv) * 128 + a.n_scored) * sizeof(float);
+  cfg.dynamicSmemBytes = ((size_t)a.qb.nQ * (a.Hkv * CPG + a.Hkv) * 128 + a.n_scored) * sizeof(float);
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -903,13 +935,19 @@ cudaError_t launch_retrieve_kernel(const RetrieveArgs& a, int nl, bool no_cluste
   const bool cacheable = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < REKV_MAX_DEVICES;
   char state = cacheable ? known[dev][a.CL] : 0;
   if (!state) {
-    state = cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<V4, RB>, &cfg) == cudaSuccess && n > 0 ? 1 : 2;
+    state = cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<V4, RB, CPG>, &cfg) == cudaSuccess && n > 0 ? 1 : 2;
     if (state == 2) cudaGetLastError();
     if (cacheable) known[dev][a.CL] = state;
   }
   if (state == 2 || no_cluster) return cudaSuccess;
   *launched = true;
-  return cudaLaunchKernelEx(&cfg, retrieve_kernel<V4, RB>, a);
+  return cudaLaunchKernelEx(&cfg, retrieve_kernel<V4, RB, CPG>, a);
+}
+template <int V4, int CPG>
+cudaError_t launch_retrieve_rows(const RetrieveArgs& a, int nl, int rows, bool no_cluster, cudaStream_t st, bool* launched) {
+  if (V4 == 4 && rows == 4) return launch_retrieve_kernel<V4, V4 == 4 ? 4 : 2, CPG>(a, nl, no_cluster, st, launched);
+  return rows == 2 ? launch_retrieve_kernel<V4, 2, CPG>(a, nl, no_cluster, st, launched)
+                   : launch_retrieve_kernel<V4, 1, CPG>(a, nl, no_cluster, st, launched);
 }
 
 }  // namespace
@@ -960,13 +998,14 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
     cudaError_t e;
     const bool off = (c->test_retrieve & REKV_TEST_RETRIEVE_NO_CLUSTER) != 0;
     bool launched = false;
+    const int cpg = cl / s.Hkv >= 8 ? 8 : cl / s.Hkv >= 4 ? 4 : cl / s.Hkv >= 2 ? 2 : 1;
     if (s.Hkv <= 4)
-      e = rk_rows == 4   ? launch_retrieve_kernel<4, 4>(a, nl, off, st, &launched)
-          : rk_rows == 2 ? launch_retrieve_kernel<4, 2>(a, nl, off, st, &launched)
-                         : launch_retrieve_kernel<4, 1>(a, nl, off, st, &launched);
+      e = cpg == 8   ? launch_retrieve_rows<4, 8>(a, nl, rk_rows, off, st, &launched)
+          : cpg == 4 ? launch_retrieve_rows<4, 4>(a, nl, rk_rows, off, st, &launched)
+                     : launch_retrieve_rows<4, 2>(a, nl, rk_rows, off, st, &launched);
     else
-      e = rk_rows == 2 ? launch_retrieve_kernel<8, 2>(a, nl, off, st, &launched)
-                       : launch_retrieve_kernel<8, 1>(a, nl, off, st, &launched);
+      e = cpg == 2 ? launch_retrieve_rows<8, 2>(a, nl, rk_rows, off, st, &launched)
+                   : launch_retrieve_rows<8, 1>(a, nl, rk_rows, off, st, &launched);
     if (e != cudaSuccess) return e;
     if (launched) {
       c->launches += 1;

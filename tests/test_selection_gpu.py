@@ -99,27 +99,35 @@ def test_one_launch_retrieval_and_the_sizes_around_it(L, Hkv, T, b, lengths):
     g.close()
 
 
-@pytest.mark.parametrize("L,T,lengths", [(1, 64, [16]), (12, 60, [5, 9])])  # clusters of 16 and of 8 CTAs
-def test_retrieval_without_room_for_a_cluster_takes_the_three_launches(L, T, lengths):
-    s = H.Shape(L=L, Hq=8, Hkv=2, Nf=2, T=T, W=3, k=8, seed=7)
+@pytest.mark.parametrize("L,Hkv,G,T,b,lengths", [
+    (1, 2, 4, 64, 1, [16]), (12, 2, 4, 60, 1, [5, 9]),   # clusters of 16 and of 8 CTAs
+    (1, 1, 8, 90, 1, [40]), (2, 3, 2, 77, 1, [33, 1]), (9, 4, 7, 200, 1, [32]), (2, 8, 8, 100, 1, [20, 3, 30, 7]),
+    (10, 1, 4, 33, 1, [7]), (11, 5, 3, 50, 1, [50]), (12, 8, 2, 100, 1, [130]), (2, 4, 7, 163, 8, [20]), (10, 4, 7, 96, 2, [9])])
+def test_one_launch_and_three_launches_give_the_same_bits(L, Hkv, G, T, b, lengths):
+    """A context where no cluster can be resident takes the three launches, as larger tables do: the same scores to the bit,
+    and so the same selection; a layer at a time and rekv_score_frames_static as well.  (Question rows per KV group from 2 to
+    320, one to eight CTAs summing them.)"""
+    s = H.Shape(L=L, Hq=G * Hkv, Hkv=Hkv, Nf=2, T=T, W=3, k=8, seed=7, b=b)
     g = H.build_gpu(s, max_questions=len(lengths), max_q_tokens=sum(lengths))
     q, cu = H.questions(s, lengths, device="cuda")
 
     def retrieve():
         n = g.launch_count()
         idx, _, scores = g.retrieve(q, cu, 8, T, want_scores=True)
-        return idx, scores, g.launch_count() - n
+        n = g.launch_count() - n
+        idx_l = torch.empty_like(idx)
+        for l in range(L):
+            g.question_layer(l, q[l], cu, 8, T, idx=idx_l[l])
+        return idx, scores, idx_l, g.question(q, cu, 8, T), n
 
-    idx1, scores1, n1 = retrieve()
+    idx1, scores1, idx_l1, out1, n1 = retrieve()
     g.test_set_retrieve(rekv.TEST_RETRIEVE_NO_CLUSTER)
-    idx3, scores3, n3 = retrieve()
-    out3 = g.question(q, cu, 8, T)
+    idx3, scores3, idx_l3, out3, n3 = retrieve()
     g.check_status()
     assert (n1, n3) == (1, 3)
-    for l in range(L):
-        H.assert_close_rel(scores3[l], scores1[l], f"scores of layer {l}")
-    assert torch.equal(idx3, idx1)
-    g.test_set_retrieve(0)
-    assert torch.equal(g.question(q, cu, 8, T), out3)
-    g.check_status()
+    assert torch.equal(scores1, scores3) and torch.equal(idx1, idx3) and torch.equal(out1, out3)
+    assert torch.equal(idx_l1, idx1) and torch.equal(idx_l3, idx1)
+    if b == 1:
+        for l in range(L):
+            assert torch.equal(rekv.score_frames_static(q[l].contiguous(), cu, Hkv, g.get_reps(l, T)), scores1[l])
     g.close()
