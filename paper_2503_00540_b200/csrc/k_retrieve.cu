@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(512) topk_kernel(const float* __restrict__ sco
 // grid = (CTAs per cluster, layers), 512 threads; RB rows of float4 x V4 per lane are in flight per warp; CPG CTAs (1, 2, 4, 8) sum
 // the rows of one KV group.
 constexpr int RK_MAX_Q = 4;          // questions
-constexpr int RK_MAX_CL = 16;        // CTAs per cluster
+constexpr int RK_MAX_SMEM = 64 * 1024;
 constexpr int RK_MAX_ITEMS = 2048;   // items scored (the selection's histogram path)
 struct RetrieveArgs {
   const uint4* q;
@@ -891,63 +891,83 @@ cudaError_t launch_score(const ScoreArgs& a, bool pdl, cudaStream_t st) {
   return a.Dp <= 512 ? launch_score_v4<4>(a, pdl, st) : launch_score_v4<8>(a, pdl, st);
 }
 
-// CTAs per cluster of the one-launch retrieval, or 0 where the three launches are better: every warp has to hold all of its
-// rows at once (one round of loads).  28 layers of 1800 frames, 4 KV heads, one at a time: two rounds on 16 CTAs, 994 us
-// against 919 with the scores spread over 113 blocks; 9 layers of 439 frames, 8 KV heads: 229 against 253; 1 layer of 64
-// frames: 17.1 against 19.2.
+template <int V4, int RB, int CPG>
+cudaError_t prepare_retrieve_kernel() {  // once per device
+  static PerDeviceOnce attr;
+  return attr.run([] {
+    cudaError_t e = cudaFuncSetAttribute(retrieve_kernel<V4, RB, CPG>, cudaFuncAttributeMaxDynamicSharedMemorySize, RK_MAX_SMEM);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(retrieve_kernel<V4, RB, CPG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+}
+struct RetrieveLaunch {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[2];
+  RetrieveLaunch(int cl, int nl, size_t smem, cudaStream_t st) {
+    cfg.gridDim = dim3((unsigned)cl, (unsigned)nl);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)cl;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+  }
+};
+// Clusters of CL CTAs that the device can hold at once, asked once per device.  16 CTAs are beyond the portable size, and a
+// partition of the device may have no 16 SMs of one GPC: then 0.  (RB * V4 = 16: one CTA per SM, else two.)
+template <int V4, int RB, int CPG, int CL>
+int resident_retrieve_clusters() {
+  static int known[REKV_MAX_DEVICES] = {};  // + 1
+  int dev = 0, n = 0;
+  const bool cacheable = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < REKV_MAX_DEVICES;
+  if (cacheable && known[dev]) return known[dev] - 1;
+  RetrieveLaunch l(CL, 1, RK_MAX_SMEM, nullptr);
+  if (prepare_retrieve_kernel<V4, RB, CPG>() != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<V4, RB, CPG>, &l.cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  if (cacheable) known[dev] = n + 1;
+  return n;
+}
+
+// CTAs per cluster of the one-launch retrieval, or 0 where the three launches are better.
+// Every warp has to hold all of its rows at once (one round of loads): 28 layers of 1800 frames, 4 KV heads, one at a time: two
+// rounds on 16 CTAs, 994 us against 919 with the scores spread over 113 blocks; 9 layers of 439 frames, 8 KV heads: 229 against 253.
+// And all layers' clusters have to be resident at once: 16 CTAs with one per SM (7 layers), else 8 with two, less an eighth of the 33
+// that the device reports (29), since the last ones start late.  20 retrievals in a graph, clusters against three launches, us
+// each, 64 frames: 8 to 15 layers 5.9 against 8.8, 28 7.4 against 9.5, 30 7.5 against 9.6, 31 8.2 against 9.7, 32 10.1 against
+// 9.6, 80 19.4 against 15.3; 9 layers of 1000 frames on 16 CTAs 14.7 against 11.1.
 int retrieve_cluster(const QBatch& qb, const StoreView& s, int nl, int n_scored, int block, int top_k, int* rows) {
   if (qb.nQ > RK_MAX_Q || top_k <= 0 || n_scored <= 0 || (long long)qb.sumNq * s.Hq * 256 > (1 << 20)) return 0;
-  const bool few = nl * 16 <= rekv_sm_count();   // 16 CTAs per layer with up to 16 float4 per lane, or 8 with 8 (two CTAs per SM)
-  const int cl = few ? 16 : 8, most = (few ? 16 : 8) / (s.Hkv <= 4 ? 4 : 8);
+  const bool narrow = s.Hkv <= 4;
+  int cl = 16;
+  if (nl > (narrow ? resident_retrieve_clusters<4, 4, 4, 16>() : resident_retrieve_clusters<8, 2, 2, 16>())) {
+    cl = 8;
+    const int n8 = narrow ? resident_retrieve_clusters<4, 2, 2, 8>() : resident_retrieve_clusters<8, 1, 1, 8>();
+    if (nl > n8 - n8 / 8) return 0;
+  }
+  const int most = cl / (narrow ? 4 : 8);  // up to 16 float4 per lane on 16 CTAs, 8 on 8
   const long long frames = (long long)n_scored * block;
   // the fewest rows per warp that do it: short code, which every launch fetches anew
   for (*rows = 1; *rows < most && frames > (long long)cl * 16 * *rows;) *rows *= 2;
   return n_scored <= RK_MAX_ITEMS && frames <= (long long)cl * 16 * *rows ? cl : 0;
 }
-// *launched: false where no cluster of that size can be resident -- 16 CTAs are beyond the portable size, and a partition of the
-// device may have no 16 SMs of one GPC -- and nothing was launched.
 template <int V4, int RB, int CPG>
-cudaError_t launch_retrieve_kernel(const RetrieveArgs& a, int nl, bool no_cluster, cudaStream_t st, bool* launched) {
-  *launched = false;
-  static PerDeviceOnce attr;
-  cudaError_t e = attr.run([] {
-    cudaError_t e0 = cudaFuncSetAttribute(retrieve_kernel<V4, RB, CPG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-    if (e0 != cudaSuccess) return e0;
-    return cudaFuncSetAttribute(retrieve_kernel<V4, RB, CPG>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  });
+cudaError_t launch_retrieve_kernel(const RetrieveArgs& a, int nl, cudaStream_t st) {
+  const cudaError_t e = prepare_retrieve_kernel<V4, RB, CPG>();
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)a.CL, (unsigned)nl);
-  cfg.blockDim = dim3(512);
-  cfg.dynamicSmemBytes = ((size_t)a.qb.nQ * (a.Hkv * CPG + a.Hkv) * 128 + a.n_scored) * sizeof(float);
-  cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = (unsigned)a.CL;
-  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 2;
-  // clusters that can be resident, asked once per device and size: 0 unknown, 1 some, 2 none
-  static char known[REKV_MAX_DEVICES][RK_MAX_CL + 1] = {};
-  int dev = 0, n = 0;
-  const bool cacheable = cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < REKV_MAX_DEVICES;
-  char state = cacheable ? known[dev][a.CL] : 0;
-  if (!state) {
-    state = cudaOccupancyMaxActiveClusters(&n, retrieve_kernel<V4, RB, CPG>, &cfg) == cudaSuccess && n > 0 ? 1 : 2;
-    if (state == 2) cudaGetLastError();
-    if (cacheable) known[dev][a.CL] = state;
-  }
-  if (state == 2 || no_cluster) return cudaSuccess;
-  *launched = true;
-  return cudaLaunchKernelEx(&cfg, retrieve_kernel<V4, RB, CPG>, a);
+  RetrieveLaunch l(a.CL, nl, ((size_t)a.qb.nQ * (a.Hkv * CPG + a.Hkv) * 128 + a.n_scored) * sizeof(float), st);
+  return cudaLaunchKernelEx(&l.cfg, retrieve_kernel<V4, RB, CPG>, a);
 }
 template <int V4, int CPG>
-cudaError_t launch_retrieve_rows(const RetrieveArgs& a, int nl, int rows, bool no_cluster, cudaStream_t st, bool* launched) {
-  if (V4 == 4 && rows == 4) return launch_retrieve_kernel<V4, V4 == 4 ? 4 : 2, CPG>(a, nl, no_cluster, st, launched);
-  return rows == 2 ? launch_retrieve_kernel<V4, 2, CPG>(a, nl, no_cluster, st, launched)
-                   : launch_retrieve_kernel<V4, 1, CPG>(a, nl, no_cluster, st, launched);
+cudaError_t launch_retrieve_rows(const RetrieveArgs& a, int nl, int rows, cudaStream_t st) {
+  if (V4 == 4 && rows == 4) return launch_retrieve_kernel<V4, V4 == 4 ? 4 : 2, CPG>(a, nl, st);
+  return rows == 2 ? launch_retrieve_kernel<V4, 2, CPG>(a, nl, st) : launch_retrieve_kernel<V4, 1, CPG>(a, nl, st);
 }
 
 }  // namespace
@@ -974,7 +994,8 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
     tt.n_vis_frames = n_visible;
   }
   int rk_rows = 0;
-  if (const int cl = retrieve_cluster(qb, s, nl, n_scored, b, top_k, &rk_rows)) {
+  const int cl = c->test_retrieve & REKV_TEST_RETRIEVE_NO_CLUSTER ? 0 : retrieve_cluster(qb, s, nl, n_scored, b, top_k, &rk_rows);
+  if (cl) {
     RetrieveArgs a;
     a.q = (const uint4*)q;
     a.reps = s.reps;
@@ -996,21 +1017,17 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
     a.wait_limit = c->test_wait_limit;
     a.test = c->test_retrieve;
     cudaError_t e;
-    const bool off = (c->test_retrieve & REKV_TEST_RETRIEVE_NO_CLUSTER) != 0;
-    bool launched = false;
     const int cpg = cl / s.Hkv >= 8 ? 8 : cl / s.Hkv >= 4 ? 4 : cl / s.Hkv >= 2 ? 2 : 1;
     if (s.Hkv <= 4)
-      e = cpg == 8   ? launch_retrieve_rows<4, 8>(a, nl, rk_rows, off, st, &launched)
-          : cpg == 4 ? launch_retrieve_rows<4, 4>(a, nl, rk_rows, off, st, &launched)
-                     : launch_retrieve_rows<4, 2>(a, nl, rk_rows, off, st, &launched);
+      e = cpg == 8   ? launch_retrieve_rows<4, 8>(a, nl, rk_rows, st)
+          : cpg == 4 ? launch_retrieve_rows<4, 4>(a, nl, rk_rows, st)
+                     : launch_retrieve_rows<4, 2>(a, nl, rk_rows, st);
     else
-      e = cpg == 2 ? launch_retrieve_rows<8, 2>(a, nl, rk_rows, off, st, &launched)
-                   : launch_retrieve_rows<8, 1>(a, nl, rk_rows, off, st, &launched);
+      e = cpg == 2 ? launch_retrieve_rows<8, 2>(a, nl, rk_rows, st)
+                   : launch_retrieve_rows<8, 1>(a, nl, rk_rows, st);
     if (e != cudaSuccess) return e;
-    if (launched) {
-      c->launches += 1;
-      return cudaGetLastError();
-    }
+    c->launches += 1;
+    return cudaGetLastError();
   }
   if (n_scored > 0) {
     ScoreArgs a = {nl, n_scored, s.reps, c->qa, c->qnorm, qb.nQ, maxQ, s.Dp, s.Hkv, s.max_frames, scores, b, layer0, c->status};

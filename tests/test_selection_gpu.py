@@ -69,7 +69,8 @@ def test_selection_with_ties_crowded_steps_and_scores_that_are_not_numbers(patte
 
 @pytest.mark.parametrize("L,Hkv,T,b,lengths", [
     (1, 2, 256, 1, [3]), (1, 2, 1025, 1, [3]),        # 16 CTAs per layer, one row per warp at most; beyond four
-    (9, 4, 1024, 1, [5, 1]), (10, 4, 256, 1, [5]),    # ... 9 layers at most; 8 CTAs per layer from the tenth on
+    (7, 4, 1024, 1, [5, 1]), (9, 4, 1024, 1, [5, 1]), (10, 4, 256, 1, [5]),    # ... while one fits a GPC; then 8 CTAs per layer
+    (28, 2, 64, 1, [5]), (40, 2, 64, 1, [5]),         # ... while all layers' clusters are resident at once
     (10, 4, 257, 1, [5]), (2, 8, 512, 1, [2, 7, 1, 4]), (12, 8, 128, 1, [2]), (12, 8, 129, 1, [2]),
     (2, 3, 40, 1, [6]), (2, 4, 515, 8, [6]),           # idle CTAs; blocks
     (1, 1, 7, 1, [1] * 5), (2, 4, 51, 1, [1] * 7), (1, 8, 33, 1, [2] * 11), (2, 2, 50, 1, [1] * 20)])  # eight at a time, and the rest
@@ -102,7 +103,7 @@ def test_one_launch_retrieval_and_the_sizes_around_it(L, Hkv, T, b, lengths):
 @pytest.mark.parametrize("L,Hkv,G,T,b,lengths", [
     (1, 2, 4, 64, 1, [16]), (12, 2, 4, 60, 1, [5, 9]),   # clusters of 16 and of 8 CTAs
     (1, 1, 8, 90, 1, [40]), (2, 3, 2, 77, 1, [33, 1]), (9, 4, 7, 200, 1, [32]), (2, 8, 8, 100, 1, [20, 3, 30, 7]),
-    (10, 1, 4, 33, 1, [7]), (11, 5, 3, 50, 1, [50]), (12, 8, 2, 100, 1, [130]), (2, 4, 7, 163, 8, [20]), (10, 4, 7, 96, 2, [9])])
+    (10, 1, 4, 33, 1, [7]), (11, 5, 3, 50, 1, [50]), (12, 8, 2, 100, 1, [130]), (2, 4, 7, 163, 8, [20]), (10, 4, 7, 96, 2, [9]), (28, 4, 7, 64, 1, [32])])
 def test_one_launch_and_three_launches_give_the_same_bits(L, Hkv, G, T, b, lengths):
     """A context where no cluster can be resident takes the three launches, as larger tables do: the same scores to the bit,
     and so the same selection; a layer at a time and rekv_score_frames_static as well.  (Question rows per KV group from 2 to
