@@ -22,13 +22,15 @@ __device__ __forceinline__ float square_norm_of_warp(float a) {  // of the warp'
 }
 
 // ---- question vector: mean over the question's tokens and over the G query heads of each KV group
-// grid = (nQ, layers, H_kv), layer = layer0 + blockIdx.y; 1024 threads = 64 row slots x 16 lanes of 16 bytes, four rows
-// per thread in flight: a question of 36 tokens at G = 7 is one round of loads deep (latency is all this kernel has).
+// grid = (nQ, layers, H_kv), layer = layer0 + blockIdx.y; 1024 threads = 64 row slots x 16 lanes of 16 bytes, U rows
+// per thread in flight.  Latency is all this kernel has: with U = 4 a question of 36 tokens at G = 7 is one round of loads deep,
+// and a block has an SM for itself (46 registers); launches of more blocks than SMs take U = 2 and two blocks per SM.
 // Writes the group's 128 dims of the question vector and its partial sum of squares (the score kernel adds the H_kv partials).
 constexpr int QM_THREADS = 1024;
-__global__ void __launch_bounds__(QM_THREADS) qmean_kernel(const uint4* __restrict__ q, QBatch qb, int Hq, int Hkv, int G,
-                                                           float* __restrict__ qa, float* __restrict__ qsq, int maxQ,
-                                                           int layer0) {
+template <int U>
+__global__ void __launch_bounds__(QM_THREADS, U <= 2 ? 2 : 1)
+    qmean_kernel(const uint4* __restrict__ q, QBatch qb, int Hq, int Hkv, int G, float* __restrict__ qa, float* __restrict__ qsq,
+                 int maxQ, int layer0) {
   // launched with programmatic stream serialisation: its blocks are resident when the kernel before it ends (the
   // caller's, which wrote the queries, or the library's own), and wait here for that kernel's results
   rekv_ptx::grid_dep_wait();
@@ -40,15 +42,15 @@ __global__ void __launch_bounds__(QM_THREADS) qmean_kernel(const uint4* __restri
   float acc[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0.f;
-  for (int m0 = slot; m0 < rows; m0 += 256) {
-    uint4 x[4];
+  for (int m0 = slot; m0 < rows; m0 += U * Q_SLOTS) {
+    uint4 x[U];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int m = m0 + 64 * u, n = m / G;
+    for (int u = 0; u < U; ++u) {
+      const int m = m0 + Q_SLOTS * u, n = m / G;
       x[u] = m < rows ? __ldg(base + ((long long)n * Hq + (m - n * G)) * 16) : make_uint4(0, 0, 0, 0);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < U; ++u) {
       const uint32_t v[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -1032,7 +1034,7 @@ cudaError_t rekv_launch_retrieve(rekv_ctx* c, const void* q, const QBatch& qb, i
   if (n_scored > 0) {
     ScoreArgs a = {nl, n_scored, s.reps, c->qa, c->qnorm, qb.nQ, maxQ, s.Dp, s.Hkv, s.max_frames, scores, b, layer0, c->status};
     cudaError_t e;
-    e = rekv_launch_pdl(qmean_kernel, dim3(qb.nQ, nl, s.Hkv), dim3(QM_THREADS), 0, st, (const uint4*)q, qb, s.Hq,
+    e = rekv_launch_pdl((long long)qb.nQ * nl * s.Hkv > rekv_sm_count() ? qmean_kernel<2> : qmean_kernel<4>, dim3(qb.nQ, nl, s.Hkv), dim3(QM_THREADS), 0, st, (const uint4*)q, qb, s.Hq,
                         s.Hkv, s.G, c->qa, c->qnorm, maxQ, layer0);
     if (e != cudaSuccess) return e;
     c->launches += 1;
@@ -1163,7 +1165,7 @@ extern "C" int rekv_score_frames_static(const void* q, const int32_t* cu_q, int 
 
   const int Dp = n_kv_heads * REKV_HEAD_DIM, G = n_q_heads / n_kv_heads;
   cudaStream_t st = (cudaStream_t)stream;
-  qmean_kernel<<<dim3(nQ, 1, n_kv_heads), QM_THREADS, 0, st>>>((const uint4*)q, qb, n_q_heads, n_kv_heads, G, qa, qsq,
+  qmean_kernel<4><<<dim3(nQ, 1, n_kv_heads), QM_THREADS, 0, st>>>((const uint4*)q, qb, n_q_heads, n_kv_heads, G, qa, qsq,
                                                          STATIC_MAX_QUESTIONS, 0);
   const ScoreArgs a = {1, n_frames, reps, qa, qsq, nQ, STATIC_MAX_QUESTIONS, Dp, n_kv_heads, n_frames, scores_out, 1, 0, nullptr};
   e = launch_score(a, false, st);
