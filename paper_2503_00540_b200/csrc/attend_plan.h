@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <numeric>
 
 constexpr int REKV_MAX_PARTS_INSIDE = 4;  // parts of a unit that the attention kernel joins itself
 
@@ -13,33 +14,43 @@ struct AttendPlan {
 
 // total: chunks of all units; max_ch: of the longest unit; equal: every unit has max_ch; max_w: workers that can run at once;
 // may_merge: a merge launch may follow.
+//
+// What a number of workers costs (us), from launches of 1 to 28 layers: 0.75 for each chunk of a range, which run one after the
+// other; 8 for each segment of a range (the part of a unit in it: Q, the pipeline's start, the result); 4 for each end of a range
+// that cuts a unit (partials written and joined inside, at the end of the segment), or 2 for the merge launch and 0.05 for each
+// part.  The longest range decides, so that a few workers less can be faster: equal units per worker have no cuts, and ranges
+// of 4/3 units touch two units each where 1.3 units touch three.  One B200, all workers (74 pairs) against this choice, us:
+//   12 layers of 144 units of 50 chunks   151 -> 142 (72 workers)     8 layers, 96 units of 50     112 -> 104 (72)
+//   encoding step, 192 units of 15        102 -> 94 (64)              12 layers, 48 units of 113   120 -> 115 (72)
+//   28 layers one at a time, 4 units of 113: 1 worker per unit 3268, 2, 3, 4 joined inside 2096, 1672, 1490, 6, 9, 18 with the
+//   merge launch 1112, 978, 918; 8 units of 11, 9 layers: 322, 300, 288, 295, 255, 264.
 inline AttendPlan rekv_attend_plan(int total, int units, int max_ch, bool equal, int max_w, bool may_merge) {
-  // Long ranges: all workers there are, ranges cut where they fall.  A launch of few units (one layer) is a trade
-  // between chunks one after the other (0.8 us each), a range with parts of two units (a second Q, result and pipeline start:
-  // whole workers per unit avoid it), and joining parts.  The merge launch costs such a launch about 2 us, a join inside the
-  // kernel 4 to 6 (fence, counter and the parts' latency, one after the other, at its very end).  28 layers one at a time,
-  // 113 chunks, 4 units (us): 1 worker per unit 3268, 2, 3, 4 joined inside 2096, 1672, 1490, 6, 9, 18 with the merge launch
-  // 1112, 978, 918; 11 chunks, 8 units, 9 layers: 322, 300, 288, 295, 255, 264.
-  AttendPlan p;
-  p.workers = std::min(max_w, total);
-  auto joins = [&] { return (max_ch - 1) / std::max(1, total / p.workers) + 2 <= REKV_MAX_PARTS_INSIDE; };  // parts of a unit, at most
-  p.merge_inside = joins();
-  float best = 0.8f * (float)((total + p.workers - 1) / p.workers) + (units % p.workers ? 9.f : 0.f);
-  // (k: two chunks at least in the longest unit's ranges; where the others are much shorter, units * k can exceed all chunks)
-  for (int k = 1; (k == 1 || k < max_ch) && units * k <= std::min(max_w, total); ++k) {
-    const float t = 0.8f * (float)((max_ch + k - 1) / k) + (k == 1 ? 0.f : 2.f + 0.05f * (float)k);
-    if (t < best) {
-      best = t;
-      p.workers = units * k;
-      p.merge_inside = k == 1 && equal;
+  constexpr float CHUNK = 0.75f, SEGMENT = 8.f, CUT = 4.f, MERGE = 2.f, MERGE_PART = 0.05f;
+  const int most = std::min(max_w, total);
+  AttendPlan best = {0, true};
+  float best_cost = 0.f;
+  for (int w = most; w >= 1 && (3 * w >= most || best.workers == 0); --w) {
+    // the most segments of a range, partial segments of a range and parts of a unit.  Equal units, units / w = p / q in lowest
+    // terms: ranges start at multiples of 1 / q of a unit (rounded up to a chunk, which cuts no further unit).
+    int segments = units / w + 2, cuts = 2, parts = (max_ch - 1) / (total / w) + 2;
+    bool even = false;  // q whole workers for each unit
+    if (equal) {
+      const int g = std::gcd(units, w), p = units / g, q = w / g;
+      segments = (p - 1 + q - 1) / q + 1;
+      parts = (q - 1 + p - 1) / p + 1;
+      cuts = q == 1 ? 0 : p == 1 || q == 2 ? 1 : 2;
+      even = p == 1;
+    }
+    const bool inside = parts <= REKV_MAX_PARTS_INSIDE;
+    if (!inside && !may_merge) continue;
+    const bool by_merge = !inside || (even && cuts > 0 && may_merge);
+    const float join = by_merge ? MERGE + MERGE_PART * (float)parts
+                                : CUT * (float)cuts + (equal && !even && parts > 2 ? CUT * (float)(parts - 2) : 0.f);
+    const float cost = CHUNK * (float)((total + w - 1) / w) + SEGMENT * (float)segments + join;
+    if (best.workers == 0 || cost < best_cost) {
+      best = {w, !by_merge};
+      best_cost = cost;
     }
   }
-  if (!may_merge && !p.merge_inside) {
-    // Fewer workers: whole units each where all are equally long; where one is much longer than the rest, ranges of more than
-    // a third of it, so that it falls into four at most.
-    const int range = (max_ch - 1) / (REKV_MAX_PARTS_INSIDE - 1) + 1;
-    p.workers = std::min({p.workers, units, total / range});
-    p.merge_inside = true;
-  }
-  return p;
+  return best;
 }
