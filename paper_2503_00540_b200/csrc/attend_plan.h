@@ -13,19 +13,22 @@ struct AttendPlan {
 };
 
 // total: chunks of all units; max_ch: of the longest unit; equal: every unit has max_ch; max_w: workers that can run at once;
-// may_merge: a merge launch may follow.
+// may_merge: a merge launch may follow; pairs: workers are CTA pairs.
 //
-// What a number of workers costs (us), from launches of 1 to 28 layers: 0.75 for each chunk of a range, which run one after the
-// other; 8 for each segment of a range (the part of a unit in it: Q, the pipeline's start, the result); 4 for each end of a range
-// that cuts a unit (partials written and joined inside, at the end of the segment), or 2 for the merge launch and 0.05 for each
+// What a number of workers costs (us), from launches of 1 to 28 layers: 0.75 for each chunk of a range -- 1 on single CTAs, which
+// bring whole tiles -- one after the other; 8 for each segment of a range (the part of a unit in it: Q, the pipeline's start, the result); 4 for each end of a range
+// that cuts a unit (partials written and joined inside, at the end of the segment), or 2 for the merge launch and 0.15 for each
 // part.  The longest range decides, so that a few workers less can be faster: equal units per worker have no cuts, and ranges
 // of 4/3 units touch two units each where 1.3 units touch three.  One B200, all workers (74 pairs) against this choice, us:
 //   12 layers of 144 units of 50 chunks   151 -> 142 (72 workers)     8 layers, 96 units of 50     112 -> 104 (72)
 //   encoding step, 192 units of 15        102 -> 94 (64)              12 layers, 48 units of 113   120 -> 115 (72)
+//   (single CTAs, 28 layers, 112 units of 113: 148 workers 164, 140 workers 169)
 //   28 layers one at a time, 4 units of 113: 1 worker per unit 3268, 2, 3, 4 joined inside 2096, 1672, 1490, 6, 9, 18 with the
 //   merge launch 1112, 978, 918; 8 units of 11, 9 layers: 322, 300, 288, 295, 255, 264.
-inline AttendPlan rekv_attend_plan(int total, int units, int max_ch, bool equal, int max_w, bool may_merge) {
-  constexpr float CHUNK = 0.75f, SEGMENT = 8.f, CUT = 4.f, MERGE = 2.f, MERGE_PART = 0.05f;
+inline AttendPlan rekv_attend_plan(int total, int units, int max_ch, bool equal, int max_w, bool may_merge,
+                                    bool pairs) {
+  const float CHUNK = pairs ? 0.75f : 1.f;
+  constexpr float SEGMENT = 8.f, CUT = 4.f, MERGE = 2.f, MERGE_PART = 0.15f;
   const int most = std::min(max_w, total);
   AttendPlan best = {0, true};
   float best_cost = 0.f;

@@ -1130,7 +1130,7 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
   if (total > 0x7fffffff / 2) return cudaErrorInvalidValue;
   p.total = (int)total;
   // (split launches: no merge launch between or after the two)
-  const AttendPlan plan = rekv_attend_plan(p.total, p.nl * p.Hkv * blocks, max_ch, equal, max_workers<CG>(), !p.split_rem);
+  const AttendPlan plan = rekv_attend_plan(p.total, p.nl * p.Hkv * blocks, max_ch, equal, max_workers<CG>(), !p.split_rem, CG == 2);
   p.W = plan.workers;
   p.merge_inside = plan.merge_inside;
   cudaLaunchConfig_t cfg = {};

@@ -12,8 +12,8 @@ import pytest
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2503_00540_b200", "csrc")
 SOURCE = """
 #include "attend_plan.h"
-extern "C" int plan(int total, int units, int max_ch, int equal, int max_w, int may_merge, int* workers) {
-  const AttendPlan p = rekv_attend_plan(total, units, max_ch, equal != 0, max_w, may_merge != 0);
+extern "C" int plan(int total, int units, int max_ch, int equal, int max_w, int may_merge, int pairs, int* workers) {
+  const AttendPlan p = rekv_attend_plan(total, units, max_ch, equal != 0, max_w, may_merge != 0, pairs != 0);
   *workers = p.workers;
   return p.merge_inside;
 }
@@ -32,7 +32,7 @@ def plan(tmp_path_factory):
         """chunks: of one (layer, KV head)'s units, in launch order; lh: how many (layer, KV head) there are"""
         w = ctypes.c_int()
         inside = fn(sum(chunks) * lh, len(chunks) * lh, max(chunks), int(min(chunks) == max(chunks)), max_w, int(may_merge),
-                    ctypes.byref(w))
+                    int(max_w <= 74), ctypes.byref(w))
         return w.value, bool(inside)
     return call
 
