@@ -110,14 +110,14 @@ typedef struct {
   int32_t last_ctx_frames;   /* k_eff + window frames of the last gather */
   double last_attend_kernel_us; /* device time of the last attention kernel launch (REKV_FLAG_TIMING, HBM
                                    tier): it includes the joining of units cut between CTAs when the kernel does
-                                   that itself (two or three parts per unit), not a merge kernel that followed
+                                   that itself (at most four parts per unit), not a merge kernel that followed
                                    (last_merge_us); 0 when not measured */
   double last_retrieve_us;      /* REKV_FLAG_TIMING: steps 2-3 of the last question (question vectors, scores,
                                    selection) on the caller's stream; 0 when not measured or not finished yet */
   double last_pull_us;          /* REKV_FLAG_TIMING, offloaded contexts: the last gather's pulls over the host
                                    link, all layers, on the internal stream; 0 when not measured or not finished */
   double last_merge_us;         /* REKV_FLAG_TIMING: the merge kernel that followed the last attention kernel
-                                   (units cut into more than three parts); 0 when none ran or not measured */
+                                   (launches of few units, several workers each); 0 when none ran or not measured */
 } rekv_stats_t;
 
 /* Creates a context on cfg->device: allocates the frame store (HBM tier, and the pinned-host tier
@@ -196,7 +196,8 @@ int rekv_attend(rekv_ctx* ctx, const void* q, const int32_t* cu_q, int nQ, void*
  * paragraph): context token j (context order: retrieved frames ascending, then the trailing frames) has
  * position j, token s of X has position n_ctx + s.  q, k_self and the stored keys are given UN-rotated;
  * rotated vectors are rounded to bf16.  The rotated copies of the context's keys are written to a
- * workspace first (one extra pass over the context's K).
+ * workspace first (one extra pass over the context's K), but for batches of at most 16 rows per KV head and
+ * question (decode steps), whose keys are rotated on the way.
  * Needs max_self_tokens > 0 at creation.  Returns 0 or an error code (REKV_ERR_STATE without a gather). */
 int rekv_attend_full(rekv_ctx* ctx, const void* q, const void* k_self, const void* v_self, const int32_t* cu_q,
                      const int32_t* cu_self, int nQ, void* out, void* stream);
@@ -231,7 +232,8 @@ int rekv_question(rekv_ctx* ctx, const void* q, const int32_t* cu_q, int nQ, int
  *   cu_q, nQ, top_k, n_visible   as in rekv_retrieve
  *   idx_out   device int32 [nQ][top_k] (nullable): the layer's selection, ascending, -1 past k_eff
  *   out       device bf16 [sum_Nq][H_q][D]
- * Same arithmetic, kernels and results as the all-layer calls restricted to that layer.  Nothing is
+ * The selection is that of the all-layer calls, to the bit; the output is theirs to the rounding of bf16 (the
+ * attention of one layer is cut elsewhere, and its parts joined in another order).  Nothing is
  * allocated and the host is not synchronised; on a context whose cache is all in HBM the call may be
  * captured into a CUDA graph (one graph per layer, replayed while the stored frames, n_visible and the
  * buffers stay the same); an offloaded context uses the internal side stream and must not be captured.

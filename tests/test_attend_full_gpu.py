@@ -63,7 +63,7 @@ def test_batch_of_mixed_lengths_with_generated_tokens(theta):
 
 @pytest.mark.parametrize("theta", THETAS)
 def test_decode_step_with_a_long_own_history(theta):
-    """One query row per question, 150 tokens of own K/V (three 64-token tiles in the self kernel)."""
+    """One query row per question, 150 tokens of own K/V (one 208-token tile of X behind the frames)."""
     s = H.Shape(L=2, Hq=28, Hkv=4, Nf=196, T=24, W=4, k=8, seed=7)
     _run(s, [1, 1], [150, 65], theta)
 
@@ -75,8 +75,8 @@ def test_72b_head_shape(theta):
 
 @pytest.mark.parametrize("theta", THETAS)
 def test_units_cut_in_two_or_three_are_finished_in_the_kernel_with_the_part_over_x(theta):
-    """80 units of two row tiles over 146 CTAs: every unit is cut into two or three parts, which the CTA that completes
-    the last one joins -- together with the part over X, the first part in the fixed order."""
+    """80 units of two row tiles over 72 CTA pairs: nearly every unit, whose last chunk holds X, is cut in two, and the pair
+    that completes the second part joins them."""
     s = H.Shape(L=10, Hq=16, Hkv=8, Nf=100, T=28, W=4, k=16, seed=2503)
     _run(s, [80], [96], theta)
 
@@ -109,9 +109,8 @@ def test_many_units_take_the_whole_unit_path(theta):
 
 
 @pytest.mark.parametrize("theta", THETAS)
-def test_many_short_questions_half_streams(theta):
-    """640 uncut units of one row tile each: two half-streams per unit, joined with the part over X by the merge
-    kernel."""
+def test_many_short_questions_in_one_batch(theta):
+    """640 units of one row tile and a few chunks each, single CTAs with several units one after the other."""
     s = H.Shape(L=4, Hq=16, Hkv=8, Nf=33, T=12, W=2, k=4, seed=540)
     nq = [9 + (7 * i) % 32 for i in range(20)]
     _run(s, nq, [n + (i % 3) for i, n in enumerate(nq)], theta)
@@ -209,8 +208,7 @@ def test_layer_calls_of_eq3_in_full(theta, tail, k):
     """What a decoder layer calls with the Q, K, V it has just made of X: rekv_question_layer_full per layer (steps 2-5
     with Eq. 3 in full), then decode steps through rekv_attend_full_layer over the layer's context -- against the
     oracle per layer, and against the all-layer calls on the same selection."""
-    # (k = 26: 30 context frames, ten or eleven partials per unit of a one-layer launch -- the merge kernel for units of
-    # many parts takes the part over X in)
+    # (k = 26: 30 context frames, many parts per unit of a one-layer launch, joined by the merge kernel)
     s = H.Shape(L=3, Hq=28, Hkv=4, Nf=196, T=40, W=4, k=k, seed=540, tail=tail)
     nq, ns = [24, 33], [24, 40]
     g = H.build_gpu(s, max_questions=2, max_q_tokens=sum(nq), max_self_tokens=sum(ns) + 2, rope_theta=theta)
@@ -252,8 +250,7 @@ def test_layer_calls_of_eq3_in_full(theta, tail, k):
 
 @pytest.mark.parametrize("theta", THETAS)
 def test_layer_calls_of_eq3_in_full_replayed_from_a_cuda_graph(theta):
-    """A decoder captured whole: the layers' rekv_question_layer_full calls as nodes of one graph (the part over X forks
-    to the library's internal stream and joins again inside the capture).  The replay gives the eager calls' bits,
+    """A decoder captured whole: the layers' rekv_question_layer_full calls as nodes of one graph.  The replay gives the eager calls' bits,
     also after the buffers were given another question."""
     s = H.Shape(L=3, Hq=28, Hkv=4, Nf=196, T=40, W=4, k=8, seed=7)
     g = H.build_gpu(s, max_questions=1, max_q_tokens=32, max_self_tokens=32, rope_theta=theta)

@@ -45,14 +45,14 @@ def _expire_then_recover(s: H.Shape, lengths, skip_entry: int):
 @pytest.mark.parametrize("skip_entry", [0, 1, 3])
 def test_tensor_core_kernel_gives_up_when_a_tile_never_arrives(skip_entry):
     """64 query rows per KV head: the tcgen05 kernel.  Entry 0 is a K tile (the S product waits for it), entry 1 a V
-    tile (the P V product waits), entry 3 the second chunk's V tile of the first CTA's range (320 (unit, frame) steps
-    over 148 CTAs: three 48-token frames = two chunks per CTA)."""
+    tile (the P V product waits), entry 3 the second chunk's V tile of the first CTA's range (eight units
+    of 15 chunks, eight CTAs each)."""
     s = H.Shape(L=4, Hq=8, Hkv=2, Nf=48, T=60, W=4, k=36, seed=7)
     _expire_then_recover(s, [16], skip_entry)
 
 
 def test_a_cta_that_gives_up_leaves_its_units_unfinished_and_their_counters_are_cleared():
-    """80 units of two row tiles, each cut into two or three parts that the attention kernel joins itself by counting
+    """80 units of two row tiles, most of them cut in two parts that the attention kernel joins itself by counting
     the parts per unit.  The first CTA gives up on its first K tile: its parts are never counted, the units it shares
     stay unfinished behind the status word, and reading the status clears the counters -- the next question would
     otherwise join the wrong parts."""

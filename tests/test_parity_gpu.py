@@ -8,7 +8,7 @@ from tests import harness as H
 
 pytestmark = pytest.mark.gpu
 
-# both attention kernels are checked: the tcgen05 one (default) and the mma.sync one
+# (the decode-shaped kernel, mma.sync, has its own file)
 ATT = [pytest.param(0, id="tcgen05")]
 
 
@@ -84,42 +84,40 @@ def test_72b_head_shape(flags):
     _run_question_parity(s, [64], flags=flags)
 
 
-def test_many_short_questions_whole_units_as_half_streams():
-    """640 units of one row tile each (more than four per SM, so no unit is cut at a CTA boundary): every unit runs
-    as two half-streams; the half that finishes second joins the other's partial inside the kernel, with partial slots
-    counted per such unit."""
+def test_many_short_questions_in_one_batch():
+    """640 units of one row tile and two chunks each: single CTAs that take several units one after the other, with Q and
+    result double-buffered between them."""
     s = H.Shape(L=4, Hq=16, Hkv=8, Nf=33, T=12, W=2, k=4, seed=540)
     lengths = [9 + (7 * i) % 32 for i in range(20)]  # 18..80 rows per KV head
     _run_question_parity(s, lengths, max_questions=20)
 
 
-def test_half_streams_over_a_context_of_a_single_chunk():
-    """As above with three context frames of 33 tokens (113 stream rows: one chunk): the second half-stream of every
-    unit has no chunk at all and contributes the neutral part."""
+def test_many_short_questions_over_a_context_of_a_single_chunk():
+    """As above with three context frames of 33 tokens (113 stream rows: one chunk, with gap rows inside): the first chunk
+    of every unit is its last."""
     s = H.Shape(L=4, Hq=16, Hkv=8, Nf=33, T=12, W=1, k=2, seed=7)
     lengths = [9 + (7 * i) % 32 for i in range(20)]
     _run_question_parity(s, lengths, max_questions=20)
 
 
 def test_short_question_cut_at_cta_boundaries():
-    """One 10-token question at the 7B head shape: 70 rows = one row tile per unit, units cut at CTA boundaries
-    (four to six partials per unit: the merge kernel joins them)."""
+    """One 10-token question at the 7B head shape: 70 rows = one row tile per unit, several whole CTAs per unit, whose
+    parts the merge kernel joins."""
     s = H.Shape(L=3, Hq=28, Hkv=4, Nf=196, T=30, W=4, k=12, seed=7)
     _run_question_parity(s, [10])
 
 
 def test_units_of_two_questions_cut_into_a_few_parts():
-    """The same regime with a batch: 80 units of two questions (160 and 144 rows per KV head), cut into two or three
+    """The same regime with a batch: 80 units of two questions (160 and 144 rows per KV head), cut into two
     parts and finished inside the kernel."""
     s = H.Shape(L=5, Hq=16, Hkv=8, Nf=100, T=28, W=4, k=16, seed=540)
     _run_question_parity(s, [80, 72])
 
 
 def test_units_cut_into_a_few_parts_are_finished_inside_the_kernel():
-    """80 units of two row tiles over 146 CTAs (on 148 SMs), eleven of a unit's twenty context frames per CTA: every
-    unit is cut into two or three parts, and the CTA that finishes a unit's last part joins them (from its own
-    accumulator if the others are already there, from the written partials otherwise).  Both ways do the same
-    arithmetic in part order: repeated launches give the same bits whichever CTA came last."""
+    """80 units of two row tiles over 72 CTA pairs: nearly every unit is cut in two, and the pair that finishes its second
+    part joins them (from its own accumulator if the other is already there, from the written partials otherwise).  Both
+    ways do the same arithmetic in part order: repeated launches give the same bits whichever came last."""
     s = H.Shape(L=10, Hq=16, Hkv=8, Nf=100, T=28, W=4, k=16, seed=2503)
     _run_question_parity(s, [80])
     g = H.build_gpu(s, max_questions=1, max_q_tokens=80)
@@ -132,11 +130,18 @@ def test_units_cut_into_a_few_parts_are_finished_inside_the_kernel():
     g.close()
 
 
+def test_the_few_remainders_of_a_large_batch_are_cut_in_four():
+    """15 questions of one CTA pair per unit and one with 24 rows more: a launch of pairs and one of single CTAs beside it,
+    four whole CTAs for each of its 32 units, whose parts are joined in the kernel."""
+    s = H.Shape(L=8, Hq=28, Hkv=4, Nf=64, T=20, W=4, k=16, seed=540)
+    _run_question_parity(s, [32] * 15 + [40])
+
+
 @pytest.mark.parametrize("n_tokens", [40, 10, 1])
 def test_few_units_of_many_parts_each(n_tokens):
-    """Two units (one layer, two KV heads) over 48 context frames: three or four frames per CTA, 13 to 34 partials per
-    unit, joined by the merge kernel for units of many parts -- with two row tiles (40 tokens x 4 heads), as two
-    half-streams (10 tokens) and in the decode-shaped kernel (1 token)."""
+    """Two units (one layer, two KV heads) over 48 context frames, several workers each: with two row tiles (40 tokens x 4
+    heads: pairs) and one (10 tokens: single CTAs), joined by the merge kernel, and in the decode-shaped kernel (1 token),
+    which joins its parts itself."""
     s = H.Shape(L=1, Hq=8, Hkv=2, Nf=16, T=80, W=8, k=40, seed=7)
     _run_question_parity(s, [n_tokens])
 
@@ -312,8 +317,8 @@ def test_logits_far_above_the_first_chunk_raise_the_reference_maximum(n_tokens):
     """The attention kernel keeps the row maximum of a range's first 128-token chunk as the reference of its
     exponentials and only checks that a chunk's row sum stays below 2^60.  Here the last context frame holds keys whose
     logits lie about 80 octaves above everything before them: the rare path (true maximum, rescaling of O and of the
-    running sum, second pass) must give the oracle's answer.  16 tokens: one row tile, two half-streams; 40 tokens: two
-    row tiles."""
+    running sum, second pass) must give the oracle's answer.  16 tokens: one row tile, a single CTA; 40 tokens: two
+    row tiles, a CTA pair."""
     s = H.Shape(L=1, Hq=8, Hkv=2, Nf=48, T=12, W=2, k=6, seed=7)
     g = rekv.ReKV(s.L, s.Hq, s.Hkv, s.D, s.Nf, s.T, s.W, max_q_tokens=n_tokens, max_topk=s.k)
     o = orc.OracleCache(s.L, s.Hq, s.Hkv, s.D, s.Nf, s.W)
