@@ -41,9 +41,10 @@
 // marked, put out no result, and is run again at the end of the CTA's range chunk by chunk, with O rescaled when the
 // maximum is raised (never with ordinary inputs).
 //
-// A segment that is not a whole unit is a part of it, (max, sum, O) per row.  With up to four parts per unit the
-// worker that completes the last one joins them: if every other part is counted when its own is done, straight from its O
-// registers.  Nobody waits for anybody.  With more parts merge_tc5_kernel joins them.
+// A segment that is not a whole unit is a part of it, (max, sum, O) per row.  Up to four parts per unit are joined by the
+// worker that completes the last one: if every other part is counted when its own is done, straight from its O
+// registers.  Nobody waits for anybody.  Else merge_tc5_kernel joins them
+// (attend_plan.h says when).
 // Every wait is bounded: on expiry the status word is set and the CTA leaves.
 #include <algorithm>
 #include <type_traits>
@@ -977,7 +978,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
   if (warp == 0) tmem_dealloc<CG>(tmem, TMEM_COLS);
 }
 
-// Joins the parts of units that were cut into more than MAX_PARTS_INSIDE (launches of few units, such as one layer).
+// Joins the parts of units where the attention kernel does not (launches of few units, such as one layer: several whole workers
+// each; units of more than MAX_PARTS_INSIDE parts).
 // grid = (units, CTAs of a pair, 32 column quads), 256 threads: a thread per (row, every second part), consecutive threads on
 // consecutive rows, so that a part is read in 2 KB runs and 16 parts are one round of loads deep; the two groups' results
 // meet in shared memory.  (28 layers, 28 heads, 72 frames, one layer at a time: 946 us; four groups 962; a thread walking all parts of a row,
