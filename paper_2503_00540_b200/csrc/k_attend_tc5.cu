@@ -879,9 +879,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
                 finish = *s_last != 0;
               }
             }
+            // every part is counted: nobody else touches the counter in this launch, and the next one finds it at zero (a CTA
+            // whose rows all lie beyond the unit's counts like any other)
+            if (finish && put && boss) *cnt = 0;
             if (finish && put && !warp_idle) {
               __threadfence();
-              if (boss) *cnt = 0;  // every part is counted: nobody else touches it in this launch
               // M = the maximum over the parts, weights 2^(m_k - M), numerators and denominator accumulated in part order: the
               // same arithmetic whichever worker came last
               const int own = fast ? worker_e - w_first : -1;  // (its own partial, where it wrote one, is read like the others)

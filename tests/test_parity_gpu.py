@@ -130,6 +130,27 @@ def test_units_cut_into_a_few_parts_are_finished_inside_the_kernel():
     g.close()
 
 
+def test_the_counters_of_joined_units_are_left_at_zero():
+    """80-token questions (160 rows: both CTAs of a pair) and a 40-token one beside them (80 rows: the second CTA has none), in
+    turns on one context: units are cut at other places in each launch, and a count left behind by one -- by the CTA without
+    rows too -- would let the next join parts that are not there yet."""
+    s = H.Shape(L=10, Hq=16, Hkv=8, Nf=100, T=28, W=4, k=16, seed=2503)
+    g = H.build_gpu(s, max_questions=2, max_q_tokens=120)
+    o = H.build_oracle(s)
+    q1, cu1 = H.questions(s, [80], device="cuda")
+    q2, cu2 = H.questions(s, [80, 40], device="cuda")
+    first = g.question(q1, cu1, s.k, s.T).clone()
+    ref = o.question(q1.cpu(), s.k, s.T)
+    idx = ref["idx"][:, None].contiguous().cuda()
+    H.assert_attention(g.question(q1, cu1, s.k, s.T, idx=idx), ref["out"], "80 tokens")
+    both = g.question(q2, cu2, s.k, s.T).clone()
+    for _ in range(4):
+        assert torch.equal(g.question(q1, cu1, s.k, s.T), first)
+        assert torch.equal(g.question(q2, cu2, s.k, s.T), both)
+    g.check_status()
+    g.close()
+
+
 def test_the_few_remainders_of_a_large_batch_are_cut_in_four():
     """15 questions of one CTA pair per unit and one with 24 rows more: a launch of pairs and one of single CTAs beside it,
     four whole CTAs for each of its 32 units, whose parts are joined in the kernel."""
