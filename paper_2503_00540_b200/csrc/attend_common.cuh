@@ -1,6 +1,6 @@
 // The decode-shaped attention kernel of step 5 (Eq. 3): the launch parameters and the decoding of a unit index.  A unit is
-// (layer, kv head, question); a launch covers units * steps steps -- a step is a context frame, or a tile of X's tokens --
-// cut into contiguous ranges of `per` steps per CTA.
+// (layer, kv head, question); a launch covers units * steps steps -- a step is one or several context frames, or a tile of X's
+// tokens -- cut into contiguous ranges of `per` steps per CTA.
 #pragma once
 
 #include "ptx_helpers.cuh"
@@ -27,14 +27,18 @@ struct TcParams {
   QBatch qb;
   int Hq, Hkv, G, Nf, Npad, ncf, MP, layer0;
   int early;         // the context table and its pages are complete whatever the kernels just before this launch do
-  int steps;         // steps of a unit: its context frames, then tiles of N_pad tokens of X
+  int F;             // frames of a step
+  int fsteps;        // steps of a unit: its context frames, F at a time ...
+  int steps;         // ... then tiles of F * N_pad tokens of X
   // test-only knobs (0 = off): iteration limit of the bounded waits, and the frame whose copy CTA 0 leaves out so that a
   // wait runs out with nothing in flight
   unsigned wait_limit;
   int skip_copy_entry;
   int part_slots;    // capacity of part_o / part_ml in 16-row parts
   int per;           // steps per CTA, when parts == 0
-  int parts;         // > 0: CTAs per unit, each with an even share of its steps
+  int parts;         // > 0: CTAs per unit (CTA k * units + u is part k of unit u); frame_parts of them share the unit's first
+  int frame_parts;   // `split` steps evenly, the last part has the rest of its steps (alone, or besides its share)
+  int split, units;
   long long total;   // units * steps
   float scale_log2;
 };
