@@ -31,9 +31,11 @@
 //   warp 3      second CTA of a pair: passes its tiles' arrivals on to the issuing CTA
 //   warp 3 (warp 1 in a pair's second CTA)   the next segment's Q tile (cp.async, double-buffered)
 //   warps 4-7, 8-11   softmax of the even / odd chunks, one thread per row (= TMEM lane), fp32
-// After set-up the service warpgroup shrinks to 72 registers per thread and the softmax warpgroups grow to 216
-// (setmaxnreg), so that a softmax thread holds a whole S row chunk: one TMEM load and two TMEM stores per chunk (a warp's
-// tcgen05.ld/st cost about 90 cycles each whatever their width).
+//   warps 12-15 (OUT)   the segments' results, so that the softmax warps go on with the next segment's chunks meanwhile; in
+//                       launches without them (one segment per worker, or short ones) the softmax warps put out the results
+// After set-up the service warpgroup shrinks to 72 (56 with output warps) registers per thread and the softmax warpgroups grow to
+// 216 (176) (setmaxnreg), so that a softmax thread holds a whole S row chunk: one or two TMEM loads and two TMEM stores per
+// chunk (a warp's tcgen05.ld/st cost about 90 cycles each whatever their width).
 //
 // The exponentials of a segment (the part of a unit in one range) take the row maximum of its first chunk as their
 // reference m: a softmax does not depend on m, and 2^(x - m) far above 1 loses nothing in fp32 or in bf16's exponent.
@@ -57,9 +59,18 @@ using namespace rekv_att;
 
 namespace {
 
-constexpr int TC_THREADS = 384;
-constexpr int SM_WARP0 = 4;                            // first softmax warp
-constexpr int REGS_SERVICE = 72, REGS_SOFTMAX = 216;   // 128 * service + 256 * softmax <= 384 * 168
+constexpr int SM_WARP0 = 4, OUT_WARP0 = 12;            // first softmax warp, first output warp
+// OUT: four more warps put out the segments' results, else the softmax warps do it themselves.
+// Registers per thread: 128 * service + 256 * softmax (+ 128 * output) <= threads * those at launch
+// One B200, us without / with output warps: 1800-frame question (units of 113 chunks) 262 / 254, Eq. 3 in full 240 / 228, 10-token
+// question 182 / 179, 16-question batch (63 chunks) 3160 / 3130; encoding step (units of 15 chunks) 254 / 259.
+constexpr int OUT_MIN_CHUNKS = 32;
+template <bool OUT>
+struct Warps {
+  static constexpr int THREADS = OUT ? 512 : 384;
+  static constexpr int REGS_SERVICE = OUT ? 56 : 72, REGS_SOFTMAX = OUT ? 176 : 216, REGS_OUT = 104;
+  static constexpr int OUT_WARPS = OUT ? 4 : 8, COLUMNS = OUT ? 128 : 64;   // columns of a row that an output thread puts out
+};
 constexpr int CHUNK = 128;                             // stream rows per chunk
 constexpr int S_BUFS = 3;                              // S/P buffers in tensor memory
 constexpr uint32_t TMEM_COLS = 512;                    // O [0,128), S/P [128,512)
@@ -87,13 +98,13 @@ constexpr uint32_t V_HALF = CHUNK * 128;
 
 // barrier slots (8 bytes each)
 constexpr int B_KFULL = 0, B_KEMPTY = 5, B_VFULL = 10, B_VEMPTY = 15, B_SFULL = 20, B_PREADY = 23, B_QFULL = 26,
-              B_QFREE = 28, B_OFULL = 30, B_OFREE = 31, B_MREADY = 32, B_LREADY = 33, B_COUNT = 34;
+              B_QFREE = 28, B_OFULL = 30, B_OFREE = 31, B_MREADY = 32, B_LREADY = 34, B_LFREE = 36, B_COUNT = 38;
 // small shared state after the barriers (bytes)
-constexpr uint32_t OFF_M = 8 * B_COUNT;               // float [128]: the segment's reference maxima
-constexpr uint32_t OFF_L = OFF_M + 512;               // float [2 parity][2 warpgroups][128]: row sums
-constexpr uint32_t OFF_REDO = OFF_L + 2048;           // u64: segments to run again
-constexpr uint32_t OFF_WORDS = OFF_REDO + 8;          // u32: tmem slot, abort, overflow marks [2], fast [2], last, bad, counter
-constexpr uint32_t SMALL_BYTES = OFF_WORDS + 40;
+constexpr uint32_t OFF_M = 8 * B_COUNT;               // float [2 parity][128]: the segment's reference maxima
+constexpr uint32_t OFF_L = OFF_M + 1024;              // float [2 parity][128]: row sums
+constexpr uint32_t OFF_REDO = OFF_L + 1024;           // u64: segments to run again
+constexpr uint32_t OFF_WORDS = OFF_REDO + 8;          // u32: tmem slot, abort, overflow marks [2], fast, last
+constexpr uint32_t SMALL_BYTES = OFF_WORDS + 24;
 constexpr size_t TC_SMEM = 2 * Q_TILE_BYTES + RING_BYTES + SMALL_BYTES;  // (the dynamic segment is 1024-byte aligned)
 static_assert(TC_SMEM <= 227 * 1024, "shared-memory plan of the attention kernel");
 
@@ -204,9 +215,25 @@ __device__ __forceinline__ void store_row_part(__nv_bfloat16* dst, const float* 
   }
 }
 
-template <int CG>
-__global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_constant__ Tc5Params p) {
+// the output warps meet; the conjunction of their values
+template <int THREADS>
+__device__ __forceinline__ bool out_and(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "barrier.cta.red.and.pred q, 1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)v), "n"(THREADS)
+      : "memory");
+  return r != 0;
+}
+
+template <int CG, bool OUT>
+__global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(const __grid_constant__ Tc5Params p) {
   using R = Ring<CG>;
+  using WP = Warps<OUT>;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = smem_raw;
   const uint32_t s_q = smem_u32(smem);                  // two Q tiles
@@ -219,16 +246,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
   const uint32_t s_bar = s_q + 2 * Q_TILE_BYTES + RING_BYTES;
   unsigned char* small = smem + 2 * Q_TILE_BYTES + RING_BYTES;
   volatile float* s_m = reinterpret_cast<volatile float*>(small + OFF_M);
-  volatile float* s_l = reinterpret_cast<volatile float*>(small + OFF_L);
+  float* s_l = reinterpret_cast<float*>(small + OFF_L);
   unsigned long long* s_redo = reinterpret_cast<unsigned long long*>(small + OFF_REDO);
   volatile uint32_t* s_words = reinterpret_cast<volatile uint32_t*>(small + OFF_WORDS);
   volatile uint32_t* s_tmem_slot = s_words;
   volatile uint32_t* s_abort = s_words + 1;
   volatile uint32_t* s_over = s_words + 2;   // [2] by segment parity: number (+ 1) of the last segment with an overflow
-  volatile uint32_t* s_fast = s_words + 4;   // [2] by segment parity: every other part of the unit is in place
-  volatile uint32_t* s_last = s_words + 6;
-  volatile uint32_t* s_bad = s_words + 7;    // a warp of this CTA did not write its part
-  volatile int* s_cnt_at = reinterpret_cast<volatile int*>(s_words + 8);
+  volatile uint32_t* s_fast = s_words + 4;   // every other part of the unit is in place
+  volatile uint32_t* s_last = s_words + 5;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
@@ -263,10 +288,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
       mbar_init(bar(B_QFREE + i), 1);
     }
     mbar_init(bar(B_OFULL), 1);
-    mbar_init(bar(B_OFREE), 8 * CG);
-    mbar_init(bar(B_MREADY), 4);
-    mbar_init(bar(B_LREADY), 8);
-    for (int i = 1; i < 8; ++i) s_words[i] = 0;
+    mbar_init(bar(B_OFREE), WP::OUT_WARPS * CG);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(bar(B_MREADY + i), 4);
+      mbar_init(bar(B_LREADY + i), 8);
+      mbar_init(bar(B_LFREE + i), WP::OUT_WARPS);
+    }
+    for (int i = 1; i < 6; ++i) s_words[i] = 0;
     *s_redo = 0ull;
     fence_barrier_init();
   }
@@ -282,7 +310,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
   const uint32_t tmem = *s_tmem_slot;
   // (With early_q the softmax warps load the first Q tile before their wait.)  No warp releases the next launch before its own
   // wait: one thread's release counts for its CTA, and the next launch may take what this one's predecessors wrote as complete.
-  const bool waits_later = p.early_q && warp >= SM_WARP0;
+  const bool loads_q = warp >= SM_WARP0 && warp < OUT_WARP0;
+  const bool waits_later = p.early_q && loads_q;
   if (!waits_later) {
     if (!p.second) grid_dep_wait();
     grid_dep_launch();
@@ -340,7 +369,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
     __syncwarp();
   };
 
-  if (warp >= SM_WARP0) {  // the first segment's Q
+  if (loads_q) {  // the first segment's Q
     load_q(decode_seg<CG>(p, range0, range1), 0, (warp - SM_WARP0) * 16, std::integral_constant<int, 8>{});
     if (lane == 0) mbar_arrive(bar(B_QFULL));
     if (waits_later) {
@@ -349,11 +378,165 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
     }
   }
 
+  // ================= a segment's result, one thread per row (and half of its columns without output warps) =================
+  // With output warps (OUT) the softmax warps go on with the next segment's chunks meanwhile.
+  auto result = [&](const Seg& s, int si, int pos, uint32_t segn, bool safe, bool& ok, int part) {
+    const uint32_t par = segn & 1u;
+    int row = ((warp & 3) << 5) | lane;
+    if constexpr (!OUT) asm volatile("" : "+r"(row));   // (see the call)
+    const int rr = s.m0 + (int)rank * 128 + row;
+    const bool valid = rr < s.rows_q;
+    const bool warp_idle = s.m0 + (int)rank * 128 + ((warp & 3) << 5) >= s.rows_q;
+    const int n = rr / p.G, j = rr - n * p.G;
+    const bool cut = s.I0 != 0 || s.I1 != s.nch;
+    const bool boss = warp == (OUT ? OUT_WARP0 : SM_WARP0) && lane == 0;
+    const int w_first = cut ? worker_of(p, s.uc0) : worker;
+    const int n_parts = cut ? worker_of(p, s.uc0 + s.nch - 1) - w_first + 1 : 1;
+    int* cnt = p.unit_cnt + w_first * CG + (int)rank;
+    if (ok) ok = wait(B_LREADY + par, (segn >> 1) & 1u);
+    const float m_own = s_m[par * 128 + row], l_own = s_l[par * 128 + row] * TRUNC_GAIN_INV;  // (the sums are of scaled values)
+    const bool over = s_over[par] == segn + 1;
+    if (boss && cut && p.merge_inside) *s_fast = __ldcg(cnt) == n_parts - 1;
+    __syncwarp();
+    if (OUT && lane == 0) mbar_arrive(bar(B_LFREE + par));
+    if (ok) ok = wait(B_OFULL, segn & 1u);
+    // (a wait that ran out ran out for all warps that meet below)
+    if (OUT || (cut && p.merge_inside)) ok = out_and<32 * WP::OUT_WARPS>(ok);
+    bool put = ok;
+    if (ok && !safe && over) {
+      put = false;
+      if (boss) {
+        atomicOr(s_redo, redo_bit(si, s, pos));
+        if (CG == 2) fence_cluster();  // (the barrier at the end of the pass does not publish it)
+      }
+    }
+    if (safe && !(redo_mask(false) & redo_bit(si, s, pos))) put = false;  // (the pair's other CTA asked for it)
+    // O, 32 of the row's columns at a time.  The next segment's first P V waits until it has been read.
+    const uint32_t t_o = tmem + ((uint32_t)((warp & 3) << 5) << 16);
+    const int col0 = part * WP::COLUMNS;
+    auto load_o = [&](int c0, float (&o)[32]) {
+      uint32_t ou[32];
+      tmem_ld32(t_o + (uint32_t)c0, ou);
+      tmem_wait_ld32(ou);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) o[i] = __uint_as_float(ou[i]);
+    };
+    auto o_free = [&]() {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) arrive_lead(B_OFREE);
+    };
+    if (put) tc_fence_after();
+    __nv_bfloat16* dst = p.out + ((s.q_row0 + (valid ? n : 0)) * p.Hq + s.g * p.G + (valid ? j : 0)) * 128;
+    if (!cut) {
+      if (put && !warp_idle) {
+        const float inv = l_own > 0.f ? 1.f / l_own : 0.f;
+#pragma unroll 1
+        for (int c0 = col0; c0 < col0 + WP::COLUMNS; c0 += 32) {
+          float o[32];
+          load_o(c0, o);
+          if (valid) store_row_part(dst + c0, o, inv);
+        }
+      }
+      o_free();
+    } else {
+      // a part of a unit: slot 2 w + 1 for a unit that starts in worker w's range, 2 w for one that started before
+      const int slot = (2 * worker + (s.I0 == 0 ? 1 : 0)) * CG + (int)rank;
+      const bool slot_ok = REKV_CHECK(slot >= 0 && slot < p.part_slots, p.status, 32);  // (checks build)
+      const bool fast = p.merge_inside && *s_fast != 0;  // every other part is counted: no partial of its own
+      bool finish = fast;
+      if (!fast) {
+        if (put && !warp_idle) {
+#pragma unroll 1
+          for (int c0 = col0; c0 < col0 + WP::COLUMNS; c0 += 32) {
+            float o[32];
+            load_o(c0, o);
+            float4* po = p.part_o + ((long long)slot * 32 + (c0 >> 2)) * 128 + row;
+            if (valid && slot_ok) {
+#pragma unroll
+              for (int v = 0; v < 8; ++v)
+                po[(long long)v * 128] = make_float4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
+            }
+          }
+          if (part == 0 && valid && slot_ok) p.part_ml[(long long)slot * 128 + row] = make_float2(m_own, l_own);
+        }
+        o_free();
+        if (p.merge_inside) {  // publish, count, and join the parts if this one was the last
+          __threadfence();
+          out_and<32 * WP::OUT_WARPS>(true);
+          if (boss) *s_last = put && atomicAdd(cnt, 1) == n_parts - 1;
+          out_and<32 * WP::OUT_WARPS>(true);
+          finish = *s_last != 0;
+        }
+      }
+      // every part is counted: nobody else touches the counter in this launch, and the next one finds it at zero (a CTA
+      // whose rows all lie beyond the unit's counts like any other)
+      if (finish && put && boss) *cnt = 0;
+      if (finish && put && !warp_idle) {
+        __threadfence();
+        // M = the maximum over the parts, weights 2^(m_k - M), numerators and denominator accumulated in part order: the
+        // same arithmetic whichever worker came last
+        const int own = fast ? worker - w_first : -1;  // (its own partial, where it wrote one, is read like the others)
+        float2 ml[MAX_PARTS_INSIDE];
+        float M = -1e30f;
+#pragma unroll
+        for (int k = 0; k < MAX_PARTS_INSIDE; ++k) {
+          ml[k] = make_float2(-INFINITY, 0.f);
+          if (k < n_parts) {
+            const int sk = (2 * (w_first + k) + (k == 0 ? 1 : 0)) * CG + (int)rank;
+            ml[k] = k == own ? make_float2(m_own, l_own) : __ldcg(p.part_ml + (long long)sk * 128 + row);
+            M = fmaxf(M, ml[k].x);
+          }
+        }
+        float den = 0.f;
+#pragma unroll
+        for (int k = 0; k < MAX_PARTS_INSIDE; ++k) {
+          ml[k].x = ex2(ml[k].x - M);
+          den = fmaf(ml[k].x, ml[k].y, den);
+        }
+        const float inv = den > 0.f ? 1.f / den : 0.f;
+#pragma unroll 1
+        for (int c0 = col0; c0 < col0 + WP::COLUMNS; c0 += 32) {
+          float acc[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+#pragma unroll
+          for (int k = 0; k < MAX_PARTS_INSIDE; ++k)
+            if (k < n_parts) {
+              const float w = ml[k].x;
+              if (k == own) {
+                float o[32];
+                load_o(c0, o);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) acc[i] = fmaf(w, o[i], acc[i]);
+              } else {
+                const int sk = (2 * (w_first + k) + (k == 0 ? 1 : 0)) * CG + (int)rank;
+                const float4* po = p.part_o + ((long long)sk * 32 + (c0 >> 2)) * 128 + row;
+                float4 x[8];
+#pragma unroll
+                for (int v = 0; v < 8; ++v) x[v] = __ldcg(po + (long long)v * 128);
+#pragma unroll
+                for (int v = 0; v < 8; ++v) {
+                  acc[4 * v] = fmaf(w, x[v].x, acc[4 * v]);
+                  acc[4 * v + 1] = fmaf(w, x[v].y, acc[4 * v + 1]);
+                  acc[4 * v + 2] = fmaf(w, x[v].z, acc[4 * v + 2]);
+                  acc[4 * v + 3] = fmaf(w, x[v].w, acc[4 * v + 3]);
+                }
+              }
+            }
+          if (valid) store_row_part(dst + c0, acc, inv);
+        }
+      }
+      if (fast) o_free();
+      if (p.merge_inside) out_and<32 * WP::OUT_WARPS>(true);  // (s_fast and s_last have been read)
+    }
+  };
+
   // The roles run the same range loop with the role as a compile-time constant, so that each side of the register
   // reallocation below is compiled against its own register budget.  Pass 0 runs the whole range; pass 1, only
   // if some row's reference maximum was too low, runs the marked segments again.
   auto run = [&](auto role) {
-    constexpr bool SOFTMAX = decltype(role)::value;
+    constexpr int ROLE = decltype(role)::value;  // 0: copies and products, 1: softmax, 2: output
     uint32_t t = 0;        // chunks so far (both passes): ring slots and barrier phases follow from it
     uint32_t segn = 0;     // segments so far
     uint32_t issued = 0, phase = 0;  // producers: tiles whose copies are on their way; parity of the ring's current round
@@ -366,8 +549,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
       uint32_t t_base = t;                                  // first chunk of the pass
       uint32_t pend0 = 0, pend1 = 0, pend2 = 0;             // MMA issuer: P V of the chunks t-3, t-2, t-1
       int pos = range0;
+      // (without output warps the softmax warps meet at the cut segments of launches that join them: a warp whose wait ran out goes
+      // through the rest of the range without waiting, so that it is missing at no such meeting)
+      const bool meets = ROLE == 1 && !OUT && p.merge_inside != 0;
 #pragma unroll 1
-      for (int si = 0; pos < range1 && ok; ++si) {
+      for (int si = 0; pos < range1 && (ok || meets); ++si) {
         const Seg s = decode_seg<CG>(p, pos, range1);
         const int nseg = s.I1 - s.I0;
         if (safe && !(redo_mask(true) & redo_bit(si, s, pos))) {
@@ -378,7 +564,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
         const int R_end = stream_rows(p, s.nx);
         const int x_off = s.nx ? ((p.sb.cu[s.qi] + 7) & ~7) + 8 * s.qi : 0;  // X's first staged row
 
-        if constexpr (!SOFTMAX) {
+        if constexpr (ROLE == 0) {
           auto produce = [&](auto which) {
             // ================= producers =================
             constexpr int kv = decltype(which)::value;
@@ -590,8 +776,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
               if (lane == 0) mbar_arrive_n(bar(B_QFULL + par), 8);
             }
           }
-        } else {
-          // ================= softmax + output, one thread per row =================
+        } else if constexpr (ROLE == 1) {
+          // ================= softmax, one thread per row =================
           const int wg = (warp - SM_WARP0) >> 2;           // this warpgroup takes the chunks with t % 2 == wg
           const uint32_t lane_base = (uint32_t)((warp & 3) << 5) << 16;
           const int row = ((warp & 3) << 5) | lane;
@@ -602,14 +788,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
           const int first_wg = safe ? 0 : (int)(t & 1u);
           const int rows_in = s.nx ? Rc : R_end;           // chunks that end at or before this row need no tail mask
           const uint32_t gap_bits = p.Ns != p.Nf ? (0xFFu << (p.Nf & 7)) & 0xFFu : 0u;  // gap columns of an 8-row group
-          if (warp == SM_WARP0) {  // where the segment's unit counts its parts, if it is one of several (see the result)
-            const bool counts = p.merge_inside && (s.I0 != 0 || s.I1 != s.nch);
-            if (lane == 0) *s_cnt_at = counts ? worker_of(p, s.uc0) * CG + (int)rank : -1;
-            __syncwarp();
-          }
-          int seen = -1;                                   // parts counted when this warp's last chunk began
           float m_used = 0.f, l_sum = 0.f;
           bool over = false, have_m = false;
+          // the state of the segment before the last has been read: its places and barriers are this one's
+          // (without output warps this warpgroup has read it itself, after the other one was done with it)
+          if (OUT && segn >= 2) ok = wait(B_LFREE + par, ((segn >> 1) - 1) & 1u);
           int i0 = wg ^ first_wg;
           if (safe && wg != 0) i0 = nseg;
           const int istep = safe ? 1 : 2;
@@ -633,14 +816,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
               tc_fence_before();
               __syncwarp();
               if (lane == 0) {
-                if (i == 0) mbar_arrive(bar(B_MREADY));
+                if (i == 0) mbar_arrive(bar(B_MREADY + par));
                 arrive_lead(B_PREADY + buf);
               }
               continue;
             }
             const float NEG_INF = -INFINITY;
             uint32_t sv[128];
-            tmem_ld128(t_s, sv);
+            if constexpr (OUT) {  // (an instruction's registers must fit those at launch)
+              tmem_ld64<0>(t_s, sv);
+              tmem_ld64<64>(t_s + 64, sv);
+            } else {
+              tmem_ld128(t_s, sv);
+            }
             tmem_wait_ld128(sv);
             // Columns without a token.  N_s is a multiple of 8 and so is every frame's start, so a frame's gap is the end
             // of one aligned 8-column group, with the same bits in every frame: the groups that have one are found by
@@ -730,15 +918,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
             if (i == 0) {  // the segment's first chunk: its row maximum becomes the reference of both warpgroups
               m_used = fmaxf(row_max(), -1e30f);  // (a row that sees nothing keeps a finite reference)
               have_m = true;
-              s_m[row] = m_used;
+              s_m[par * 128 + row] = m_used;
+              s_l[par * 128 + row] = 0.f;
               __syncwarp();
-              if (lane == 0) mbar_arrive(bar(B_MREADY));
+              if (lane == 0) mbar_arrive(bar(B_MREADY + par));
             } else if (!have_m) {
-              if (!wait(B_MREADY, segn & 1u)) {
+              if (!wait(B_MREADY + par, (segn >> 1) & 1u)) {
                 ok = false;
                 break;
               }
-              m_used = s_m[row];
+              m_used = s_m[par * 128 + row];
               have_m = true;
             }
             if (safe && i > 0) {
@@ -761,7 +950,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
                 }
               }
             }
-            if (warp == SM_WARP0 && i + istep >= nseg && *s_cnt_at >= 0) seen = __ldcg(p.unit_cnt + *s_cnt_at);
             const float cs = exp_pass();
             // (a logit more than 60 octaves above the reference: the segment has to be run again)
             if (__any_sync(0xffffffffu, !(cs < RESCALE_SUM_LIMIT))) over = true;
@@ -772,170 +960,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
             if (lane == 0) arrive_lead(B_PREADY + buf);
           }
 
-          // ---- the segment's result -------------------------------------------------------------------
-          // (worked out again, from values the compiler cannot trace back, instead of being held in registers -- or in local
-          // memory -- through the chunk loop, as everything that is constant over the segments otherwise would be)
-          int pos_e = pos, row_e = row, wg_e = wg, worker_e = worker, rank_e = (int)rank;
-          asm volatile("" : "+r"(pos_e), "+r"(row_e), "+r"(wg_e), "+r"(worker_e), "+r"(rank_e));
-          const Seg e = decode_seg<CG>(p, pos_e, range1);
-          const int rr = e.m0 + rank_e * 128 + row_e;
-          const bool valid = rr < e.rows_q;
-          const int n = rr / p.G, j = rr - n * p.G;
-          const bool cut = e.I0 != 0 || e.I1 != e.nch;
-          const bool boss = warp == SM_WARP0 && lane == 0;
-          const int w_first = cut ? worker_of(p, e.uc0) : worker_e;
-          const int n_parts = cut ? worker_of(p, e.uc0 + e.nch - 1) - w_first + 1 : 1;
-          int* cnt = p.unit_cnt + w_first * CG + rank_e;
-          // (s_m is read before this segment's B_LREADY completes, so that the next segment may write it; after a segment
-          // that was run again, by warpgroup 0 alone, its final reference travels in the other warpgroup's place)
-          if (ok && !safe && !have_m && !warp_idle) {
-            ok = wait(B_MREADY, segn & 1u);
-            m_used = s_m[row_e];
+          // the row's sum and reference for the output warps (two addends, whose order does not matter; a segment that is run
+          // again is warpgroup 0's alone)
+          if (!warp_idle) {
+            if (safe && wg == 0) {
+              s_l[par * 128 + row] = l_sum;
+              s_m[par * 128 + row] = m_used;
+            } else if (have_m) {
+              atomicAdd(s_l + par * 128 + row, l_sum);
+            }
+            if (over) s_over[par] = segn + 1;
           }
-          if (!safe)
-            s_l[(par * 2 + wg_e) * 128 + row_e] = l_sum;
-          else if (wg_e == 0) {
-            s_l[par * 256 + row_e] = l_sum;
-            s_l[par * 256 + 128 + row_e] = m_used;
-          }
-          if (over && !warp_idle) s_over[par] = segn + 1;
-          if (boss && cut && p.merge_inside) s_fast[par] = (seen >= 0 ? seen : __ldcg(cnt)) == n_parts - 1;
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar(B_LREADY));
-          if (ok) ok = wait(B_LREADY, segn & 1u);
-          if (ok) ok = wait(B_OFULL, segn & 1u);
-          bool put = ok;
-          if (ok && !safe && s_over[par] == segn + 1) {
-            put = false;
-            if (boss) {
-              atomicOr(s_redo, redo_bit(si, e, pos));
-              if (CG == 2) fence_cluster();  // (the barrier at the end of the pass does not publish it)
-            }
+          if (lane == 0) mbar_arrive(bar(B_LREADY + par));
+          if constexpr (!OUT) {
+            // (worked out again, from values the compiler cannot trace back, instead of being held in registers -- or in local
+            // memory -- through the chunk loop, as everything that is constant over the segments otherwise would be)
+            int pos_e = pos, wg_e = wg;
+            asm volatile("" : "+r"(pos_e), "+r"(wg_e));
+            result(decode_seg<CG>(p, pos_e, range1), si, pos_e, segn, safe, ok, wg_e);
           }
-          if (safe && !(redo_mask(false) & redo_bit(si, e, pos))) put = false;  // (the pair's other CTA asked for it)
-          const float x_l = s_l[par * 256 + 128 + row_e];
-          const float m_own = safe ? x_l : m_used;
-          const float l_own = (s_l[par * 256 + row_e] + (safe ? 0.f : x_l)) * TRUNC_GAIN_INV;  // (the sums are of scaled values)
-          // O: this warpgroup's half of the row's columns, 32 at a time (32 registers live, not 64: the chunk loop's
-          // registers are what is left of the budget).  The next segment's first P V waits until it has been read.
-          const uint32_t t_o = tmem + lane_base + 64u * wg_e;
-          auto load_o = [&](int hf, float (&o)[32]) {
-            uint32_t ou[32];
-            tmem_ld32(t_o + 32u * hf, ou);
-            tmem_wait_ld32(ou);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] = __uint_as_float(ou[i]);
-          };
-          auto o_free = [&]() {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) arrive_lead(B_OFREE);
-          };
-          if (put) tc_fence_after();
-          __nv_bfloat16* dst = p.out + ((e.q_row0 + (valid ? n : 0)) * p.Hq + e.g * p.G + (valid ? j : 0)) * 128 + 64 * wg_e;
-          if (!cut) {
-            if (put && !warp_idle) {
-              const float inv = l_own > 0.f ? 1.f / l_own : 0.f;
-#pragma unroll 1
-              for (int hf = 0; hf < 2; ++hf) {
-                float o[32];
-                load_o(hf, o);
-                if (valid) store_row_part(dst + 32 * hf, o, inv);
-              }
-            }
-            o_free();
-          } else {
-            // a part of a unit: slot 2 w + 1 for a unit that starts in worker w's range, 2 w for one that started before
-            const int slot = (2 * worker_e + (e.I0 == 0 ? 1 : 0)) * CG + rank_e;
-            const bool slot_ok = REKV_CHECK(slot >= 0 && slot < p.part_slots, p.status, 32);  // (checks build)
-            // (every warp meets here, after a wait that ran out too: s_fast is then the same for all of them)
-            if (p.merge_inside) asm volatile("bar.sync 1, 256;" ::: "memory");
-            const bool fast = p.merge_inside && s_fast[par] != 0;  // every other part is counted: no partial of its own
-            bool finish = fast;
-            if (!fast) {
-              if (put && !warp_idle) {
-#pragma unroll 1
-                for (int hf = 0; hf < 2; ++hf) {
-                  float o[32];
-                  load_o(hf, o);
-                  float4* po = p.part_o + ((long long)slot * 32 + wg_e * 16 + hf * 8) * 128 + row_e;
-                  if (valid && slot_ok) {
-#pragma unroll
-                    for (int v = 0; v < 8; ++v)
-                      po[(long long)v * 128] = make_float4(o[4 * v], o[4 * v + 1], o[4 * v + 2], o[4 * v + 3]);
-                  }
-                }
-                if (wg_e == 0 && valid && slot_ok) p.part_ml[(long long)slot * 128 + row_e] = make_float2(m_own, l_own);
-              }
-              o_free();
-              if (p.merge_inside) {
-                // publish, count, and join the parts if this one was the last.  All eight warps meet here whether or not
-                // their rows got written (a wait that ran out): then the part is not counted.
-                if (!ok) *s_bad = 1;
-                __threadfence();
-                asm volatile("bar.sync 1, 256;" ::: "memory");
-                if (boss) *s_last = put && !*s_bad && atomicAdd(cnt, 1) == n_parts - 1;
-                asm volatile("bar.sync 1, 256;" ::: "memory");
-                finish = *s_last != 0;
-              }
-            }
-            // every part is counted: nobody else touches the counter in this launch, and the next one finds it at zero (a CTA
-            // whose rows all lie beyond the unit's counts like any other)
-            if (finish && put && boss) *cnt = 0;
-            if (finish && put && !warp_idle) {
-              __threadfence();
-              // M = the maximum over the parts, weights 2^(m_k - M), numerators and denominator accumulated in part order: the
-              // same arithmetic whichever worker came last
-              const int own = fast ? worker_e - w_first : -1;  // (its own partial, where it wrote one, is read like the others)
-              float2 ml[MAX_PARTS_INSIDE];
-              float M = -1e30f;
-#pragma unroll
-              for (int k = 0; k < MAX_PARTS_INSIDE; ++k) {
-                ml[k] = make_float2(-INFINITY, 0.f);
-                if (k < n_parts) {
-                  const int sk = (2 * (w_first + k) + (k == 0 ? 1 : 0)) * CG + rank_e;
-                  ml[k] = k == own ? make_float2(m_own, l_own) : __ldcg(p.part_ml + (long long)sk * 128 + row_e);
-                  M = fmaxf(M, ml[k].x);
-                }
-              }
-              float den = 0.f;
-#pragma unroll
-              for (int k = 0; k < MAX_PARTS_INSIDE; ++k) {
-                ml[k].x = ex2(ml[k].x - M);
-                den = fmaf(ml[k].x, ml[k].y, den);
-              }
-              const float inv = den > 0.f ? 1.f / den : 0.f;
-#pragma unroll 1
-              for (int hf = 0; hf < 2; ++hf) {
-                float o[32], acc[32];
-                if (fast) load_o(hf, o);
-#pragma unroll
-                for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-#pragma unroll
-                for (int k = 0; k < MAX_PARTS_INSIDE; ++k)
-                  if (k < n_parts) {
-                    const float w = ml[k].x;
-                    if (k == own) {
-#pragma unroll
-                      for (int i = 0; i < 32; ++i) acc[i] = fmaf(w, o[i], acc[i]);
-                    } else {
-                      const int sk = (2 * (w_first + k) + (k == 0 ? 1 : 0)) * CG + rank_e;
-                      const float4* po = p.part_o + ((long long)sk * 32 + wg_e * 16 + hf * 8) * 128 + row_e;
-#pragma unroll
-                      for (int v = 0; v < 8; ++v) {
-                        const float4 x = __ldcg(po + (long long)v * 128);
-                        acc[4 * v] = fmaf(w, x.x, acc[4 * v]);
-                        acc[4 * v + 1] = fmaf(w, x.y, acc[4 * v + 1]);
-                        acc[4 * v + 2] = fmaf(w, x.z, acc[4 * v + 2]);
-                        acc[4 * v + 3] = fmaf(w, x.w, acc[4 * v + 3]);
-                      }
-                    }
-                  }
-                if (valid) store_row_part(dst + 32 * hf, acc, inv);
-              }
-            }
-            if (fast) o_free();
-          }
+        } else {
+          result(s, si, pos, segn, safe, ok, 0);
         }
         t += (uint32_t)nseg;
         ++segn;
@@ -951,7 +997,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
         if (redo_mask(true) == 0ull || *s_abort) break;
       }
     }
-    if constexpr (!SOFTMAX) {
+    if constexpr (ROLE == 0) {
       // A CTA that gives up must not return while copies into its shared memory are still on their way: the producers
       // wait (bounded) for the tiles they have issued and nobody consumed -- at most the rings' depth.
       if (*s_abort && (warp == 0 || warp == 2)) {
@@ -963,11 +1009,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) attend_tc5_kernel(const __grid_
     }
   };
   if (warp < SM_WARP0) {
-    reg_dealloc<REGS_SERVICE>();
-    run(std::false_type{});
+    reg_dealloc<WP::REGS_SERVICE>();
+    run(std::integral_constant<int, 0>{});
+  } else if (warp < OUT_WARP0) {
+    reg_alloc<WP::REGS_SOFTMAX>();
+    run(std::integral_constant<int, 1>{});
   } else {
-    reg_alloc<REGS_SOFTMAX>();
-    run(std::true_type{});
+    if constexpr (OUT) {
+      reg_dealloc<WP::REGS_OUT>();
+      run(std::integral_constant<int, 2>{});
+    }
   }
 
   __syncwarp();
@@ -1078,11 +1129,11 @@ __global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __g
   *reinterpret_cast<uint2*>(p.out + ((((long long)l * p.qb.sumNq + p.qb.cu[qi] + n) * p.Hq + g * p.G + j) * 128 + quad * 4)) = packed;
 }
 
-template <int CG>
+template <int CG, bool OUT>
 cudaError_t prepare_tc5() {  // the kernel's shared-memory limit, once per device
   static PerDeviceOnce attr;
   return attr.run([] {
-    return cudaFuncSetAttribute(attend_tc5_kernel<CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
+    return cudaFuncSetAttribute(attend_tc5_kernel<CG, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM);
   });
 }
 
@@ -1098,7 +1149,7 @@ int max_workers() {
   if (CG == 2) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * n);
-    cfg.blockDim = dim3(TC_THREADS);
+    cfg.blockDim = dim3(Warps<true>::THREADS);
     cfg.dynamicSmemBytes = TC_SMEM;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1107,7 +1158,7 @@ int max_workers() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int m = 0;
-    if (prepare_tc5<CG>() == cudaSuccess && cudaOccupancyMaxActiveClusters(&m, attend_tc5_kernel<CG>, &cfg) == cudaSuccess && m > 0)
+    if (prepare_tc5<CG, true>() == cudaSuccess && cudaOccupancyMaxActiveClusters(&m, attend_tc5_kernel<CG, true>, &cfg) == cudaSuccess && m > 0)
       n = std::min(n, m);
     else
       cudaGetLastError();
@@ -1118,8 +1169,6 @@ int max_workers() {
 
 template <int CG>
 cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
-  cudaError_t e = prepare_tc5<CG>();
-  if (e != cudaSuccess) return e;
   p.per_lh = 0;
   int blocks = 0, max_ch = 1;
   bool equal = true;  // every unit has max_ch chunks
@@ -1139,7 +1188,9 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
   p.merge_inside = plan.merge_inside;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(p.W * CG));
-  cfg.blockDim = dim3(TC_THREADS);
+  // output warps where a worker's range has several segments, and long ones
+  const bool out = p.W < p.nl * p.Hkv * blocks && max_ch >= OUT_MIN_CHUNKS;
+  cfg.blockDim = dim3(out ? Warps<true>::THREADS : Warps<false>::THREADS);
   cfg.dynamicSmemBytes = TC_SMEM;
   cfg.stream = st;
   cudaLaunchAttribute at[2];
@@ -1151,7 +1202,8 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
   cfg.attrs = at;
   cfg.numAttrs = 2;
   if (timed && !p.second) cudaEventRecord(c->ev_t0, st);
-  e = cudaLaunchKernelEx(&cfg, attend_tc5_kernel<CG>, p);
+  cudaError_t e = out ? prepare_tc5<CG, true>() : prepare_tc5<CG, false>();
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, out ? attend_tc5_kernel<CG, true> : attend_tc5_kernel<CG, false>, p);
   if (e != cudaSuccess) return e;
   c->launches += 1;
   if (timed) {

@@ -347,6 +347,14 @@ __device__ __forceinline__ void tmem_ld128(uint32_t taddr, uint32_t (&r)[128]) {
                : "r"(taddr)
                : "memory");
 }
+// half of it: columns H .. H + 63 of the 128 registers
+template <int H>
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, uint32_t (&r)[128]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
+               : "=r"(r[H + 0]), "=r"(r[H + 1]), "=r"(r[H + 2]), "=r"(r[H + 3]), "=r"(r[H + 4]), "=r"(r[H + 5]), "=r"(r[H + 6]), "=r"(r[H + 7]), "=r"(r[H + 8]), "=r"(r[H + 9]), "=r"(r[H + 10]), "=r"(r[H + 11]), "=r"(r[H + 12]), "=r"(r[H + 13]), "=r"(r[H + 14]), "=r"(r[H + 15]), "=r"(r[H + 16]), "=r"(r[H + 17]), "=r"(r[H + 18]), "=r"(r[H + 19]), "=r"(r[H + 20]), "=r"(r[H + 21]), "=r"(r[H + 22]), "=r"(r[H + 23]), "=r"(r[H + 24]), "=r"(r[H + 25]), "=r"(r[H + 26]), "=r"(r[H + 27]), "=r"(r[H + 28]), "=r"(r[H + 29]), "=r"(r[H + 30]), "=r"(r[H + 31]), "=r"(r[H + 32]), "=r"(r[H + 33]), "=r"(r[H + 34]), "=r"(r[H + 35]), "=r"(r[H + 36]), "=r"(r[H + 37]), "=r"(r[H + 38]), "=r"(r[H + 39]), "=r"(r[H + 40]), "=r"(r[H + 41]), "=r"(r[H + 42]), "=r"(r[H + 43]), "=r"(r[H + 44]), "=r"(r[H + 45]), "=r"(r[H + 46]), "=r"(r[H + 47]), "=r"(r[H + 48]), "=r"(r[H + 49]), "=r"(r[H + 50]), "=r"(r[H + 51]), "=r"(r[H + 52]), "=r"(r[H + 53]), "=r"(r[H + 54]), "=r"(r[H + 55]), "=r"(r[H + 56]), "=r"(r[H + 57]), "=r"(r[H + 58]), "=r"(r[H + 59]), "=r"(r[H + 60]), "=r"(r[H + 61]), "=r"(r[H + 62]), "=r"(r[H + 63])
+               : "r"(taddr)
+               : "memory");
+}
 __device__ __forceinline__ void tmem_wait_ld128(uint32_t (&r)[128]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]), "+r"(r[32]), "+r"(r[33]), "+r"(r[34]), "+r"(r[35]), "+r"(r[36]), "+r"(r[37]), "+r"(r[38]), "+r"(r[39]), "+r"(r[40]), "+r"(r[41]), "+r"(r[42]), "+r"(r[43]), "+r"(r[44]), "+r"(r[45]), "+r"(r[46]), "+r"(r[47]), "+r"(r[48]), "+r"(r[49]), "+r"(r[50]), "+r"(r[51]), "+r"(r[52]), "+r"(r[53]), "+r"(r[54]), "+r"(r[55]), "+r"(r[56]), "+r"(r[57]), "+r"(r[58]), "+r"(r[59]), "+r"(r[60]), "+r"(r[61]), "+r"(r[62]), "+r"(r[63]), "+r"(r[64]), "+r"(r[65]), "+r"(r[66]), "+r"(r[67]), "+r"(r[68]), "+r"(r[69]), "+r"(r[70]), "+r"(r[71]), "+r"(r[72]), "+r"(r[73]), "+r"(r[74]), "+r"(r[75]), "+r"(r[76]), "+r"(r[77]), "+r"(r[78]), "+r"(r[79]), "+r"(r[80]), "+r"(r[81]), "+r"(r[82]), "+r"(r[83]), "+r"(r[84]), "+r"(r[85]), "+r"(r[86]), "+r"(r[87]), "+r"(r[88]), "+r"(r[89]), "+r"(r[90]), "+r"(r[91]), "+r"(r[92]), "+r"(r[93]), "+r"(r[94]), "+r"(r[95]), "+r"(r[96]), "+r"(r[97]), "+r"(r[98]), "+r"(r[99]), "+r"(r[100]), "+r"(r[101]), "+r"(r[102]), "+r"(r[103]), "+r"(r[104]), "+r"(r[105]), "+r"(r[106]), "+r"(r[107]), "+r"(r[108]), "+r"(r[109]), "+r"(r[110]), "+r"(r[111]), "+r"(r[112]), "+r"(r[113]), "+r"(r[114]), "+r"(r[115]), "+r"(r[116]), "+r"(r[117]), "+r"(r[118]), "+r"(r[119]), "+r"(r[120]), "+r"(r[121]), "+r"(r[122]), "+r"(r[123]), "+r"(r[124]), "+r"(r[125]), "+r"(r[126]), "+r"(r[127])

@@ -360,3 +360,34 @@ def test_logits_far_above_the_first_chunk_raise_the_reference_maximum(n_tokens):
     # the big logits are 2.0 * 2.5 * 128 / sqrt(128) = 56.6 nats = 81.6 octaves above the others' (about 0)
     H.assert_attention(out, ref["out"], "attention with a late, very large logit")
     g.close()
+
+
+@pytest.mark.parametrize("late", [False, True], ids=["ordinary", "late_large_logits"])
+@pytest.mark.parametrize("L,n_tokens", [(20, 16), (10, 80), (10, 140)])
+def test_results_put_out_while_the_next_segment_goes_on(L, n_tokens, late):
+    """Units of 34 chunks, more of them than workers: four warps of their own put out a segment's result (whole, and parts that
+    are joined) while the softmax warps work on the next one.  16 tokens: single CTAs; 80: pairs, their second CTA a quarter
+    full; 140: pairs and a second launch for the remaining rows.  With late large logits every segment that holds the
+    last frame's first tokens is run again."""
+    s = H.Shape(L=L, Hq=16, Hkv=8, Nf=80, T=56, W=2, k=52, seed=7)
+    g = rekv.ReKV(s.L, s.Hq, s.Hkv, s.D, s.Nf, s.T, s.W, max_q_tokens=n_tokens, max_topk=s.k)
+    o = orc.OracleCache(s.L, s.Hq, s.Hkv, s.D, s.Nf, s.W)
+    gen = torch.Generator().manual_seed(11)
+    sign = (torch.randint(0, 2, (s.D,), generator=gen) * 2 - 1).float()
+    for f in range(s.T):
+        k = ((0.1 if late else 1.0) * torch.randn(s.L, s.Nf, s.Hkv, s.D, generator=gen)).to(torch.bfloat16)
+        v = torch.randn(s.L, s.Nf, s.Hkv, s.D, generator=gen).to(torch.bfloat16)
+        if late and f == s.T - 1:
+            k[:, 5:40] = (2.5 * sign).to(torch.bfloat16)
+        assert g.append_frame(k.cuda(), v.cuda()) == f
+        o.append(k, v)
+    if late:
+        q = (2.0 * sign).to(torch.bfloat16).expand(s.L, n_tokens, s.Hq, s.D).contiguous()
+    else:
+        q = torch.randn(s.L, n_tokens, s.Hq, s.D, generator=gen).to(torch.bfloat16)
+    ref = o.question(q, s.k, s.T)
+    for _ in range(2):  # (the second time on counters that the first one left behind)
+        out = g.question(q.cuda(), [0, n_tokens], s.k, s.T, idx=ref["idx"][:, None].contiguous().cuda())
+        g.check_status()
+        H.assert_attention(out, ref["out"], "attention")
+    g.close()
