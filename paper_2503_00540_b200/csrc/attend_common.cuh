@@ -19,6 +19,7 @@ struct TcParams {
   // rotary embedding: (cos, sin) per [position][64], or null; context token j is at position j when rot_ctx is set (else it
   // is not rotated), token s of X at pos_x + s
   const float2* tab;
+  const float2* tab_c;   // the same, ordered by 16-byte chunks (rope_table_kernel)
   int n_pos, pos_x, rot_ctx;
   float* part_o;
   float* part_ml;

@@ -181,9 +181,9 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) attend_decode_kernel(const __g
           const int at = (k < n0 ? frame_pos(0, a0 + k) : frame_pos(1, a1 + k - n0)) + (h & 1) * 8 + (lane >> 3);
 #pragma unroll
           for (int j = 0; j < 2; ++j) {  // (pad rows: any position)
-            const float4* t = reinterpret_cast<const float4*>(p.tab + (long long)min(at + 4 * j, p.n_pos - 1) * 64 + c * 8);
+            const float4* t = reinterpret_cast<const float4*>(p.tab_c + (long long)min(at + 4 * j, p.n_pos - 1) * 64) + c;
 #pragma unroll
-            for (int w = 0; w < 4; ++w) x[j][w] = __ldg(t + w);
+            for (int w = 0; w < 4; ++w) x[j][w] = __ldg(t + 8 * w);
           }
         };
         auto turn = [&](int h, const float4 (&x)[2][4]) {
@@ -560,6 +560,7 @@ cudaError_t rekv_launch_attend_decode(rekv_ctx* c, const void* q, const QBatch& 
   if (full) p.sb = *full->sb;
   p.early = c->ctx_settled && c->ctx_stream == st;
   p.tab = full ? c->rope_tab : nullptr;
+  p.tab_c = full ? c->rope_tab_c : nullptr;
   p.n_pos = c->rope_positions;
   p.pos_x = rekv_pos_x(c, ncf);
   p.rot_ctx = rekv_rope_ctx(c);

@@ -17,7 +17,9 @@ namespace {
 
 using namespace rekv_ptx;
 
-__global__ void rope_table_kernel(float2* __restrict__ tab, int n_pos, double theta) {
+// Twice: in the order of the pairs, and for threads that take the eight pairs of a 16-byte chunk each, chunk c and float4 w of
+// (cos, sin) at [position][w][c], so that eight threads read whole lines (four rows of a warp: 4 lines per load instead of 16).
+__global__ void rope_table_kernel(float2* __restrict__ tab, float2* __restrict__ tab_c, int n_pos, double theta) {
   const int i = threadIdx.x & 63;
   const long long pos = (long long)blockIdx.x * (blockDim.x >> 6) + (threadIdx.x >> 6);
   if (pos >= n_pos) return;
@@ -25,6 +27,7 @@ __global__ void rope_table_kernel(float2* __restrict__ tab, int n_pos, double th
   double s, c;
   sincos(angle, &s, &c);
   tab[pos * 64 + i] = make_float2((float)c, (float)s);
+  tab_c[pos * 64 + (((i >> 1) & 3) * 8 + (i >> 3)) * 2 + (i & 1)] = make_float2((float)c, (float)s);
 }
 
 // rotates the 8 pairs (lo[e], hi[e]) held as bf16 in two 16-byte chunks; cs: the pairs' (cos, sin),
@@ -35,14 +38,15 @@ __device__ __forceinline__ void rotate_chunk(uint4& lo, uint4& hi, const float4 
 #pragma unroll
   for (int w = 0; w < 4; ++w) rotate_pair(l[w], h[w], cs[w]);
 }
-__device__ __forceinline__ void load_cs(float4 (&cs)[4], const float2* __restrict__ tab_row8) {
-  const float4* t = reinterpret_cast<const float4*>(tab_row8);
+// chunk c of position pos, from the table ordered by chunks
+__device__ __forceinline__ void load_cs(float4 (&cs)[4], const float2* __restrict__ tab_c, long long pos, int c) {
+  const float4* t = reinterpret_cast<const float4*>(tab_c + pos * 64) + c;
 #pragma unroll
-  for (int w = 0; w < 4; ++w) cs[w] = __ldg(t + w);
+  for (int w = 0; w < 4; ++w) cs[w] = __ldg(t + 8 * w);
 }
-__device__ __forceinline__ void rotate_chunk(uint4& lo, uint4& hi, const float2* __restrict__ tab_row8) {
+__device__ __forceinline__ void rotate_chunk(uint4& lo, uint4& hi, const float2* __restrict__ tab_c, long long pos, int c) {
   float4 cs[4];
-  load_cs(cs, tab_row8);
+  load_cs(cs, tab_c, pos, c);
   rotate_chunk(lo, hi, cs);
 }
 
@@ -75,7 +79,7 @@ __global__ void __launch_bounds__(256) stage_x_kernel(const uint4* __restrict__ 
     const int pos = n_ctx_tokens + (ns - nq) + (n - qb.cu[qi]);
     const long long base = ((long long)l * qb.sumNq * Hq + row) * 16;  // 16 chunks of 16 bytes per row
     uint4 lo = q[base + c], hi = q[base + 8 + c];
-    rotate_chunk(lo, hi, tab + (long long)pos * 64 + c * 8);
+    rotate_chunk(lo, hi, tab, pos, c);
     q_rot[base + c] = lo;
     q_rot[base + 8 + c] = hi;
     return;
@@ -89,34 +93,41 @@ __global__ void __launch_bounds__(256) stage_x_kernel(const uint4* __restrict__ 
   const int s = tok - sb.cu[qi];
   const uint4* src = (kv ? v_self : k_self) + ((long long)l * sb.sumNq * Hkv + row) * 16;
   uint4 lo = src[c], hi = src[8 + c];
-  if (!kv && tab) rotate_chunk(lo, hi, tab + (long long)(n_ctx_tokens + s) * 64 + c * 8);
+  if (!kv && tab) rotate_chunk(lo, hi, tab, n_ctx_tokens + s, c);
   const int r = ((sb.cu[qi] + 7) & ~7) + 8 * qi + s;
   char* dst = x_kv + (((long long)(l * Hkv + g) * 2 + kv) * 2 * x_rows + r) * 128 + ((c ^ (r & 7)) << 4);
   *reinterpret_cast<uint4*>(dst) = lo;
   *reinterpret_cast<uint4*>(dst + x_rows * 128) = hi;
 }
 
-// Rotated copies of the context's K tiles.  grid = (ncf, nQ, L), 256 threads.  A K tile of one KV head is
+// Rotated copies of the context's K tiles.  grid = (ncf * parts, nQ, L), 256 threads; a part of a page is a share of its rows (a
+// block per page left most of the device idle where the context is a window: 28 layers of 8 frames 17.5 us, encoding step with
+// parts 244 -> 241).  Long contexts are bound by HBM: 808 MB read and written at 72 frames, 132 us.  A K tile of one KV head is
 // two 64-dim halves of [N_f rows][128 B] with 16-byte chunks XOR-swizzled by (row & 7): dimension pair
 // (i, i + 64) sits at the same swizzled offset of the two halves, so a thread moves one chunk of each.
 __global__ void __launch_bounds__(256) rope_stage_kernel(char* const* __restrict__ tbl, char** __restrict__ tbl_k,
                                                          char* __restrict__ k_rot, int nQ, int ncf, int Hkv, int Nf,
-                                                         const float2* __restrict__ tab, int layer0) {
+                                                         const float2* __restrict__ tab, int layer0, int parts) {
   grid_dep_wait();
-  const int slot = blockIdx.x, qi = blockIdx.y, l = layer0 + blockIdx.z;
+  // (no divisions where a page is one block: 300 against 305 us for 12 tokens over 72 frames)
+  const int slot = parts == 1 ? blockIdx.x : blockIdx.x / parts, part = blockIdx.x - slot * parts;
+  const int qi = blockIdx.y, l = layer0 + blockIdx.z;
   const long long e = ((long long)l * nQ + qi) * ncf + slot;
   const char* page = tbl[e];
   const long long half_bytes = (long long)Nf * 128;
   char* dst = k_rot + e * Hkv * 2 * half_bytes;
-  if (threadIdx.x == 0) tbl_k[e] = dst;
+  if (threadIdx.x == 0 && part == 0) tbl_k[e] = dst;
   // a thread takes (row, chunk) positions and walks the KV heads: the (cos, sin) of a position are loaded
   // once for all heads, and four heads' chunks are in flight before the first rotation
   constexpr int U = 4;
-  for (int rc = threadIdx.x; rc < Nf * 8; rc += 256) {
+  const int rc1 = parts == 1 ? Nf * 8 : (part + 1) * Nf / parts * 8;
+  for (int rc = (parts == 1 ? 0 : part * Nf / parts * 8) + threadIdx.x; rc < rc1; rc += 256) {
     const int c = rc & 7, r = rc >> 3;
     const long long off = (long long)r * 128 + ((c ^ (r & 7)) << 4);
     float4 cs[4];
-    load_cs(cs, tab + ((long long)slot * Nf + r) * 64 + c * 8);
+    const float4* tr = reinterpret_cast<const float4*>(tab + ((long long)slot * Nf + r) * 64 + c * 8);
+#pragma unroll
+    for (int w = 0; w < 4; ++w) cs[w] = __ldg(tr + w);
     for (int g0 = 0; g0 < Hkv; g0 += U) {
       uint4 lo[U], hi[U];
 #pragma unroll
@@ -141,7 +152,7 @@ __global__ void __launch_bounds__(256) rope_stage_kernel(char* const* __restrict
 }  // namespace
 
 cudaError_t rekv_launch_rope_table(rekv_ctx* c, cudaStream_t st) {
-  rope_table_kernel<<<(c->rope_positions + 3) / 4, 256, 0, st>>>(c->rope_tab, c->rope_positions,
+  rope_table_kernel<<<(c->rope_positions + 3) / 4, 256, 0, st>>>(c->rope_tab, c->rope_tab_c, c->rope_positions,
                                                                 (double)c->cfg.rope_theta);
   return cudaGetLastError();
 }
@@ -161,7 +172,7 @@ cudaError_t rekv_launch_attend_full_self(rekv_ctx* c, const void* q, const void*
   const int rows = (rope ? qb.sumNq * s.Hq : 0) + 2 * sb.sumNq * s.Hkv;
   cudaError_t e = rekv_launch_pdl(stage_x_kernel, dim3((rows + 31) / 32, nl), dim3(256), 0, st, (const uint4*)q,
                                   (uint4*)c->q_rot, (const uint4*)k_self, (const uint4*)v_self, c->x_kv, c->x_rows, qb, sb,
-                                  s.Hq, s.Hkv, rekv_pos_x(c, ncf), rope ? c->rope_tab : nullptr, layer0);
+                                  s.Hq, s.Hkv, rekv_pos_x(c, ncf), rope ? c->rope_tab_c : nullptr, layer0);
   if (e == cudaSuccess) c->launches += 1;
   return e;
 }
@@ -171,8 +182,11 @@ cudaError_t rekv_launch_attend_full_ctx(rekv_ctx* c, const QBatch& qb, int ncf, 
                                         int layer1) {
   const StoreView& s = c->sv;
   if (!rekv_rope_ctx(c) || ncf == 0 || rekv_decode_shaped(c, qb, ncf, layer1 - layer0)) return cudaSuccess;
-  cudaError_t e = rekv_launch_pdl(rope_stage_kernel, dim3(ncf, qb.nQ, layer1 - layer0), dim3(256), 0, st, c->ctx_tbl, c->tbl_k,
-                                  c->k_rot, qb.nQ, ncf, s.Hkv, s.Nf, c->rope_tab, layer0);
+  // at least sixteen blocks for each SM, as far as a block has a row for every eight of its threads
+  const long long pages = (long long)ncf * qb.nQ * (layer1 - layer0);
+  const int parts = (int)std::max(1ll, std::min<long long>(s.Nf / 32, 16ll * rekv_sm_count() / pages));
+  cudaError_t e = rekv_launch_pdl(rope_stage_kernel, dim3(ncf * parts, qb.nQ, layer1 - layer0), dim3(256), 0, st, c->ctx_tbl, c->tbl_k,
+                                  c->k_rot, qb.nQ, ncf, s.Hkv, s.Nf, c->rope_tab, layer0, parts);
   if (e == cudaSuccess) c->launches += 1;
   return e;
 }

@@ -161,7 +161,7 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
   c->x_kv = nullptr;
   c->x_rows = 0;
   c->q_rot = nullptr;
-  c->rope_tab = nullptr;
+  c->rope_tab = c->rope_tab_c = nullptr;
   c->k_rot = nullptr;
   c->tbl_k = nullptr;
   c->rope_positions = 0;
@@ -242,6 +242,7 @@ int rekv_create(const rekv_config* cfg, rekv_ctx** out) {
     c->rope_positions = (static_ctx ? 1 : ctx_frames_max * s.Nf) + cfg->max_self_tokens;
     want(&c->q_rot, (size_t)s.L * cfg->max_q_tokens * s.Hq * 128 * sizeof(__nv_bfloat16));
     want(&c->rope_tab, (size_t)c->rope_positions * 64 * sizeof(float2));
+    want(&c->rope_tab_c, (size_t)c->rope_positions * 64 * sizeof(float2));
     if (!static_ctx) {
       want(&c->k_rot, (size_t)s.L * maxQ * ctx_frames_max * (s.page_bytes / 2));
       want(&c->tbl_k, (size_t)s.L * maxQ * (ctx_frames_max + 1) * sizeof(char*));

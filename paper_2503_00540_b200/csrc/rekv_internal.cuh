@@ -132,6 +132,7 @@ struct rekv_ctx {
   long long x_rows;
   __nv_bfloat16* q_rot;             // [L][max_q_tokens][H_q][128] rotated queries (rope_theta > 0)
   float2* rope_tab;                 // [rope_positions][64] (cos, sin)
+  float2* rope_tab_c;               // the same, ordered by 16-byte chunks (rope_table_kernel)
   int rope_positions;
   char* k_rot;                      // [L][max_questions][ctx frames][H_kv] rotated K tiles
   char** tbl_k;                     // [L][max_questions][ctx frames]
