@@ -311,11 +311,13 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
   // (With early_q the softmax warps load the first Q tile before their wait.)  No warp releases the next launch before its own
   // wait: one thread's release counts for its CTA, and the next launch may take what this one's predecessors wrote as complete.
   const bool loads_q = warp >= SM_WARP0 && warp < OUT_WARP0;
+  // The service warps wait where they first need what this launch's predecessors wrote: their index work comes before that.
   const bool waits_later = p.early_q && loads_q;
-  if (!waits_later) {
+  auto depend = [&]() {
     if (!p.second) grid_dep_wait();
     grid_dep_launch();
-  }
+  };
+  if (!waits_later && warp >= SM_WARP0) depend();
 
   const uint32_t wait_limit = p.wait_limit ? p.wait_limit : WAIT_LIMIT;
   auto try_wait = [&](int b, uint32_t parity) -> bool {
@@ -372,10 +374,7 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
   if (loads_q) {  // the first segment's Q
     load_q(decode_seg<CG>(p, range0, range1), 0, (warp - SM_WARP0) * 16, std::integral_constant<int, 8>{});
     if (lane == 0) mbar_arrive(bar(B_QFULL));
-    if (waits_later) {
-      grid_dep_wait();
-      grid_dep_launch();
-    }
+    if (waits_later) depend();
   }
 
   // ================= a segment's result, one thread per row (and half of its columns without output warps) =================
@@ -588,6 +587,7 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
             int f_lo = a / p.Ns, pos_a = a - f_lo * p.Ns;    // row a is row pos_a of frame f_lo
             int fb = -64;                                    // a lane holds the page pointer of frame fb + lane
             const char* my_page = nullptr;
+            if (issued == 0) depend();
 #pragma unroll 1
             for (int I = s.I0; I < s.I1 && ok; ++I) {
               if (f_lo < p.ncf && f_lo + 17 >= fb + 32) {
@@ -770,6 +770,7 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
             // ================= Q of the segments after the first, behind the current one's work =================
             // (the first segment's rows are loaded by the eight softmax warps, which have nothing else to do yet: by one
             // warp they took 5 us)
+            if (segn == 1) depend();
             if (segn >= 2) ok = wait(B_QFREE + par, ((segn >> 1) - 1) & 1u);
             if (ok) {
               load_q(s, par, 0, std::integral_constant<int, 64>{});
