@@ -1035,11 +1035,12 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
 // Joins the parts of units where the attention kernel does not (launches of few units, such as one layer: several whole workers
 // each; units of more than MAX_PARTS_INSIDE parts).
 // grid = (units, CTAs of a pair, 32 column quads), 256 threads: a thread per (row, every second part), consecutive threads on
-// consecutive rows, so that a part is read in 2 KB runs and 16 parts are one round of loads deep; the two groups' results
-// meet in shared memory.  (28 layers, 28 heads, 72 frames, one layer at a time: 946 us; four groups 962; a thread walking all parts of a row,
-// three rounds for the 19 parts of a layer, about 1040.)
+// consecutive rows, so that a part is read in 2 KB runs and all parts are one round of loads deep: MERGE_AHEAD in flight per
+// thread, as many as the launch needs; the two groups' results meet in shared memory.  (28 layers, 28 heads, 72 frames, one layer
+// at a time, 19 parts: eight in flight 844 us, ten 827; 20 layers of 8 KV heads, 11 parts: six 502, eight 502, ten 511, twelve 520.
+// Four groups instead of two, eight in flight: 962 against 946 then.)
 constexpr int MERGE_GROUPS = 2;
-template <int CG>
+template <int CG, int MERGE_AHEAD>
 __global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __grid_constant__ Tc5Params p) {
   const int lh = (int)blockIdx.x / p.W, rank = blockIdx.y;  // blockIdx.x counts (layer, kv head) x row blocks; W = row blocks
   int mp = (int)blockIdx.x - lh * p.W, qi = 0, c0 = lh * p.per_lh;
@@ -1067,11 +1068,11 @@ __global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __g
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
   if (rr < rows_q) {
 #pragma unroll 1
-    for (int k0 = grp; k0 < n_parts; k0 += 8 * MERGE_GROUPS) {
-      float2 ml[8];
-      float4 o[8];
+    for (int k0 = grp; k0 < n_parts; k0 += MERGE_AHEAD * MERGE_GROUPS) {
+      float2 ml[MERGE_AHEAD];
+      float4 o[MERGE_AHEAD];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < MERGE_AHEAD; ++i) {
         const int k = k0 + i * MERGE_GROUPS;
         ml[i] = make_float2(-INFINITY, 0.f);
         o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1083,7 +1084,7 @@ __global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __g
       }
       float Mn = M;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) Mn = fmaxf(Mn, ml[i].x);
+      for (int i = 0; i < MERGE_AHEAD; ++i) Mn = fmaxf(Mn, ml[i].x);
       const float a = ex2(M - Mn);
       M = Mn;
       den *= a;
@@ -1092,7 +1093,7 @@ __global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __g
       acc.z *= a;
       acc.w *= a;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < MERGE_AHEAD; ++i) {
         const float w = ex2(ml[i].x - M);
         den = fmaf(w, ml[i].y, den);
         acc.x = fmaf(w, o[i].x, acc.x);
@@ -1216,7 +1217,12 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
     Tc5Params m = p;
     m.merge_inside = p.W;
     m.W = blocks;
-    e = rekv_launch_pdl(merge_tc5_kernel<CG>, dim3((unsigned)(p.nl * p.Hkv * blocks), CG, 32), dim3(128 * MERGE_GROUPS), 0, st, m);
+    const int parts = std::min(p.W, (max_ch - 1) / (p.total / p.W) + 2);   // of a unit, at most
+    const auto merge = parts <= 4 * MERGE_GROUPS   ? merge_tc5_kernel<CG, 4>
+                       : parts <= 6 * MERGE_GROUPS ? merge_tc5_kernel<CG, 6>
+                       : parts <= 8 * MERGE_GROUPS ? merge_tc5_kernel<CG, 8>
+                                                   : merge_tc5_kernel<CG, 10>;
+    e = rekv_launch_pdl(merge, dim3((unsigned)(p.nl * p.Hkv * blocks), CG, 32), dim3(128 * MERGE_GROUPS), 0, st, m);
     if (e != cudaSuccess) return e;
     c->launches += 1;
     if (timed) {

@@ -391,3 +391,10 @@ def test_results_put_out_while_the_next_segment_goes_on(L, n_tokens, late):
         g.check_status()
         H.assert_attention(out, ref["out"], "attention")
     g.close()
+
+
+@pytest.mark.parametrize("Hkv,n_tokens", [(1, 20), (2, 37), (3, 20), (4, 20), (5, 9), (6, 40), (8, 20), (8, 5)])
+def test_one_layers_parts_joined_by_the_merge_launch(Hkv, n_tokens):
+    """Units of 51 chunks, few of them: from about fifty parts of a unit to about nine, every number in flight that the merge launch
+    is compiled for, on pairs and on single CTAs."""
+    _run_question_parity(H.Shape(L=1, Hq=7 * Hkv, Hkv=Hkv, Nf=196, T=36, W=2, k=31, seed=7), [n_tokens])
