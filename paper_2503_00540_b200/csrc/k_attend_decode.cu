@@ -16,7 +16,7 @@ namespace rekv_att {
 // dependency wait, in us: Q 0.7, two frames 3.4, parts out 0.9, join 4; and the copies of the frames, 6.7 from a CTA's start, which
 // can begin when the SM's CTA of the launch before has left.  So everything that does not depend on the launch before is done
 // before the wait (the frames, their rotation), X is asked for right after it, and the join has all its loads in flight:
-// 562 -> 397 us, 20 -> 14 a layer.
+// 562 -> 391 us, 20 -> 14 a layer.
 // Rotary embedding: the queries are rotated as they are loaded.  The keys of a CTA's first two steps are rotated in place in
 // shared memory before the dependency wait (where the context is known to be complete), later ones in registers between ldmatrix
 // and mma -- the dimensions i and i + 64 of a token lie in the same lane's fragments of k-blocks kb and kb + 4 -- with (cos, sin)
