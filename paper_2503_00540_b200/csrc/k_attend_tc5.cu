@@ -1000,6 +1000,9 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
       }
     }
     if constexpr (ROLE == 0) {
+      // The other CTA's hand-back of the last segment's O arrives at this CTA's shared memory: it must have landed before this
+      // CTA leaves.  (Every earlier one was waited for by the P V behind it.)
+      if (CG == 2 && warp == 1 && leader && ok && segn > 0) wait(B_OFREE, (segn - 1) & 1u);
       // A CTA that gives up must not return while copies into its shared memory are still on their way: the producers
       // wait (bounded) for the tiles they have issued and nobody consumed -- at most the rings' depth.
       if (*s_abort && (warp == 0 || warp == 2)) {
@@ -1025,10 +1028,15 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
 
   __syncwarp();
   tc_fence_before();
-  if constexpr (CG == 2)
-    cluster_sync_relaxed();
-  else
+  if constexpr (CG == 2) {
+    // (a pair that gave up has not waited for each other's arrivals: the barrier orders them)
+    if (__any_sync(0xffffffffu, *s_abort != 0))
+      cluster_sync_all();
+    else
+      cluster_sync_relaxed();
+  } else {
     __syncthreads();
+  }
   if (p.second) grid_dep_wait();
   if (warp == 0) tmem_dealloc<CG>(tmem, TMEM_COLS);
 }

@@ -66,6 +66,16 @@ def test_decode_kernel_gives_up_when_a_frame_never_arrives():
     _expire_then_recover(s, [1], 0)
 
 
+@pytest.mark.parametrize("n_tokens,skip_entry", [(16, 0), (16, 1), (16, 68), (16, 69), (80, 0), (80, 1), (80, 69), (80, 136)])
+def test_results_of_several_segments_are_given_up_with_the_rest(n_tokens, skip_entry):
+    """160 units of 34 chunks over 144 single CTAs (16 tokens) or 64 pairs (80), several segments each.  The first CTA misses its
+    first K tile, its first V tile, or one of its second or third segment (34 chunks each): the warps that put out a segment's
+    result then wait for a product that never comes, and where they are warps of their own the softmax warps wait for them.  A
+    pair's CTAs leave together."""
+    s = H.Shape(L=20, Hq=16, Hkv=8, Nf=80, T=56, W=2, k=52, seed=7)
+    _expire_then_recover(s, [n_tokens], skip_entry)
+
+
 @pytest.mark.parametrize("L,lengths", [(1, [16]), (12, [5, 3, 4])])  # clusters of 16 and of 8 CTAs
 @pytest.mark.parametrize("mode", [rekv.TEST_RETRIEVE_SKIP_SUM, rekv.TEST_RETRIEVE_SKIP_SCORE])
 def test_one_launch_retrieval_gives_up_when_a_part_never_arrives(L, lengths, mode):
