@@ -387,8 +387,9 @@ __global__ void __launch_bounds__(DEC_THREADS, 1) attend_decode_kernel(const __g
       }
     }
     if (!ok) {
-      // a copy never completed: record it and give the copies still in flight -- the last two steps issued, one
-      // per stage -- a bounded chance to land before the CTA's shared memory is given up
+      // a copy never completed: record it and give the copies still in flight -- every thread's share of X, and the last two
+      // steps of frames issued, one per stage (a bounded chance) -- time to land before the CTA's shared memory is given up
+      cp_async_wait_all();
       if (tid == 0) {
         atomicExch(p.status, REKV_ERR_TIMEOUT);
         for (uint32_t e = issued > 2 ? issued - 2 : 0; e < issued; ++e)

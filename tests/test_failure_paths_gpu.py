@@ -76,6 +76,37 @@ def test_results_of_several_segments_are_given_up_with_the_rest(n_tokens, skip_e
     _expire_then_recover(s, [n_tokens], skip_entry)
 
 
+@pytest.mark.parametrize("s,nq,ns,skip_entry", [
+    (H.Shape(L=3, Hq=28, Hkv=4, Nf=196, T=80, W=2, k=70, seed=7), 1, 48, 0),    # two frames on a CTA, the first missing
+    (H.Shape(L=3, Hq=28, Hkv=4, Nf=196, T=80, W=2, k=70, seed=7), 1, 48, 1),    # ... the second
+    (H.Shape(L=2, Hq=32, Hkv=8, Nf=16, T=10, W=2, k=6, seed=7), 16, 5, 0),      # eight frames in a step, X's copies behind them
+], ids=["first", "second", "x_in_flight"])
+def test_a_frame_rotated_before_the_dependency_wait_never_arrives(s, nq, ns, skip_entry):
+    """One token at a time over a context that earlier launches on the stream have read: its first frames are copied, and their keys
+    rotated, before the dependency wait.  The wait for the frame that is left out is the rotation's."""
+    g = H.build_gpu(s, max_questions=nq, max_q_tokens=nq, max_self_tokens=nq * ns, rope_theta=1e6)
+    q, cu = H.questions(s, [1] * nq, device="cuda")
+    ks, vs, cus = H.self_kv(s, [ns] * nq, device="cuda")
+    g.gather(g.retrieve(q, cu, s.k, s.T)[0], nq, s.k, s.T)
+
+    def token():
+        return torch.stack([g.attend_full_layer(l, q[l], ks[l], vs[l], cu, cus) for l in range(s.L)])
+    token()
+    out0 = token()
+    g.check_status()
+    g.test_set_wait_limit(20000, skip_entry)
+    token()
+    with pytest.raises(rekv.RekvError) as e:
+        g.check_status()
+    assert e.value.code == rekv.ERR_TIMEOUT
+    g.check_status()
+    g.test_set_wait_limit(0, -1)
+    assert torch.equal(token(), out0)
+    assert torch.equal(token(), out0)
+    g.check_status()
+    g.close()
+
+
 @pytest.mark.parametrize("L,lengths", [(1, [16]), (12, [5, 3, 4])])  # clusters of 16 and of 8 CTAs
 @pytest.mark.parametrize("mode", [rekv.TEST_RETRIEVE_SKIP_SUM, rekv.TEST_RETRIEVE_SKIP_SCORE])
 def test_one_launch_retrieval_gives_up_when_a_part_never_arrives(L, lengths, mode):
