@@ -1,5 +1,5 @@
-// How many workers a launch of the tensor-core attention kernel takes, and who joins the parts of cut units.  Plain host code
-// (no CUDA), so that the rule can be walked over many batches without a device.
+// How many workers a launch of the tensor-core attention kernel takes, who joins the parts of cut units, and who puts out the
+// results.  Plain host code (no CUDA), so that the rules can be walked over many batches without a device.
 #pragma once
 
 #include <algorithm>
@@ -56,4 +56,19 @@ inline AttendPlan rekv_attend_plan(int total, int units, int max_ch, bool equal,
     }
   }
   return best;
+}
+
+// Whether four warps of their own put out the segments' results while the softmax warps go on with the next segment.  They take
+// registers from the softmax warps (216 -> 176 a thread: two loads of a row instead of one, and spills in the pair), which a
+// range of one segment or of short ones does not get back, and pairs never do: their softmax warps are the pace.  One B200, us
+// without / with, the same contexts in turn (a library against itself: within 1 %):
+//   pairs   28 layers of 4 KV heads, 64 tokens, 19, 63, 113 chunks  107 / 118, 262 / 276, 444 / 456; 32 tokens, 113 chunks 232 / 236
+//           40 layers of 8 KV heads, 32 tokens, 63 chunks 388 / 411; 16 questions, 63 chunks 3050 / 3108
+//           (in runs of seconds, at the power limit: 1800-frame question 261 / 265, 16 questions 3187 / 3232)
+//   single  40 layers of 8 KV heads, 16 tokens, 13, 32, 63, 113 chunks  84.7 / 85.8, 159 / 154, 251 / 248, 450 / 432;
+//           5 tokens, 13, 32, 44, 113 chunks  77 / 80, 139 / 141, 170 / 170, 396 / 381; 28 layers of 4 KV heads, 3 questions of
+//           12 tokens, 13, 32, 113 chunks  87 / 91, 151 / 148, 458 / 446
+inline bool rekv_attend_output_warps(int workers, int units, int max_ch, bool pairs) {
+  constexpr int MIN_CHUNKS = 32;
+  return !pairs && workers < units && max_ch >= MIN_CHUNKS;
 }

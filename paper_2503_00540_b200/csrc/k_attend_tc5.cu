@@ -32,8 +32,8 @@
 //   warp 3      second CTA of a pair: passes its tiles' arrivals on to the issuing CTA
 //   warp 3 (warp 1 in a pair's second CTA)   the next segment's Q tile (cp.async, double-buffered)
 //   warps 4-7, 8-11   softmax of the even / odd chunks, one thread per row (= TMEM lane), fp32
-//   warps 12-15 (OUT)   the segments' results, so that the softmax warps go on with the next segment's chunks meanwhile; in
-//                       launches without them (one segment per worker, or short ones) the softmax warps put out the results
+//   warps 12-15 (OUT)   the segments' results, so that the softmax warps go on with the next segment's chunks meanwhile: single
+//                       CTAs with several long segments each (attend_plan.h); else the softmax warps put out the results
 // After set-up the service warpgroup shrinks to 72 (56 with output warps) registers per thread and the softmax warpgroups grow to
 // 216 (176) (setmaxnreg), so that a softmax thread holds a whole S row chunk: one or two TMEM loads and two TMEM stores per
 // chunk (a warp's tcgen05.ld/st cost about 90 cycles each whatever their width).
@@ -61,11 +61,8 @@ using namespace rekv_att;
 namespace {
 
 constexpr int SM_WARP0 = 4, OUT_WARP0 = 12;            // first softmax warp, first output warp
-// OUT: four more warps put out the segments' results, else the softmax warps do it themselves.
+// OUT: four more warps put out the segments' results, else the softmax warps do it themselves (rekv_attend_output_warps).
 // Registers per thread: 128 * service + 256 * softmax (+ 128 * output) <= threads * those at launch
-// One B200, us without / with output warps: 1800-frame question (units of 113 chunks) 262 / 254, Eq. 3 in full 240 / 228, 10-token
-// question 182 / 179, 16-question batch (63 chunks) 3160 / 3130; encoding step (units of 15 chunks) 254 / 259.
-constexpr int OUT_MIN_CHUNKS = 32;
 template <bool OUT>
 struct Warps {
   static constexpr int THREADS = OUT ? 512 : 384;
@@ -1160,7 +1157,7 @@ int max_workers() {
   if (CG == 2) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * n);
-    cfg.blockDim = dim3(Warps<true>::THREADS);
+    cfg.blockDim = dim3(Warps<false>::THREADS);
     cfg.dynamicSmemBytes = TC_SMEM;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1169,7 +1166,7 @@ int max_workers() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int m = 0;
-    if (prepare_tc5<CG, true>() == cudaSuccess && cudaOccupancyMaxActiveClusters(&m, attend_tc5_kernel<CG, true>, &cfg) == cudaSuccess && m > 0)
+    if (prepare_tc5<CG, false>() == cudaSuccess && cudaOccupancyMaxActiveClusters(&m, attend_tc5_kernel<CG, false>, &cfg) == cudaSuccess && m > 0)
       n = std::min(n, m);
     else
       cudaGetLastError();
@@ -1194,13 +1191,14 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
   if (total > 0x7fffffff / 2) return cudaErrorInvalidValue;
   p.total = (int)total;
   // (split launches: no merge launch between or after the two)
-  const AttendPlan plan = rekv_attend_plan(p.total, p.nl * p.Hkv * blocks, max_ch, equal, max_workers<CG>(), !p.split_rem, CG == 2);
+  const int units = p.nl * p.Hkv * blocks;
+  const AttendPlan plan = rekv_attend_plan(p.total, units, max_ch, equal, max_workers<CG>(), !p.split_rem, CG == 2);
   p.W = plan.workers;
   p.merge_inside = plan.merge_inside;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(p.W * CG));
-  // output warps where a worker's range has several segments, and long ones
-  const bool out = p.W < p.nl * p.Hkv * blocks && max_ch >= OUT_MIN_CHUNKS;
+  bool out = false;
+  if constexpr (CG == 1) out = rekv_attend_output_warps(p.W, units, max_ch, false);   // (pairs are not compiled with output warps)
   cfg.blockDim = dim3(out ? Warps<true>::THREADS : Warps<false>::THREADS);
   cfg.dynamicSmemBytes = TC_SMEM;
   cfg.stream = st;
@@ -1213,8 +1211,16 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
   cfg.attrs = at;
   cfg.numAttrs = 2;
   if (timed && !p.second) cudaEventRecord(c->ev_t0, st);
-  cudaError_t e = out ? prepare_tc5<CG, true>() : prepare_tc5<CG, false>();
-  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, out ? attend_tc5_kernel<CG, true> : attend_tc5_kernel<CG, false>, p);
+  auto launch = [&](auto with_out) {
+    constexpr bool OUT = decltype(with_out)::value;
+    const cudaError_t ep = prepare_tc5<CG, OUT>();
+    return ep == cudaSuccess ? cudaLaunchKernelEx(&cfg, attend_tc5_kernel<CG, OUT>, p) : ep;
+  };
+  cudaError_t e;
+  if constexpr (CG == 1)
+    e = out ? launch(std::true_type{}) : launch(std::false_type{});
+  else
+    e = launch(std::false_type{});
   if (e != cudaSuccess) return e;
   c->launches += 1;
   if (timed) {
@@ -1231,7 +1237,7 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
                        : parts <= 6 * MERGE_GROUPS ? merge_tc5_kernel<CG, 6>
                        : parts <= 8 * MERGE_GROUPS ? merge_tc5_kernel<CG, 8>
                                                    : merge_tc5_kernel<CG, 10>;
-    e = rekv_launch_pdl(merge, dim3((unsigned)(p.nl * p.Hkv * blocks), CG, 32), dim3(128 * MERGE_GROUPS), 0, st, m);
+    e = rekv_launch_pdl(merge, dim3((unsigned)units, CG, 32), dim3(128 * MERGE_GROUPS), 0, st, m);
     if (e != cudaSuccess) return e;
     c->launches += 1;
     if (timed) {

@@ -17,16 +17,24 @@ extern "C" int plan(int total, int units, int max_ch, int equal, int max_w, int 
   *workers = p.workers;
   return p.merge_inside;
 }
+extern "C" int output_warps(int workers, int units, int max_ch, int pairs) {
+  return rekv_attend_output_warps(workers, units, max_ch, pairs != 0);
+}
 """
 
 
 @pytest.fixture(scope="module")
-def plan(tmp_path_factory):
+def rules(tmp_path_factory):
     d = tmp_path_factory.mktemp("plan")
     src, so = d / "plan.cpp", d / "plan.so"
     src.write_text(SOURCE)
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, "-o", str(so), str(src)])
-    fn = ctypes.CDLL(str(so)).plan
+    return ctypes.CDLL(str(so))
+
+
+@pytest.fixture(scope="module")
+def plan(rules):
+    fn = rules.plan
 
     def call(chunks, lh, max_w, may_merge):
         """chunks: of one (layer, KV head)'s units, in launch order; lh: how many (layer, KV head) there are"""
@@ -77,3 +85,13 @@ def test_units_joined_in_the_kernel_have_at_most_four_parts(plan):
                 parts = (at + n - 1) * w // total - at * w // total + 1
                 assert parts <= 4, (chunks, lh, max_w, may_merge, w)
                 at += n
+
+
+@pytest.mark.parametrize("layers,n_tokens,expected", [(20, 16, True), (20, 80, False), (10, 80, False), (4, 16, False)])
+def test_output_warps_only_on_single_ctas_of_several_long_segments(plan, rules, layers, n_tokens, expected):
+    """The units of test_parity_gpu.py's and test_failure_paths_gpu.py's launches of several segments: 8 KV heads of two query heads
+    and 34 chunks; 16 tokens are 32 rows (single CTAs), 80 are 160 (pairs).  (4 layers: a worker for every unit.)"""
+    pairs = n_tokens * 2 > 128
+    workers, _ = plan([34], 8 * layers, 74 if pairs else 148, True)
+    assert rules.output_warps(workers, 8 * layers, 34, int(pairs)) == int(expected)
+    assert rules.output_warps(workers, 8 * layers, 31, int(pairs)) == 0

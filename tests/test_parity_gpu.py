@@ -365,9 +365,9 @@ def test_logits_far_above_the_first_chunk_raise_the_reference_maximum(n_tokens):
 @pytest.mark.parametrize("late", [False, True], ids=["ordinary", "late_large_logits"])
 @pytest.mark.parametrize("L,n_tokens", [(20, 16), (10, 80), (10, 140)])
 def test_results_put_out_while_the_next_segment_goes_on(L, n_tokens, late):
-    """Units of 34 chunks, more of them than workers: four warps of their own put out a segment's result (whole, and parts that
-    are joined) while the softmax warps work on the next one.  16 tokens: single CTAs; 80: pairs, their second CTA a quarter
-    full; 140: pairs and a second launch for the remaining rows.  With late large logits every segment that holds the
+    """Units of 34 chunks, several segments (whole units, and parts that are joined) per worker.  16 tokens: single CTAs, where four
+    warps of their own put out a segment's result while the softmax warps work on the next one; 80: pairs, their second CTA a
+    quarter full; 140: pairs and a second launch, of single CTAs, for the remaining rows.  With late large logits every segment that holds the
     last frame's first tokens is run again."""
     s = H.Shape(L=L, Hq=16, Hkv=8, Nf=80, T=56, W=2, k=52, seed=7)
     g = rekv.ReKV(s.L, s.Hq, s.Hkv, s.D, s.Nf, s.T, s.W, max_q_tokens=n_tokens, max_topk=s.k)
