@@ -101,8 +101,8 @@ constexpr int B_KFULL = 0, B_KEMPTY = 5, B_VFULL = 10, B_VEMPTY = 15, B_SFULL = 
 constexpr uint32_t OFF_M = 8 * B_COUNT;               // float [2 parity][128]: the segment's reference maxima
 constexpr uint32_t OFF_L = OFF_M + 1024;              // float [2 parity][128]: row sums
 constexpr uint32_t OFF_REDO = OFF_L + 1024;           // u64: segments to run again
-constexpr uint32_t OFF_WORDS = OFF_REDO + 8;          // u32: tmem slot, abort, overflow marks [2], fast, last
-constexpr uint32_t SMALL_BYTES = OFF_WORDS + 24;
+constexpr uint32_t OFF_WORDS = OFF_REDO + 8;          // u32: tmem slot, abort, overflow marks [2], fast, last, again
+constexpr uint32_t SMALL_BYTES = OFF_WORDS + 32;
 constexpr size_t TC_SMEM = 2 * Q_TILE_BYTES + RING_BYTES + SMALL_BYTES;  // (the dynamic segment is 1024-byte aligned)
 static_assert(TC_SMEM <= 227 * 1024, "shared-memory plan of the attention kernel");
 
@@ -252,6 +252,7 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
   volatile uint32_t* s_over = s_words + 2;   // [2] by segment parity: number (+ 1) of the last segment with an overflow
   volatile uint32_t* s_fast = s_words + 4;   // every other part of the unit is in place
   volatile uint32_t* s_last = s_words + 5;
+  volatile uint32_t* s_again = s_words + 6;  // segments are run again
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
       mbar_init(bar(B_LREADY + i), 8);
       mbar_init(bar(B_LFREE + i), WP::OUT_WARPS);
     }
-    for (int i = 1; i < 6; ++i) s_words[i] = 0;
+    for (int i = 1; i < 7; ++i) s_words[i] = 0;
     *s_redo = 0ull;
     fence_barrier_init();
   }
@@ -375,6 +376,11 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
     if (waits_later) depend();
   }
 
+  auto hand_back_o = [&]() {  // O has been read: the next segment's first P V may overwrite it
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) arrive_lead(B_OFREE);
+  };
   // ================= a segment's result, one thread per row (and half of its columns without output warps) =================
   // With output warps (OUT) the softmax warps go on with the next segment's chunks meanwhile.
   auto result = [&](const Seg& s, int si, int pos, uint32_t segn, bool safe, bool& ok, int part) {
@@ -408,7 +414,10 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
       }
     }
     if (safe && !(redo_mask(false) & redo_bit(si, s, pos))) put = false;  // (the pair's other CTA asked for it)
-    // O, 32 of the row's columns at a time.  The next segment's first P V waits until it has been read.
+    // O, 32 of the row's columns at a time.  The next segment's first P V waits until it has been read.  The range's last segment has
+    // none behind it and hands nothing back: nobody would wait for the other CTA's arrival before the issuing one's shared memory is
+    // given away.  (Waiting for it at the kernel's end: 28 layers, 64 tokens, 12 frames 107 -> 110 us, encoding step 239 -> 250.)
+    const bool last = !safe && pos + (s.I1 - s.I0) >= range1;
     const uint32_t t_o = tmem + ((uint32_t)((warp & 3) << 5) << 16);
     const int col0 = part * WP::COLUMNS;
     auto load_o = [&](int c0, float (&o)[32]) {
@@ -419,9 +428,7 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
       for (int i = 0; i < 32; ++i) o[i] = __uint_as_float(ou[i]);
     };
     auto o_free = [&]() {
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) arrive_lead(B_OFREE);
+      if (!last) hand_back_o();
     };
     if (put) tc_fence_after();
     __nv_bfloat16* dst = p.out + ((s.q_row0 + (valid ? n : 0)) * p.Hq + s.g * p.G + (valid ? j : 0)) * 128;
@@ -994,12 +1001,11 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
         else
           __syncthreads();
         if (redo_mask(true) == 0ull || *s_abort) break;
+        *s_again = 1;
+        if constexpr (ROLE == (OUT ? 2 : 1)) hand_back_o();   // the last segment's, after all
       }
     }
     if constexpr (ROLE == 0) {
-      // The other CTA's hand-back of the last segment's O arrives at this CTA's shared memory: it must have landed before this
-      // CTA leaves.  (Every earlier one was waited for by the P V behind it.)
-      if (CG == 2 && warp == 1 && leader && ok && segn > 0) wait(B_OFREE, (segn - 1) & 1u);
       // A CTA that gives up must not return while copies into its shared memory are still on their way: the producers
       // wait (bounded) for the tiles they have issued and nobody consumed -- at most the rings' depth.
       if (*s_abort && (warp == 0 || warp == 2)) {
@@ -1026,8 +1032,8 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
   __syncwarp();
   tc_fence_before();
   if constexpr (CG == 2) {
-    // (a pair that gave up has not waited for each other's arrivals: the barrier orders them)
-    if (__any_sync(0xffffffffu, *s_abort != 0))
+    // (a pair that gave up, or ran segments again, has not waited for all of each other's arrivals: the barrier orders them)
+    if (__any_sync(0xffffffffu, (*s_abort | *s_again) != 0))
       cluster_sync_all();
     else
       cluster_sync_relaxed();
