@@ -10,6 +10,7 @@ constexpr int REKV_MAX_PARTS_INSIDE = 4;  // parts of a unit that the attention 
 struct AttendPlan {
   int workers;        // each takes a contiguous range of the launch's chunks, equal to one chunk
   bool merge_inside;  // cut units are joined by the worker that finishes the last part, else by a merge launch
+  int parts;          // of a unit, at most (equal units: the most that one has)
 };
 
 // total: chunks of all units; max_ch: of the longest unit; equal: every unit has max_ch; max_w: workers that can run at once;
@@ -30,7 +31,7 @@ inline AttendPlan rekv_attend_plan(int total, int units, int max_ch, bool equal,
   const float CHUNK = pairs ? 0.75f : 1.f;
   constexpr float SEGMENT = 8.f, CUT = 4.f, MERGE = 2.f, MERGE_PART = 0.15f;
   const int most = std::min(max_w, total);
-  AttendPlan best = {0, true};
+  AttendPlan best = {0, true, 1};
   float best_cost = 0.f;
   for (int w = most; w >= 1 && (3 * w >= most || best.workers == 0); --w) {
     // the most segments of a range, partial segments of a range and parts of a unit.  Equal units, units / w = p / q in lowest
@@ -51,7 +52,7 @@ inline AttendPlan rekv_attend_plan(int total, int units, int max_ch, bool equal,
                                 : CUT * (float)cuts + (equal && !even && parts > 2 ? CUT * (float)(parts - 2) : 0.f);
     const float cost = CHUNK * (float)((total + w - 1) / w) + SEGMENT * (float)segments + join;
     if (best.workers == 0 || cost < best_cost) {
-      best = {w, !by_merge};
+      best = {w, !by_merge, parts};
       best_cost = cost;
     }
   }
@@ -71,4 +72,15 @@ inline AttendPlan rekv_attend_plan(int total, int units, int max_ch, bool equal,
 inline bool rekv_attend_output_warps(int workers, int units, int max_ch, bool pairs) {
   constexpr int MIN_CHUNKS = 32;
   return !pairs && workers < units && max_ch >= MIN_CHUNKS;
+}
+
+// Parts that a thread of the merge launch (two threads for a row's column quad, a block for 128 rows of 32 quads) has in flight.  More
+// of them are fewer rounds of loads but more registers, and a grid that is not resident at once pays a second start: 4, 8 or 10 in
+// flight (48, 73, 94 registers) let 5, 3 or 2 blocks be resident on an SM.  So 4 where 8 would not be resident, 10 only where it is
+// and saves a round.  One B200, 12 layers one at a time, us with 4 / 8 / 10 (a library against itself: within 2 %):
+//   320 blocks, 13 parts 268 / 258 / 270; 480, 7 parts 326 / 339 / 347; 512, 9 parts 400 / 414 / 422; 1024, 4 parts 417 / 441 / 465;
+//   256 blocks, 18 parts 322 / 308 / 298; 64, 19 parts 221 / 221 / 216; 64, 27 parts 240 / 235 / 240; 192, 22 parts 304 / 297 / 305
+inline int rekv_merge_ahead(int parts, long long blocks, int sms) {
+  if (blocks > 3ll * sms) return 4;
+  return parts > 16 && parts <= 20 && blocks <= 2ll * sms ? 10 : 8;
 }

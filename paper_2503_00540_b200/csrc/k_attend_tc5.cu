@@ -1047,13 +1047,12 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
 // Joins the parts of units where the attention kernel does not (launches of few units, such as one layer: several whole workers
 // each; units of more than MAX_PARTS_INSIDE parts).
 // grid = (units, CTAs of a pair, 32 column quads), 256 threads: a thread per (row, every second part), consecutive threads on
-// consecutive rows, so that a part is read in 2 KB runs and all parts are one round of loads deep: MERGE_AHEAD in flight per
-// thread, as many as the launch needs; the two groups' results meet in shared memory.  (28 layers, 28 heads, 72 frames, one layer
-// at a time, 19 parts: eight in flight 844 us, ten 827; 20 layers of 8 KV heads, 11 parts: six 502, eight 502, ten 511, twelve 520.
-// Four groups instead of two, eight in flight: 962 against 946 then.)
+// consecutive rows, so that a part is read in 2 KB runs and up to 20 parts are one round of loads: MERGE_AHEAD in flight per thread
+// (rekv_merge_ahead); the two groups' results meet in shared memory.  (Four groups instead of two, eight in flight: 962 us against 946
+// for 28 layers of 28 heads, 72 frames, one at a time.)
 constexpr int MERGE_GROUPS = 2;
 template <int CG, int MERGE_AHEAD>
-__global__ void __launch_bounds__(128 * MERGE_GROUPS) merge_tc5_kernel(const __grid_constant__ Tc5Params p) {
+__global__ void __launch_bounds__(128 * MERGE_GROUPS, MERGE_AHEAD <= 4 ? 5 : MERGE_AHEAD <= 8 ? 3 : 2) merge_tc5_kernel(const __grid_constant__ Tc5Params p) {
   const int lh = (int)blockIdx.x / p.W, rank = blockIdx.y;  // blockIdx.x counts (layer, kv head) x row blocks; W = row blocks
   int mp = (int)blockIdx.x - lh * p.W, qi = 0, c0 = lh * p.per_lh;
   for (; qi < p.qb.nQ - 1; ++qi) {
@@ -1238,11 +1237,10 @@ cudaError_t launch_tc5(rekv_ctx* c, Tc5Params& p, cudaStream_t st, bool timed) {
     Tc5Params m = p;
     m.merge_inside = p.W;
     m.W = blocks;
-    const int parts = std::min(p.W, (max_ch - 1) / (p.total / p.W) + 2);   // of a unit, at most
-    const auto merge = parts <= 4 * MERGE_GROUPS   ? merge_tc5_kernel<CG, 4>
-                       : parts <= 6 * MERGE_GROUPS ? merge_tc5_kernel<CG, 6>
-                       : parts <= 8 * MERGE_GROUPS ? merge_tc5_kernel<CG, 8>
-                                                   : merge_tc5_kernel<CG, 10>;
+    long long tiles = 0;   // of 128 rows: a block without rows leaves at once
+    for (int i = 0; i < p.qb.nQ; ++i) tiles += ((p.qb.cu[i + 1] - p.qb.cu[i]) * p.G + 127) / 128;
+    const int ahead = rekv_merge_ahead(plan.parts, tiles * p.nl * p.Hkv * 32, rekv_sm_count());
+    const auto merge = ahead == 4 ? merge_tc5_kernel<CG, 4> : ahead == 8 ? merge_tc5_kernel<CG, 8> : merge_tc5_kernel<CG, 10>;
     e = rekv_launch_pdl(merge, dim3((unsigned)units, CG, 32), dim3(128 * MERGE_GROUPS), 0, st, m);
     if (e != cudaSuccess) return e;
     c->launches += 1;

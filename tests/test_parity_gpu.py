@@ -395,6 +395,23 @@ def test_results_put_out_while_the_next_segment_goes_on(L, n_tokens, late):
 
 @pytest.mark.parametrize("Hkv,n_tokens", [(1, 20), (2, 37), (3, 20), (4, 20), (5, 9), (6, 40), (8, 20), (8, 5)])
 def test_one_layers_parts_joined_by_the_merge_launch(Hkv, n_tokens):
-    """Units of 51 chunks, few of them: from about fifty parts of a unit to about nine, every number in flight that the merge launch
-    is compiled for, on pairs and on single CTAs."""
+    """Units of 52 chunks, few of them, in 18 parts (two groups of ten in flight, one round, on pairs and on single CTAs), six or nine
+    (four in flight)."""
     _run_question_parity(H.Shape(L=1, Hq=7 * Hkv, Hkv=Hkv, Nf=196, T=36, W=2, k=31, seed=7), [n_tokens])
+
+
+# KV heads, question lengths, retrieved frames, and what the merge launch makes of them on 148 SMs (test_attend_plan.py holds the
+# rules to it): parts of a unit, parts in flight
+MERGED = [
+    (5, [20], 31, 13, 8),        # pairs, one round of eight in flight
+    (3, [9], 7, 8, 8),           # single CTAs, half a round
+    (8, [5, 5], 31, 9, 4),       # single CTAs, two rounds of four
+    (8, [20, 20], 31, 4, 4),     # pairs, half a round of four
+    (1, [20], 63, 26, 8),        # pairs, two rounds of eight
+    (1, [5], 63, 34, 8),         # single CTAs, three rounds
+]
+
+
+@pytest.mark.parametrize("Hkv,lengths,k,parts,ahead", MERGED)
+def test_merge_launch_by_parts_and_parts_in_flight(Hkv, lengths, k, parts, ahead):
+    _run_question_parity(H.Shape(L=1, Hq=7 * Hkv, Hkv=Hkv, Nf=196, T=k + 5, W=2, k=k, seed=7), lengths)
