@@ -23,8 +23,8 @@ import torch
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# The headline workload is BASELINE configs[1] (Qwen2-7B-like decoder, 1-hour stream at 0.5 fps, whole
-# cache in HBM).  The other full-size configurations can be timed with --workload; they are parity-test
+# The headline workload is a Qwen2-7B-like decoder over a 1-hour stream at 0.5 fps (1800 frames), the whole
+# cache in HBM.  The other full-size configurations can be timed with --workload; they are parity-test
 # cases, not the bench line.
 WORKLOADS = {
     "7b_hbm_1800f": dict(L=28, Hq=28, Hkv=4, D=128, Nf=196, T=1800, W=8, k=64, Nq=32, seed=2503, off_scale=0.5,
@@ -155,7 +155,7 @@ class ClockSampler:
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one attention launch from the committed ncu capture
 # (profiles/), scaled to the full workload by the layers processed; None where no capture exists.
-TRAFFIC_NCU = {"7b_hbm_1800f": 850.2e6, "7b_hbm_decode_1tok": 826.4e6}
+TRAFFIC_NCU = {"7b_hbm_1800f": 844.1e6, "7b_hbm_decode_1tok": 822.7e6}
 
 
 def algorithmic_bytes(w, sum_nq=None, nQ=1):

@@ -304,8 +304,9 @@ int rekv_check_status(rekv_ctx* ctx, void* stream);
  * and returns, and the context stays usable.  This call makes that path reachable without a fault:
  *   iterations       limit of every bounded wait of the kernels launched from now on (0 = the
  *                    built-in limit, about a third of a second)
- *   skip_copy_entry  >= 0: the copy producer of the attention kernel's first CTA leaves out the K/V tile copy
- *                    with this sequence number, so that the wait for it expires with nothing in flight; -1 = off
+ *   skip_copy_entry  >= 0: the copy producer of the attention kernel's first CTA leaves out the copy with this
+ *                    sequence number -- 2 c for the K tile of its chunk c and 2 c + 1 for the V tile, or, for
+ *                    decode-shaped questions, a step of one or several frames -- so that the wait for it expires; -1 = off
  * The affected launches produce no valid output; rekv_check_status then returns REKV_ERR_TIMEOUT once.
  * Host-side only; returns REKV_OK. */
 int rekv_test_set_wait_limit(rekv_ctx* ctx, unsigned iterations, int skip_copy_entry);

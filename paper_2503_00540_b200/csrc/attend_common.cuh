@@ -31,8 +31,8 @@ struct TcParams {
   int F;             // frames of a step
   int fsteps;        // steps of a unit: its context frames, F at a time ...
   int steps;         // ... then tiles of F * N_pad tokens of X
-  // test-only knobs (0 = off): iteration limit of the bounded waits, and the frame whose copy CTA 0 leaves out so that a
-  // wait runs out with nothing in flight
+  // test-only knobs (0 / -1 = off): iteration limit of the bounded waits, and the step (of one or several frames) whose copies CTA 0
+  // leaves out so that a wait runs out
   unsigned wait_limit;
   int skip_copy_entry;
   int part_slots;    // capacity of part_o / part_ml in 16-row parts

@@ -182,7 +182,7 @@ cudaError_t rekv_launch_attend_full_ctx(rekv_ctx* c, const QBatch& qb, int ncf, 
                                         int layer1) {
   const StoreView& s = c->sv;
   if (!rekv_rope_ctx(c) || ncf == 0 || rekv_decode_shaped(c, qb, ncf, layer1 - layer0)) return cudaSuccess;
-  // at least sixteen blocks for each SM, as far as a block has a row for every eight of its threads
+  // a page's rows over several blocks while that makes at most sixteen blocks for each SM, and 32 rows for a block
   const long long pages = (long long)ncf * qb.nQ * (layer1 - layer0);
   const int parts = (int)std::max(1ll, std::min<long long>(s.Nf / 32, 16ll * rekv_sm_count() / pages));
   cudaError_t e = rekv_launch_pdl(rope_stage_kernel, dim3(ncf * parts, qb.nQ, layer1 - layer0), dim3(256), 0, st, c->ctx_tbl, c->tbl_k,

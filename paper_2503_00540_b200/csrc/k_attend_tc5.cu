@@ -8,9 +8,9 @@
 // on one product (tcgen05 cta_group::2): each CTA owns one 128-row tile and brings half of every K and V tile, so tensor
 // memory holds O and THREE buffers of S (P over S) and the ring twice as many chunks.  S runs up to three chunks ahead,
 // two softmax warpgroups take the chunks alternately, and neither waits for a product of its own chunk.
-// 28 layers, 72 frames of 196 tokens, 32 query tokens: 218 -> 181 us at 1965 MHz (0.695 of the copy rate; a chunk takes 1536 cycles,
-// of which HBM alone needs 1476); in runs of seconds the card's 1000 W hold the whole question at 259 us, which is why fewer
-// instructions and bytes are what counts.
+// 28 layers, 72 frames of 196 tokens, 32 query tokens: 218 -> 179 to 194 us at 1965 MHz, by box (0.65 to 0.70 of the copy rate; a chunk
+// takes 1536 cycles, of which HBM alone needs 1476); in runs of seconds the card's 1000 W hold the whole question at 249 to 261 us,
+// which is why fewer instructions and bytes are what counts.
 //
 // Work split ("stream-K" in chunks).  A unit is (layer, kv head, question, 128 or 256 rows), a row being (question
 // token, query head of the KV group).  Eq. 3 without a positional term does not depend on the order or grouping of the
