@@ -415,9 +415,9 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
     }
     if (safe && !(redo_mask(false) & redo_bit(si, s, pos))) put = false;  // (the pair's other CTA asked for it)
     // O, 32 of the row's columns at a time.  The next segment's first P V waits until it has been read.  The range's last segment has
-    // none behind it and hands nothing back: nobody would wait for the other CTA's arrival before the issuing one's shared memory is
-    // given away.  (Waiting for it at the kernel's end: 28 layers, 64 tokens, 12 frames 107 -> 110 us, encoding step 239 -> 250.)
-    const bool last = !safe && pos + (s.I1 - s.I0) >= range1;
+    // none behind it, and a pair hands nothing back: nobody would wait for the other CTA's arrival before the issuing one's shared memory
+    // is given away.  (Waiting for it at the kernel's end: 28 layers, 64 tokens, 12 frames 107 -> 110 us, encoding step 239 -> 250.)
+    const bool last = CG == 2 && !safe && pos + (s.I1 - s.I0) >= range1;
     const uint32_t t_o = tmem + ((uint32_t)((warp & 3) << 5) << 16);
     const int col0 = part * WP::COLUMNS;
     auto load_o = [&](int c0, float (&o)[32]) {
@@ -1001,8 +1001,10 @@ __global__ void __launch_bounds__(Warps<OUT>::THREADS, 1) attend_tc5_kernel(cons
         else
           __syncthreads();
         if (redo_mask(true) == 0ull || *s_abort) break;
-        *s_again = 1;
-        if constexpr (ROLE == (OUT ? 2 : 1)) hand_back_o();   // the last segment's, after all
+        if constexpr (CG == 2) {
+          *s_again = 1;
+          if constexpr (ROLE == (OUT ? 2 : 1)) hand_back_o();   // the last segment's, after all
+        }
       }
     }
     if constexpr (ROLE == 0) {
